@@ -126,7 +126,7 @@ def measured_traffic(instances: int, dtype: str, schedule: dict):
         return None
     if instances != t["instances"] or tuple(N_RANGE) != t["n_range"] or dtype != t["dtype"]:
         return None
-    if (schedule["stage_path"], schedule["pipe_slots"], schedule["pipe_ctas_per_sm"]) != ("pipe", 2, 0):
+    if (schedule["stage_path"], schedule["pipe_slots"], schedule["pipe_ctas_per_sm"], schedule["resident"]) != ("pipe", 2, 0, 0):
         return None  # captured with the default schedule
     return t["bytes_per_launch"]
 
@@ -286,7 +286,7 @@ def e2e_leg(specs, opts, schedule: dict, steps: int, world: int, barrier):
     sts = [bq.State([bq.problem_from_spec(p) for p in part], opts) for part in parts]
     for st in sts:
         st.set_tune(stage_path=schedule["stage_path"], pipe_slots=schedule["pipe_slots"],
-                    pipe_ctas_per_sm=schedule["pipe_ctas_per_sm"])
+                    pipe_ctas_per_sm=schedule["pipe_ctas_per_sm"], resident=schedule["resident"])
     streams = [torch.cuda.Stream() for _ in parts]
     hosts = []
     for st in sts:
@@ -433,7 +433,7 @@ def batched_leg(world: int):
     t_step = timed(lambda: st2.step(DT, n_steps))
     out["streamed"] = {"seconds": t_step, "solves_per_s": 4096 / t_step,
                        "updates_per_s": 4 * pts * n_steps / t_step,
-                       "launches_per_step": 1 if st2.get_tune()["pipe_fused"] else 4}
+                       "launches_per_step": 1 / n_steps if st2.get_tune()["resident"] else 1 if st2.get_tune()["pipe_fused"] else 4}
     out["bq_solve_path"] = out["schedule"]["solve_kernel"]  # what bq_solve runs after bq_autotune
     # one instance per launch: 16 sampled instances, 2000 steps each, scaled
     sample = list(range(0, 4096, 256))
@@ -723,16 +723,19 @@ def secular_leg(B: int = 32768, steps: int = 20):
     torch.cuda.synchronize()
     s_step = e0.elapsed_time(e1) / 1e3 / steps
     pts = points_of(specs)
-    achieved = 16 * 8 * pts / 4 / (s_step / 4) / 1e9
     variant = st.stage_variant()
-    own = 18 if variant == "pipelined" else 19  # + the FP32 update's residual (and Kahan) transfers
+    resident = variant == "pipelined" and st.get_tune()["resident"] == 1
+    # resident: y and its residual in and out once per call; else the streamed 16 per step
+    bytes_per_point = 4 * 8 / steps if resident else 16 * 8
+    achieved = bytes_per_point * pts / s_step / 1e9
+    own = 4 / steps if resident else 18 if variant == "pipelined" else 19  # + the update's residual (and Kahan) transfers
     peak = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("hbm_gbs", 6800.0) \
         if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else 6800.0
     return {"workload": f"secular_batch x{B} (kerr_batch draws, secular dissipator, T_E = 0), complex FP32, "
-                        f"{steps} RK4 steps", "kernel": {"pipelined": "bq::k_stage_pipe", "single_mode": "bq::k_stage_m1",
-                                               "generic": "bq::k_stage"}[variant],
+                        f"{steps} RK4 steps", "kernel": "bq::k_resident" if resident else
+            {"pipelined": "bq::k_stage_pipe", "single_mode": "bq::k_stage_m1", "generic": "bq::k_stage"}[variant],
             "updates_per_s": 4 * pts / s_step, "ms_per_step": 1e3 * s_step,
-            "bytes_per_point_stage": 32, "kernel_transfers_per_step": own,
+            "bytes_per_point_stage": bytes_per_point / 4, "kernel_transfers_per_step": own,
             "achieved_gbs": achieved, "frac_of_measured_hbm": achieved / peak}
 
 
@@ -884,9 +887,14 @@ def main():
     # paths launch once per stage
     variant = state.stage_variant()
     fused = variant == "pipelined" and state.get_tune()["pipe_fused"] == 1
+    # the resident kernel keeps every system on chip for the whole step and moves 4 transfers (y
+    # and its rounding residual, in and out): its roofline counts those, not the streamed 16
+    resident = variant == "pipelined" and state.get_tune()["resident"] == 1
+    fused = fused or resident
     stages_per_launch = 4 if fused else 1
-    bytes_per_launch = stages_per_launch * 4 * csz * pts
-    kernel_bytes_per_launch = stages_per_launch * 18 * csz * pts / 4
+    bytes_per_launch = stages_per_launch * (1 if resident else 4) * csz * pts
+    transfers = 4 if resident else 18
+    kernel_bytes_per_launch = stages_per_launch * transfers * csz * pts / 4
     launch_s = stage_ms / 1e3 / (4 * args.steps / stages_per_launch)
     achieved = bytes_per_launch / launch_s / 1e9
     peaks = {}
@@ -897,11 +905,11 @@ def main():
     peak = peaks.get("hbm_gbs", 6800.0)
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": measured_traffic(args.instances, args.dtype, schedule) if fused else None,
-            "kernel": "bq::k_steps_pipe" if fused else {"pipelined": "bq::k_stage_pipe", "single_mode": "bq::k_stage_m1",
+            "kernel": "bq::k_resident" if resident else "bq::k_steps_pipe" if fused else {"pipelined": "bq::k_stage_pipe", "single_mode": "bq::k_stage_m1",
                                                           "generic": "bq::k_stage"}[variant],
             "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
-            "stages_per_launch": stages_per_launch, "bytes_per_launch": bytes_per_launch, "bytes_per_point_stage": 4 * csz,
-            "kernel_bytes_per_launch": kernel_bytes_per_launch, "kernel_transfers_per_step": 18,
+            "stages_per_launch": stages_per_launch, "bytes_per_launch": bytes_per_launch, "bytes_per_point_stage": (1 if resident else 4) * csz,
+            "kernel_bytes_per_launch": kernel_bytes_per_launch, "kernel_transfers_per_step": transfers,
             "avg_launch_us": launch_s * 1e6}
 
     # ---- end to end through the C ABI: state from pinned host memory, observables back ---
@@ -951,7 +959,7 @@ def main():
                                        "Tr(rho0 A) per instance per step",
                            "instances_per_gpu": args.instances, "n_range": list(N_RANGE), "grid_points_per_gpu": pts,
                            "schedule": {k: schedule[k] for k in ("stage_path", "pipe_slots", "pipe_ctas_per_sm",
-                                                                 "n_candidates", "step_us")},
+                                                                 "resident", "n_candidates", "step_us")},
                            "state_bytes_per_array": nbytes, "l2": "inputs larger than L2 (5 arrays x "
                            f"{nbytes / 1e6:.0f} MB vs 129 MB)", "parallelism": f"replicas x{world}"},
                 "roofline": roof, "e2e": e2e, "alu_peaks": peaks_alu, "fp64": fp64, "batched": batched, "grads": grads, "methods": methods, "secular": secular, "fig2": fig2, "cpu_baseline": cpu, "clocks": clocks, "gpu_launches": launches}

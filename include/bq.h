@@ -176,16 +176,18 @@ int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* opts, void*
 /* ---- stepping (Eqs. 9a-c / 303a-c, classical RK4) ----------------------------------- */
 
 /* Advances every system of the state by n_steps RK4 steps of size dt (the mapped value
- * of dt must not exceed the bound checked at bq_map).  Fused stage kernels: on the
- * pipelined single-mode path the four stages of a step run in one launch (bq_tune
- * pipe_fused), otherwise one launch per stage; replayed from a CUDA graph; asynchronous on
- * stream. */
+ * of dt must not exceed the bound checked at bq_map).  Single-mode states of the resident form
+ * (bq_tune resident): all n_steps in one launch, every system on chip.  Else fused stage
+ * kernels: on the pipelined single-mode path the four stages of a step run in one launch
+ * (bq_tune pipe_fused), otherwise one launch per stage; replayed from a CUDA graph.
+ * Asynchronous on stream. */
 int bq_step(bq_state* s, double dt, int64_t n_steps, void* stream);
 
 /* Batched persistent solve (one launch for all steps of all systems of the batch; the
  * paper's independent initial conditions, main text after Eq. 13, processed as a work
- * queue): every CTA takes systems from an atomic queue, largest first, and keeps the
- * system on chip for all n_steps steps (the RK4 stage buffers, stage sums and compensation
+ * queue).  Single-mode states of the resident form run bq_step's resident kernel (bq_tune
+ * resident); in the others every CTA takes systems from an atomic queue, largest first, and
+ * keeps the system on chip for all n_steps steps (the RK4 stage buffers, stage sums and compensation
  * in shared memory, the state in registers).  The same arithmetic as bq_step (classical
  * RK4, compensated state update) up to rounding order.  Where bq_autotune measured stepping
  * faster (bq_tune solve_kernel = BQ_SOLVE_STEP), bq_solve runs bq_step instead.  Applies to single-mode
@@ -240,7 +242,10 @@ typedef struct bq_tune {
   int pipe_fused;        /* BQ_PATH_PIPE: 1 = the four stages of a step in one launch (every CTA
                           * runs its own systems' stages in order; no CTA waits for another),
                           * 0 = one launch per RK4 stage.  The arithmetic is the same. */
-  int pad;
+  int resident;          /* BQ_PATH_PIPE, and BQ_SOLVE_MERGED with solve_ctas_per_sm = 0: 1 = the
+                          * resident kernel where the state has the form it takes (the default
+                          * there): all steps of a call in one launch, every system on chip, whatever
+                          * the other pipe_* fields say; 0 = the kernels those fields describe */
 } bq_tune;
 
 /* Current schedules of the state (step_us / solve_us: last bq_autotune result, else 0). */

@@ -18,7 +18,7 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libbq.so")
 BUILD_DIR = os.path.join(HERE, "_build")
-SOURCES = ["bq_host.cu", "bq_kernels.cu", "bq_peaks.cu"]
+SOURCES = ["bq_host.cu", "bq_kernels.cu", "bq_resident_f32.cu", "bq_resident_f64.cu", "bq_peaks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -45,7 +45,7 @@ def _compile(src: str, verbose_ptxas: bool) -> str:
 
 def build(force: bool = False, verbose_ptxas: bool = False) -> str:
     srcs = [os.path.join(CSRC, s) for s in SOURCES]
-    hdrs = [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith(".h")]
+    hdrs = [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith((".h", ".cuh"))]
     hdrs.append(os.path.join(ROOT, "include", "bq.h"))
     if not force and os.path.exists(LIB):
         t = os.path.getmtime(LIB)

@@ -18,6 +18,7 @@
 #include "../../include/bq.h"
 #include "bq_internal.h"
 #include "bq_launch.h"
+#include "bq_resident.h"
 
 using cplx = std::complex<double>;
 using bq::ChanDesc;
@@ -742,8 +743,16 @@ static int compile_problem(const bq_problem* p, const bq_map_opts& o, Compiled& 
 // State.
 // ---------------------------------------------------------------------------------------
 struct Layout {
-  size_t off_sys, off_terms, off_chans, off_chpar, off_work, off_m1, off_order, off_dc, off_pparams, off_precs, off_obs, off_groups, off_entries, off_out, off_wtab, off_diag,
+  size_t off_sys, off_terms, off_chans, off_chpar, off_work, off_m1, off_order, off_dc, off_pparams, off_precs, off_obs, off_rparams, off_rgroups, off_rbins, off_rflags, off_groups, off_entries, off_out, off_wtab, off_diag,
       off_ctrl, off_init, off_y, off_comp, off_ua, off_ub, off_acc, total;
+};
+
+// A launch of the resident kernel: groups [g0, g0 + n_groups) in bins [b0, b0 + n_bins).
+//   list 0: systems Hermitian by structure and initial state, Hermitian layout;
+//   list 1: all others, general layout;
+//   list 2: the systems of list 0 in the general layout (for states loaded from outside).
+struct ResList {
+  int b0 = 0, n_bins = 0, g0 = 0, n_groups = 0, smem = 0;
 };
 
 struct bq_state {
@@ -760,6 +769,16 @@ struct bq_state {
   // streaming kernels skip reading it at their next stage 1; every other consumer clears it
   // first, see ensure_comp)
   int comp_zero = 0;
+  // resident kernel: available, its schedule switch, launch variants and lists; res_known: the
+  // systems of list 0 are known to hold Hermitian states (false once a state was loaded or
+  // another kernel stepped it: then res_dirty asks for a check of the data before the next
+  // launch, and the systems that fail it take list 2)
+  int res_ok = 0, res_on = 0, res_mode = 1, res_ns = 1, res_obs = 0, res_known = 1, res_dirty = 0;
+  ResList rlist[3];
+  // steps of equal length taken by the resident kernel since tau was run_tau0: their times are
+  // run_tau0 + i run_dt however the calls split them (run_tau: tau after the last of them)
+  double run_tau0 = 0.0, run_dt = 0.0, run_tau = 0.0;
+  int64_t run_steps = 0;
   // 1 while the per-system Tr(rho0 A) contributions the pipelined kernel's last stage 4 left
   // in the pool describe the current state (bq_evaluate then only reads them back)
   int obs_valid = 0;
@@ -802,6 +821,7 @@ struct bq_state {
 
 static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
+
 struct Plan {
   std::vector<Compiled> comp;
   std::vector<SysDesc> sys;
@@ -835,6 +855,13 @@ struct Plan {
   int grad_size = 0;
   int64_t total_elems = 0;
   double rho = 0.0, dt_max = 0.0;
+  // resident kernel (k_resident): parameter blocks per problem, groups (the Hermitian layout's,
+  // then the general layout's) and the CTAs' bins
+  int res_ok = 0, res_mode = 1, res_ns = 1, res_obs = 1;
+  std::vector<unsigned char> rparams;
+  std::vector<bq::ResGroup> rgroups;
+  std::vector<bq::ResBin> rbins;
+  ResList rlist[3];
   Layout L{};
 };
 
@@ -917,6 +944,270 @@ static void build_work(const std::vector<SysDesc>& sys, size_t cs, int tile, int
       work.push_back(w);
     }
   }
+}
+
+// ---------------------------------------------------------------------------------------
+// Plan of the resident kernel (bq_resident.cuh).  Available when every problem of a single-mode
+// batch has the separable form the kernel evaluates:
+//   * a full R of 4 <= M <= 42;
+//   * static shift-0 terms (they join the diagonal tables), and off-diagonal terms, if any, one
+//     per side and direction with coefficients a, -conj(a) (left, sources k - 1 and k + 1) and
+//     conj(a), -a (right, sources l - 1 and l + 1), as the linear drive of a Hermitian H gives;
+//   * sandwich terms with a static real coefficient and shift (-1, -1) or (+1, +1), at most one
+//     each, all of them or none restricted to k = l.
+// Anything else keeps the streaming and per-term kernels.
+// ---------------------------------------------------------------------------------------
+
+// Rows per strip and warps of a system: the fewest issue slots, counting a
+// row as 1 and a strip's fixed part (edges, stage set-up) as 1.4 rows.  0 if it does not fit.
+static int res_shape(int M, int cs, bool herm, int& rb, int& nb) {
+  const int cols = herm ? M | 1 : M, nd = herm ? cols / 2 + 1 : M;
+  const int cap = BQ_RES_WARPS(cs, herm);
+  int best = 0;
+  double cost = 1e300;
+  for (int r : {2, 4, 7}) {
+    if (r > nd || (cs == 16 && r > 4)) continue;
+    const int n = (nd + r - 1) / r, w = (cols * n + 31) / 32;
+    if (w + 1 > cap) continue;
+    if (w * (r + 1.4) < cost) {
+      cost = w * (r + 1.4);
+      rb = r;
+      nb = n;
+      best = w + 1;
+    }
+  }
+  return best;
+}
+
+static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, const EvalGroup& eg, int term_off,
+                        int wbase, size_t cs, std::vector<unsigned char>& blk, int& mode, int& ns, bool& herm) {
+  const int M = C.M[0];
+  if (M < 4 || M > 42 || !C.has_r || C.r_diag || eg.n_e > 32) return false;
+  std::vector<cplx> d(C.diag.begin(), C.diag.begin() + 2 * M);
+  std::vector<double> w[8];  // xm xp ym yp smx smy spx spy
+  for (auto& v : w) v.assign(M, 0.0);
+  const TermDesc* off[4] = {nullptr, nullptr, nullptr, nullptr};  // xm xp ym yp
+  int sdiag = -1;
+  bool splus = false;
+  for (size_t t = 0; t < C.terms.size(); ++t) {
+    const TermDesc& td = P.terms[term_off + t];
+    const cplx c(td.c_re, td.c_im);
+    auto table = [&](int dim) -> const double* {  // weights along R's dimension dim, or null (all ones)
+      for (int a = 0; a < td.n_act; ++a)
+        if (td.dim[a] == dim) return C.wtab.data() + td.wtab[a] - wbase;
+      return nullptr;
+    };
+    if (td.side == bq::SIDE_S) {
+      const int s = td.deltaGx, dg = td.diagp1 ? 1 : 0;
+      if (td.ch >= 0 || c.imag() != 0.0 || s != td.deltaGy || (s != -1 && s != 1) || (sdiag >= 0 && sdiag != dg)) return false;
+      sdiag = dg;
+      std::vector<double>&wx = w[s < 0 ? 4 : 6], &wy = w[s < 0 ? 5 : 7];
+      for (double v : wy)
+        if (v != 0.0) return false;  // a second term of this direction
+      const double *tx = table(0), *ty = table(1);
+      for (int k = 0; k < M; ++k) {
+        wx[k] = c.real() * (tx ? tx[k] : 1.0);
+        wy[k] = ty ? ty[k] : 1.0;
+      }
+      splus = splus || s > 0;
+      continue;
+    }
+    const int y = td.side == bq::SIDE_Y, s = y ? td.deltaGy : td.deltaGx;
+    const double* tw = table(y);
+    if (s == 0) {
+      if (td.ch >= 0) return false;
+      for (int k = 0; k < M; ++k) d[y * M + k] += c * (tw ? tw[k] : 1.0);
+    } else if (s == 1 || s == -1) {
+      const int q = 2 * y + (s > 0);
+      if (off[q]) return false;
+      off[q] = &td;
+      for (int k = 0; k < M; ++k) w[q][k] = tw ? tw[k] : 1.0;
+    } else {
+      return false;
+    }
+  }
+  // zero weights where the source leaves the grid (the tables hold zeros there; a term without
+  // a table would not)
+  w[0][0] = w[2][0] = w[4][0] = w[5][0] = 0.0;
+  w[1][M - 1] = w[3][M - 1] = w[6][M - 1] = w[7][M - 1] = 0.0;
+  bq::ResHdr h;
+  std::memset(&h, 0, sizeof(h));
+  h.M = M;
+  h.has_sep = C.has_sep;
+  h.sdiag = sdiag > 0;
+  int n_off = 0;
+  for (auto* o : off) n_off += o != nullptr;
+  bool imag = true;
+  if (n_off) {
+    if (n_off != 4) return false;
+    const cplx a(off[0]->c_re, off[0]->c_im);
+    const cplx want[4] = {a, -std::conj(a), std::conj(a), -a};
+    const int flip[4] = {0, 1, 1, 0};  // conjugated coefficients read the conjugate envelope
+    for (int q = 0; q < 4; ++q) {
+      if (cplx(off[q]->c_re, off[q]->c_im) != want[q] || off[q]->ch != off[0]->ch) return false;
+      if (off[0]->ch >= 0 && off[q]->conj != (off[0]->conj ^ flip[q])) return false;
+    }
+    h.a_re = a.real();
+    h.a_im = a.imag();
+    imag = a.real() == 0.0;
+    if (off[0]->ch >= 0) {
+      const ChanDesc& cd = P.chans[off[0]->ch];
+      const double* cp = P.chpar.data() + cd.par_off;
+      h.ch = 1;
+      h.conj = off[0]->conj;
+      for (int i = 0; i < 4 && i < cd.n_par; ++i) h.chan.p[i] = cp[i];
+      h.chan.kind = cd.kind;
+      h.chan.par_off = cd.par_off;
+      h.chan.n_par = cd.n_par;
+      h.chan.f[0] = (float)cp[0];
+      h.chan.f[1] = (float)cp[1];
+      switch (cd.kind) {
+        case BQ_CH_GAUSS:
+          h.chan.f[2] = (float)(1.0 / (2.0 * cp[3] * cp[3]));
+          h.chan.f[3] = (float)cp[2];
+          h.chan.c_lo = (float)(cp[2] - (double)h.chan.f[3]);
+          imag = imag && cp[1] == 0.0;
+          break;
+        case BQ_CH_CONST: imag = imag && cp[1] == 0.0; break;
+        case BQ_CH_PWC:
+          for (int i = 3; i < cd.n_par; i += 2) imag = imag && cp[i] == 0.0;
+          break;
+        default: imag = false;
+      }
+    }
+  }
+  if (!imag) mode = 2;
+  if (splus) ns = 2;
+  herm = w[0] == w[2] && w[1] == w[3];
+  for (int k = 0; k < M && herm; ++k) {
+    herm = d[M + k] == std::conj(d[k]);
+    // row and column tables of a sandwich term differ by a factor only (its rate, to rounding)
+    for (int q = 4; q < 8 && herm; q += 2)
+      for (int j = 0; j < k && herm; ++j) {
+        const double u = w[q][k] * w[q + 1][j], v = w[q][j] * w[q + 1][k];
+        herm = std::abs(u - v) <= 1e-14 * std::abs(u);
+      }
+  }
+  blk.resize(sizeof(h));
+  auto put = [&](double v) {
+    if (cs == 16) blk.insert(blk.end(), (unsigned char*)&v, (unsigned char*)&v + 8);
+    else { float f = (float)v; blk.insert(blk.end(), (unsigned char*)&f, (unsigned char*)&f + 4); }
+  };
+  for (const cplx& v : d) { put(v.real()); put(v.imag()); }
+  for (auto& v : w)
+    for (double x : v) put(x);
+  while (blk.size() % 16) blk.push_back(0);
+  h.obs_off = (int)blk.size();
+  h.n_obs = eg.n_e;
+  for (int e = 0; e < eg.n_e; ++e) {
+    const EvalEntry& en = P.entries[eg.e_off + e];
+    bq::PipeObs<double2> o;
+    std::memset(&o, 0, sizeof(o));
+    o.kx = en.kx; o.ly = en.ly; o.f = make_double2(en.f_re, en.f_im);
+    blk.insert(blk.end(), (const unsigned char*)&o, (const unsigned char*)&o + sizeof(o));
+  }
+  std::memcpy(blk.data(), &h, sizeof(h));
+  return true;
+}
+
+// Groups of the systems `which` in the given layout, packed into CTAs: within runs of 4096
+// systems (so that the systems in flight stay in one region of the state arrays) the widest
+// group first, filled up with the widest that still fits.  Every group of a launch takes about
+// the same time (strips of equal length), so a CTA's groups end together.
+static bool res_pack(Plan& P, const std::vector<int>& which, const std::vector<int>& poff, size_t cs, bool herm, ResList& L) {
+  L.b0 = (int)P.rbins.size();
+  L.g0 = (int)P.rgroups.size();
+  const int cap = BQ_RES_WARPS((int)cs, herm);
+  for (size_t r0 = 0; r0 < which.size(); r0 += 4096) {
+    std::vector<std::vector<int>> by(cap + 1);  // groups of this run by width
+    for (size_t i = r0; i < std::min(which.size(), r0 + 4096); ++i) {
+      const SysDesc& sd = P.sys[which[i]];
+      const int M = sd.M[0];
+      bq::ResGroup g;
+      std::memset(&g, 0, sizeof(g));
+      const int cols = herm ? M | 1 : M, nd = herm ? cols / 2 + 1 : M;
+      const int w = res_shape(M, (int)cs, herm, g.rb, g.nb);
+      if (!w) return false;
+      g.sys = which[i];
+      g.M = M;
+      g.blk_off = (int)(sd.has_sep ? sd.off_gx : sd.off_r);
+      g.gy_off = sd.has_sep ? (int)(sd.off_gy - sd.off_gx) : -1;
+      g.r_off = (int)(sd.off_r - g.blk_off);
+      g.blk_elems = g.r_off + ((sd.n_r + 3) & ~3);
+      g.param_off = poff[sd.prob];
+      g.nwarps = w;
+      const int buf = nd * cols;
+      g.stage_elems = std::max(g.blk_elems, 2 * buf + (BQ_RES_COMP_SMEM(cs, herm) ? g.rb * g.nb * cols : 0));
+      g.c_re = sd.c_re; g.c_im = sd.c_im; g.w_re = sd.w_re; g.w_im = sd.w_im;
+      by[w].push_back((int)P.rgroups.size());
+      P.rgroups.push_back(g);
+    }
+    std::vector<size_t> at(cap + 1, 0);
+    for (;;) {
+      bq::ResBin bin;
+      for (int& x : bin.g) x = -1;
+      int used = 0;
+      size_t smem = 0;
+      for (int w = cap; w >= 2;) {
+        if (w > cap - used || at[w] == by[w].size()) { --w; continue; }
+        const int gi = by[w][at[w]];
+        bq::ResGroup& g = P.rgroups[gi];
+        const size_t need = bq::res_group_smem(g.stage_elems, g.M, cs);
+        if (smem + need > BQ_RES_SMEM_MAX) {
+          if (!used) return false;
+          --w;
+          continue;
+        }
+        ++at[w];
+        g.warp0 = used;
+        g.smem_off = (int)smem;
+        for (int q = 0; q < w; ++q) bin.g[used + q] = gi;
+        used += w;
+        smem += need;
+      }
+      if (!used) break;
+      L.smem = std::max(L.smem, (int)smem);
+      P.rbins.push_back(bin);
+    }
+  }
+  L.n_bins = (int)P.rbins.size() - L.b0;
+  L.n_groups = (int)P.rgroups.size() - L.g0;
+  return true;
+}
+
+// progs: the term program of every problem (single-mode states).
+static void make_res_plan(Plan& P, const bq_problem* const* probs, const std::vector<bq::M1Sys>& progs, size_t cs) {
+  if (P.total_elems >= ((int64_t)1 << 31)) return;
+  const int B = (int)P.comp.size();
+  std::vector<int> term_off(B, 0), poff(B, 0);
+  for (const SysDesc& sd : P.sys) term_off[sd.prob] = sd.term_off;
+  std::vector<char> herm(B, 0);
+  std::vector<unsigned char> blk;
+  for (int b = 0; b < B; ++b) {
+    bool hm = false;
+    blk.clear();
+    if (!res_problem(P, P.comp[b], progs[b], P.groups[b], term_off[b], P.wbase[b], cs, blk, P.res_mode, P.res_ns, hm)) return;
+    if (P.comp[b].method == BQ_METHOD_DIRECT) {  // A(0) itself
+      for (auto& [kl, v] : probs[b]->measured) {
+        auto it = probs[b]->measured.find({kl.second, kl.first});
+        if (v != cplx(0, 0) && (it == probs[b]->measured.end() || it->second != std::conj(v))) hm = false;
+      }
+    }
+    herm[b] = hm;
+    poff[b] = (int)P.rparams.size();
+    P.rparams.insert(P.rparams.end(), blk.begin(), blk.end());
+  }
+  std::vector<int> hs, gs;
+  for (int i = 0; i < (int)P.sys.size(); ++i) {
+    const SysDesc& sd = P.sys[i];
+    // mapped systems start Hermitian as x^p y^p with an imaginary separation constant
+    const bool h = herm[sd.prob] && (!sd.has_sep || (sd.p_flat >= 0 && sd.p_flat == sd.q_flat && sd.c_re == 0.0));
+    (h ? hs : gs).push_back(i);
+  }
+  if (!res_pack(P, hs, poff, cs, true, P.rlist[0]) || !res_pack(P, gs, poff, cs, false, P.rlist[1]) ||
+      !res_pack(P, hs, poff, cs, false, P.rlist[2]))
+    return;
+  P.res_ok = 1;
 }
 
 static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o, Plan& P) {
@@ -1297,6 +1588,12 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
         P.use_pipe = pipe_ok && 2 * (size_t)P.pipe_slot <= 200 * 1024 ? 1 : 0;
 
       }
+      if (P.use_pipe) make_res_plan(P, probs, progs, cs);
+      if (!P.res_ok) {
+        P.rparams.clear();
+        P.rgroups.clear();
+        P.rbins.clear();
+      }
       if (solve_ok && solve_max <= 160 * 1024) {
         std::stable_sort(sz.begin(), sz.end());
         for (auto& e : sz) P.order.push_back(e.second);
@@ -1372,7 +1669,11 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
   L.off_order = seg(P.order.size() * sizeof(int));
   L.off_pparams = seg(P.pparams.size());
   L.off_precs = seg(P.precs.size() * sizeof(bq::PipeRec));
-  L.off_obs = seg(P.use_pipe ? P.sys.size() * sizeof(double2) : 0);
+  L.off_obs = seg(P.use_pipe || P.res_ok ? P.sys.size() * sizeof(double2) : 0);
+  L.off_rparams = seg(P.rparams.size());
+  L.off_rgroups = seg(P.rgroups.size() * sizeof(bq::ResGroup));
+  L.off_rbins = seg(P.rbins.size() * sizeof(bq::ResBin));
+  L.off_rflags = seg(P.res_ok ? P.sys.size() : 0);
   L.off_dc = seg(P.dc.size() * sizeof(double2));
   L.off_groups = seg(P.groups.size() * sizeof(EvalGroup));
   L.off_entries = seg(P.entries.size() * sizeof(EvalEntry));
@@ -1475,6 +1776,9 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
   CUDA_TRY(up(L.off_order, P.order.data(), P.order.size() * sizeof(int)));
   CUDA_TRY(up(L.off_pparams, P.pparams.data(), P.pparams.size()));
   CUDA_TRY(up(L.off_precs, P.precs.data(), P.precs.size() * sizeof(bq::PipeRec)));
+  CUDA_TRY(up(L.off_rparams, P.rparams.data(), P.rparams.size()));
+  CUDA_TRY(up(L.off_rgroups, P.rgroups.data(), P.rgroups.size() * sizeof(bq::ResGroup)));
+  CUDA_TRY(up(L.off_rbins, P.rbins.data(), P.rbins.size() * sizeof(bq::ResBin)));
   {
     std::vector<double2> dcv(P.dc.size());
     for (size_t i = 0; i < dcv.size(); ++i) dcv[i] = make_double2(P.dc[i].real(), P.dc[i].imag());
@@ -1543,6 +1847,11 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
     st->use_pipe = rc == BQ_OK ? 1 : 0;
   }
   st->pipe_ok = st->use_pipe;
+  st->res_ok = st->res_on = P.res_ok && st->pipe_ok;
+  st->res_mode = P.res_mode;
+  st->res_ns = P.res_ns;
+  st->res_obs = P.res_obs;
+  for (int q = 0; q < 3; ++q) st->rlist[q] = P.rlist[q];
 
   st->grad_size = P.grad_size;
   st->adj_smem = P.adj_smem;
@@ -1662,18 +1971,88 @@ static cudaError_t launch_any_stage(bq_state* s, const bq::StageArgs& a, cudaStr
     const bq::PipeArgs pa = pipe_args(s, a);
     const int q = a.stage - 1;
     s->obs_valid = a.stage == 4 && s->pipe_obs;
+    s->res_known = 0;
+    s->res_dirty = 1;
     if (a.stage == 1) s->comp_zero = 0;  // stage 4 of this step writes comp everywhere
     return bq::launch_stage_pipe(pa, s->m1_variant, s->dtype, a.stage, s->pipe_grid[q],
                                  pa.n_slots * pa.slot_bytes + s->pipe_mv_bytes, st);
   }
   s->obs_valid = 0;
+  s->res_known = 0;
+  s->res_dirty = 1;
   if (s->use_m1)
     return bq::launch_stage_m1(a, (const bq::M1Sys*)(s->pool + s->L.off_m1), s->m1_variant, s->dtype, s->n_work,
                                s->smem_bytes, st);
   return bq::launch_stage(a, s->dtype, s->nm, s->n_work, s->smem_bytes, st);
 }
 
+// The resident kernel serves bq_step on the pipelined path and bq_solve's merged kernel.
+static bool res_on(const bq_state* s) { return s->res_ok && s->res_on && s->use_pipe; }
+
+// n steps from s->tau with the resident kernel, one launch per non-empty list; advances s->tau.
+static cudaError_t enqueue_resident(bq_state* s, double dt, int64_t n, cudaStream_t st, int* launches) {
+  char* b = s->pool;
+  const Layout& L = s->L;
+  unsigned char* flags = (unsigned char*)(b + L.off_rflags);
+  const bq::ResGroup* groups = (const bq::ResGroup*)(b + L.off_rgroups);
+  *launches = 0;
+  if (s->res_dirty) {
+    const cudaError_t e = bq::launch_res_check(groups + s->rlist[0].g0, s->rlist[0].n_groups, b + L.off_y, b + L.off_comp,
+                                               s->comp_zero, s->dtype, flags, st);
+    if (e != cudaSuccess) return e;
+    if (s->rlist[0].n_groups) ++*launches;
+    s->res_dirty = 0;
+  }
+  bq::ResArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.groups = groups;
+  a.params = (const unsigned char*)(b + L.off_rparams);
+  a.chpar = (const double*)(b + L.off_chpar);
+  a.y = b + L.off_y;
+  a.comp = b + L.off_comp;
+  a.obs = s->res_obs ? (double2*)(b + L.off_obs) : nullptr;
+  a.reverse = s->reverse;
+  a.dt = dt;
+  a.horizon = s->horizon;
+  if (s->tau != s->run_tau || dt != s->run_dt || s->run_steps == 0) {
+    s->run_tau0 = s->tau;
+    s->run_dt = dt;
+    s->run_steps = 0;
+  }
+  const int64_t most = 1 << 30;  // steps per launch (32-bit counter)
+  for (int64_t done = 0; done < n;) {
+    const int64_t m = std::min(most, n - done);
+    a.n_steps = (int)m;
+    a.tau0 = s->run_tau0;
+    a.step0 = s->run_steps + done;
+    a.comp_zero = s->comp_zero;
+    for (int q = 0; q < (s->res_known ? 2 : 3); ++q) {
+      const ResList& l = s->rlist[q];
+      if (!l.n_bins) continue;
+      a.bins = (const bq::ResBin*)(b + L.off_rbins) + l.b0;
+      a.flags = q == 1 || s->res_known ? nullptr : flags;
+      a.want = q == 0;
+      const auto launch = s->dtype == BQ_F64 ? bq::launch_resident_f64 : bq::launch_resident_f32;
+      const cudaError_t e = launch(a, s->res_mode, s->res_ns, q == 0, l.n_bins, l.smem, st);
+      if (e != cudaSuccess) return e;
+      ++*launches;
+    }
+    s->comp_zero = 0;  // every system's comp is written
+    done += m;
+  }
+  s->run_steps += n;
+  s->tau = s->run_tau = s->run_tau0 + (double)s->run_steps * dt;
+  s->obs_valid = s->res_obs;
+  return cudaSuccess;
+}
+
 static cudaError_t enqueue_steps(bq_state* s, double dt, int64_t n, cudaStream_t st) {
+  if (res_on(s)) {
+    int k = 0;
+    return enqueue_resident(s, dt, n, st, &k);
+  }
+  s->res_known = 0;  // (these kernels may leave a Hermitian system Hermitian to rounding only)
+  s->res_dirty = 1;
   if (pipe_fused_on(s)) {
     // The four stages of a step in one launch of the multi-step kernel, one launch per step.
     // (Several steps per launch were slower, 146 against 110 us per step on a 4096-system
@@ -1710,6 +2089,12 @@ extern "C" int bq_step(bq_state* s, double dt, int64_t n_steps, void* stream) {
   if (n_steps == 0) return BQ_OK;
   cudaStream_t st = (cudaStream_t)stream;
   char* b = s->pool;
+  if (res_on(s)) {
+    int k = 0;
+    CUDA_TRY(enqueue_resident(s, dt, n_steps, st, &k));
+    g_launches += k;
+    return BQ_OK;
+  }
   if (!s->use_pipe) CUDA_TRY(ensure_comp(s, st));
   // tau at the start of this call; the stage kernels add counter * dt
   s->tau_base_host = s->tau;
@@ -1794,6 +2179,8 @@ extern "C" int bq_step_fixed_scratch(bq_state* s, double dt, int64_t n_steps, vo
 }
 
 static cudaError_t enqueue_solve(bq_state* s, double dt, int64_t n_steps, cudaStream_t st);
+// BQ_SOLVE_MERGED runs the resident kernel where it is available and at the occupancy limit
+static bool solve_resident(const bq_state* s) { return s->res_ok && s->res_on && s->solve_mg && s->solve_cap == 0; }
 
 extern "C" int bq_solve(bq_state* s, double dt, int64_t n_steps, void* stream) {
   if (!s) return fail(BQ_EINVAL, "state is NULL");
@@ -1803,10 +2190,15 @@ extern "C" int bq_solve(bq_state* s, double dt, int64_t n_steps, void* stream) {
   if (dt > s->dt_max * (1.0 + 1e-12))
     return fail(BQ_EUNSTABLE_DT, "dt=%g above the RK4 stability bound %g", dt, s->dt_max);
   if (n_steps == 0) return BQ_OK;
-  CUDA_TRY(ensure_comp(s, (cudaStream_t)stream));
-  CUDA_TRY(enqueue_solve(s, dt, n_steps, (cudaStream_t)stream));
-  g_launches++;
-  s->tau += (double)n_steps * dt;
+  int launches = 1;
+  if (solve_resident(s)) {
+    CUDA_TRY(enqueue_resident(s, dt, n_steps, (cudaStream_t)stream, &launches));
+  } else {
+    CUDA_TRY(ensure_comp(s, (cudaStream_t)stream));
+    CUDA_TRY(enqueue_solve(s, dt, n_steps, (cudaStream_t)stream));
+    s->tau += (double)n_steps * dt;
+  }
+  g_launches += launches;
   return BQ_OK;
 }
 
@@ -1815,6 +2207,8 @@ static cudaError_t enqueue_solve(bq_state* s, double dt, int64_t n_steps, cudaSt
   char* b = s->pool;
   const Layout& L = s->L;
   s->obs_valid = 0;
+  s->res_known = 0;
+  s->res_dirty = 1;
   cudaError_t e = cudaMemsetAsync(b + L.off_ctrl + 24, 0, 8, st);
   if (e != cudaSuccess) return e;
   bq::SolveArgs a;
@@ -1901,6 +2295,7 @@ extern "C" int bq_get_tune(const bq_state* s, bq_tune* out) {
   out->grad_coop = s->grad_coop;
   out->grad_us = s->tune_grad_us;
   out->pipe_fused = s->pipe_fused;
+  out->resident = s->res_on;
   return BQ_OK;
 }
 
@@ -1950,6 +2345,7 @@ extern "C" int bq_set_tune(bq_state* s, const bq_tune* t) {
   s->lanes = t->lanes == 0 ? default_lanes(s->sys) : t->lanes;
   s->grad_coop = t->grad_coop != 0;
   s->pipe_fused = t->pipe_fused != 0;
+  s->res_on = s->res_ok && t->resident != 0;
   drop_graph(s);
   return BQ_OK;
 }
@@ -2002,6 +2398,7 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
   char* b = s->pool;
   char* sc = (char*)scratch;
   const double tau0 = s->tau;
+  const int res_known0 = s->res_known, res_dirty0 = s->res_dirty;
   CUDA_TRY(ensure_comp(s, st));  // the saved copy is valid for every schedule
   CUDA_TRY(cudaMemcpyAsync(sc, b + s->L.off_y, n, cudaMemcpyDeviceToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(sc + n, b + s->L.off_comp, n, cudaMemcpyDeviceToDevice, st));
@@ -2010,6 +2407,7 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
     if (e == cudaSuccess) e = cudaMemcpyAsync(b + s->L.off_comp, sc + n, n, cudaMemcpyDeviceToDevice, st);
     s->obs_valid = 0;
     s->tau = tau0;
+    s->run_steps = 0;
     s->tau_base_host = tau0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(b + s->L.off_ctrl, &s->tau_base_host, sizeof(double), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(b + s->L.off_ctrl + 8, 0, 16, st);
@@ -2025,8 +2423,12 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
       CUDA_TRY(restore());
       if (rep == 1) CUDA_TRY(cudaEventRecord(e0, st));
       const int64_t ns = rep == 0 ? 1 : trial_steps;
-      CUDA_TRY(solve ? enqueue_solve(s, dt, ns, st) : enqueue_steps(s, dt, ns, st));
-      g_launches += solve ? 1 : ns * kernels_per_step(s);
+      int launches = solve ? 1 : (int)(ns * kernels_per_step(s));
+      if (solve ? solve_resident(s) : res_on(s))
+        CUDA_TRY(enqueue_resident(s, dt, ns, st, &launches));
+      else
+        CUDA_TRY(solve ? enqueue_solve(s, dt, ns, st) : enqueue_steps(s, dt, ns, st));
+      g_launches += launches;
       if (rep == 1) CUDA_TRY(cudaEventRecord(e1, st));
     }
     CUDA_TRY(cudaEventSynchronize(e1));
@@ -2045,8 +2447,9 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
   bq_get_tune(s, &best);
   double best_step = 1e300;
   {
-    struct Cand { int path, slots, cap, lanes, gread; };
+    struct Cand { int path, slots, cap, lanes, gread, resident = 0; };
     std::vector<Cand> cands;
+    if (s->res_ok) cands.push_back({BQ_PATH_PIPE, 2, 0, 1, 0, 1});
     if (s->pipe_ok) {
       for (int slots = 2; slots <= 4; ++slots) {
         if (pipe_configure(s, slots, 0) != BQ_OK) break;
@@ -2075,6 +2478,7 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
       if (c.path == BQ_PATH_PIPE) {
         if ((rc = pipe_configure(s, c.slots, c.cap)) != BQ_OK) break;
         s->use_pipe = 1;
+        s->res_on = c.resident;
       } else if (c.path == BQ_PATH_TILED) {
         if ((c.cap != s->tile || c.gread != s->gread_sched) && apply_tile(s, c.cap, c.gread) != BQ_OK) {
           g_err.clear();  // a tile that does not fit
@@ -2092,6 +2496,7 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
         best.stage_path = c.path;
         best.pipe_slots = c.path == BQ_PATH_PIPE ? c.slots : 2;
         best.pipe_ctas_per_sm = c.path == BQ_PATH_PIPE ? c.cap : 0;
+        best.resident = c.resident;
         best.tile = c.path == BQ_PATH_TILED ? c.cap : s->tile;
         best.lanes = c.path == BQ_PATH_TILED ? c.lanes : lanes0;
         best.gread = c.path == BQ_PATH_TILED ? c.gread : s->gread_sched;
@@ -2103,6 +2508,7 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
   double best_solve = 0.0;
   if (rc == BQ_OK && s->solve_ok) {
     best_solve = 1e300;
+    s->res_on = best.resident;  // (the resident kernel serves both: one switch)
     const int kinds[2] = {BQ_SOLVE_MERGED, BQ_SOLVE_PROGRAM};
     for (int kind : kinds) {
       if (kind == BQ_SOLVE_MERGED && !s->solve_mg_ok) continue;
@@ -2132,6 +2538,8 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
   if (rc != BQ_OK) return rc;
   if (er != cudaSuccess) return fail(BQ_ECUDA, "restore: %s", cudaGetErrorString(er));
   CUDA_TRY(cudaStreamSynchronize(st));
+  s->res_known = res_known0;  // the state holds what it held
+  s->res_dirty = res_dirty0;
   if ((rc = bq_set_tune(s, &best)) != BQ_OK) return rc;
   s->tune_n = ntried;
   s->tune_step_us = best_step;
@@ -2232,6 +2640,7 @@ extern "C" int bq_grad(bq_state* s, double dt, int64_t n_steps, int checkpoint_e
   const size_t cs = s->dtype == BQ_F64 ? 16 : 8;
   const size_t arr = (size_t)s->total_elems * cs;
   const double tau0 = s->tau;
+  const int res_known0 = s->res_known, res_dirty0 = s->res_dirty;
   const int k = checkpoint_every;
   CUDA_TRY(cudaMemsetAsync(w + G.grad, 0, (size_t)std::max(1, s->grad_size) * sizeof(double), st));
   // Cooperative segment kernels (tiled path): one launch per segment and direction, grids of
@@ -2418,6 +2827,8 @@ extern "C" int bq_grad(bq_state* s, double dt, int64_t n_steps, int checkpoint_e
   }
   // leave the state as it was before the call (initial content, tau0)
   s->obs_valid = 0;
+  s->res_known = res_known0;
+  s->res_dirty = res_dirty0;
   CUDA_TRY(cudaMemcpyAsync(b + L.off_y, w + G.ckpt, arr, cudaMemcpyDeviceToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(b + L.off_comp, w + G.ckpt + arr, arr, cudaMemcpyDeviceToDevice, st));
   r = set_tau(s, tau0, st);
@@ -2679,6 +3090,8 @@ extern "C" int bq_load_state(bq_state* s, const void* host, void* stream) {
   // clears it first
   s->comp_zero = 1;
   s->obs_valid = 0;
+  s->res_known = 0;
+  s->res_dirty = 1;
   return BQ_OK;
 }
 

@@ -177,8 +177,10 @@ int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* opts, void*
 
 /* Advances every system of the state by n_steps RK4 steps of size dt (the mapped value
  * of dt must not exceed the bound checked at bq_map).  Single-mode states of the resident form
- * (bq_tune resident): all n_steps in one launch, every system on chip.  Else fused stage
- * kernels: on the pipelined single-mode path the four stages of a step run in one launch
+ * (bq_tune resident): all n_steps in one launch, every system on chip.  Tiled states of that
+ * form that fit the SMs' shared memory: all n_steps in one cooperative launch with a bounded grid
+ * barrier per stage (one that waits longer than about 2 s sets the error word: BQ_ETIMEOUT from
+ * the next synchronising call).  Else fused stage kernels: on the pipelined single-mode path the four stages of a step run in one launch
  * (bq_tune pipe_fused), otherwise one launch per stage; replayed from a CUDA graph.
  * Asynchronous on stream. */
 int bq_step(bq_state* s, double dt, int64_t n_steps, void* stream);
@@ -242,10 +244,13 @@ typedef struct bq_tune {
   int pipe_fused;        /* BQ_PATH_PIPE: 1 = the four stages of a step in one launch (every CTA
                           * runs its own systems' stages in order; no CTA waits for another),
                           * 0 = one launch per RK4 stage.  The arithmetic is the same. */
-  int resident;          /* BQ_PATH_PIPE, and BQ_SOLVE_MERGED with solve_ctas_per_sm = 0: 1 = the
-                          * resident kernel where the state has the form it takes (the default
-                          * there): all steps of a call in one launch, every system on chip, whatever
-                          * the other pipe_* fields say; 0 = the kernels those fields describe */
+  int resident;          /* 1 (the default where the state has the form they take): the resident
+                          * kernels, all steps of a call in one launch with the state on chip,
+                          * whatever the other schedule fields say: BQ_PATH_PIPE (one system per
+                          * group of warps; also BQ_SOLVE_MERGED with solve_ctas_per_sm = 0) and
+                          * BQ_PATH_TILED (the state spread over the SMs, one cooperative launch;
+                          * also bq_grad's segments with grad_coop).  0 = the kernels that the
+                          * other fields describe */
 } bq_tune;
 
 /* Current schedules of the state (step_us / solve_us: last bq_autotune result, else 0). */

@@ -18,6 +18,7 @@
 #include "../../include/bq.h"
 #include "bq_internal.h"
 #include "bq_launch.h"
+#include "bq_grid.h"
 #include "bq_resident.h"
 
 using cplx = std::complex<double>;
@@ -743,7 +744,7 @@ static int compile_problem(const bq_problem* p, const bq_map_opts& o, Compiled& 
 // State.
 // ---------------------------------------------------------------------------------------
 struct Layout {
-  size_t off_sys, off_terms, off_chans, off_chpar, off_work, off_m1, off_order, off_dc, off_pparams, off_precs, off_obs, off_rparams, off_rgroups, off_rbins, off_rflags, off_groups, off_entries, off_out, off_wtab, off_diag,
+  size_t off_sys, off_terms, off_chans, off_chpar, off_work, off_m1, off_order, off_dc, off_pparams, off_precs, off_obs, off_rparams, off_rgroups, off_rbins, off_rflags, off_gprobs, off_gtab, off_gpieces, off_gctas, off_gbar, off_groups, off_entries, off_out, off_wtab, off_diag,
       off_ctrl, off_init, off_y, off_comp, off_ua, off_ub, off_acc, total;
 };
 
@@ -753,6 +754,11 @@ struct Layout {
 //   list 2: the systems of list 0 in the general layout (for states loaded from outside).
 struct ResList {
   int b0 = 0, n_bins = 0, g0 = 0, n_groups = 0, smem = 0;
+};
+
+// A launch of the grid-resident kernels: CTAs [c0, c0 + n_ctas), none where the list does not fit.
+struct GridList {
+  int c0 = 0, n_ctas = 0, smem = 0;
 };
 
 struct bq_state {
@@ -775,7 +781,12 @@ struct bq_state {
   // launch, and the systems that fail it take list 2)
   int res_ok = 0, res_on = 0, res_mode = 1, res_ns = 1, res_obs = 0, res_known = 1, res_dirty = 0;
   ResList rlist[3];
-  // steps of equal length taken by the resident kernel since tau was run_tau0: their times are
+  // grid-resident kernels: lists (forward Hermitian, forward general, adjoint) and variant sizes
+  GridList glist[3];
+  int grid_np = 0, grid_ns = 0, grid_herm = 0;
+  int grid_pieces = 0, grid_adj = 0;  // pieces in the pool so far; the adjoint's list has been built
+  std::vector<bq::GridProb> gprobs;
+  // steps of equal length taken by the resident kernels since tau was run_tau0: their times are
   // run_tau0 + i run_dt however the calls split them (run_tau: tau after the last of them)
   double run_tau0 = 0.0, run_dt = 0.0, run_tau = 0.0;
   int64_t run_steps = 0;
@@ -862,6 +873,11 @@ struct Plan {
   std::vector<bq::ResGroup> rgroups;
   std::vector<bq::ResBin> rbins;
   ResList rlist[3];
+  // grid-resident kernels (k_grid_fwd, k_grid_adj): problems, tables, capacity of the lists' pieces
+  int grid_ok = 0, grid_np = 0, grid_ns = 0, grid_herm = 0;
+  size_t grid_cap = 0;
+  std::vector<bq::GridProb> gprobs;
+  std::vector<double> gtab;
   Layout L{};
 };
 
@@ -958,6 +974,24 @@ static void build_work(const std::vector<SysDesc>& sys, size_t cs, int tile, int
 // Anything else keeps the streaming and per-term kernels.
 // ---------------------------------------------------------------------------------------
 
+// A drive envelope's record in a parameter block (FP32 constants of a Gaussian included).
+static bq::PipeChan pipe_chan(const ChanDesc& cd, const double* chpar) {
+  bq::PipeChan pc;
+  std::memset(&pc, 0, sizeof(pc));
+  for (int i = 0; i < 4 && i < cd.n_par; ++i) pc.p[i] = chpar[cd.par_off + i];
+  pc.f[0] = (float)pc.p[0];
+  pc.f[1] = (float)pc.p[1];
+  if (cd.kind == BQ_CH_GAUSS) {
+    pc.f[2] = (float)(1.0 / (2.0 * pc.p[3] * pc.p[3]));
+    pc.f[3] = (float)pc.p[2];
+    pc.c_lo = (float)(pc.p[2] - (double)pc.f[3]);
+  }
+  pc.kind = cd.kind;
+  pc.par_off = cd.par_off;
+  pc.n_par = cd.n_par;
+  return pc;
+}
+
 // Rows per strip and warps of a system: the fewest issue slots, counting a
 // row as 1 and a strip's fixed part (edges, stage set-up) as 1.4 rows.  0 if it does not fit.
 static int res_shape(int M, int cs, bool herm, int& rb, int& nb) {
@@ -977,6 +1011,19 @@ static int res_shape(int M, int cs, bool herm, int& rb, int& nb) {
     }
   }
   return best;
+}
+
+// Row and column tables of a sandwich term are alike: they differ by a factor only (its rate, to
+// rounding).
+static bool same_table(const std::vector<double>& x, const std::vector<double>& y) {
+  double r = 0.0;
+  for (size_t k = 0; k < x.size(); ++k) {
+    if ((x[k] == 0.0) != (y[k] == 0.0)) return false;
+    if (x[k] == 0.0) continue;
+    if (r == 0.0) r = x[k] / y[k];
+    if (std::abs(x[k] - r * y[k]) > 1e-14 * std::abs(x[k])) return false;
+  }
+  return true;
 }
 
 static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, const EvalGroup& eg, int term_off,
@@ -1055,19 +1102,9 @@ static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, co
       const double* cp = P.chpar.data() + cd.par_off;
       h.ch = 1;
       h.conj = off[0]->conj;
-      for (int i = 0; i < 4 && i < cd.n_par; ++i) h.chan.p[i] = cp[i];
-      h.chan.kind = cd.kind;
-      h.chan.par_off = cd.par_off;
-      h.chan.n_par = cd.n_par;
-      h.chan.f[0] = (float)cp[0];
-      h.chan.f[1] = (float)cp[1];
+      h.chan = pipe_chan(cd, P.chpar.data());
       switch (cd.kind) {
         case BQ_CH_GAUSS:
-          h.chan.f[2] = (float)(1.0 / (2.0 * cp[3] * cp[3]));
-          h.chan.f[3] = (float)cp[2];
-          h.chan.c_lo = (float)(cp[2] - (double)h.chan.f[3]);
-          imag = imag && cp[1] == 0.0;
-          break;
         case BQ_CH_CONST: imag = imag && cp[1] == 0.0; break;
         case BQ_CH_PWC:
           for (int i = 3; i < cd.n_par; i += 2) imag = imag && cp[i] == 0.0;
@@ -1079,15 +1116,8 @@ static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, co
   if (!imag) mode = 2;
   if (splus) ns = 2;
   herm = w[0] == w[2] && w[1] == w[3];
-  for (int k = 0; k < M && herm; ++k) {
-    herm = d[M + k] == std::conj(d[k]);
-    // row and column tables of a sandwich term differ by a factor only (its rate, to rounding)
-    for (int q = 4; q < 8 && herm; q += 2)
-      for (int j = 0; j < k && herm; ++j) {
-        const double u = w[q][k] * w[q + 1][j], v = w[q][j] * w[q + 1][k];
-        herm = std::abs(u - v) <= 1e-14 * std::abs(u);
-      }
-  }
+  for (int k = 0; k < M && herm; ++k) herm = d[M + k] == std::conj(d[k]);
+  herm = herm && same_table(w[4], w[5]) && same_table(w[6], w[7]);
   blk.resize(sizeof(h));
   auto put = [&](double v) {
     if (cs == 16) blk.insert(blk.end(), (unsigned char*)&v, (unsigned char*)&v + 8);
@@ -1208,6 +1238,310 @@ static void make_res_plan(Plan& P, const bq_problem* const* probs, const std::ve
       !res_pack(P, hs, poff, cs, false, P.rlist[2]))
     return;
   P.res_ok = 1;
+}
+
+// ---------------------------------------------------------------------------------------
+// Plan of the grid-resident kernels (bq_grid.cuh): every problem's terms in the form they
+// evaluate.  Taken: static shift-0 terms on one side; off-diagonal terms that come in the four
+// pieces of a Hermitian H's conjugate pair (left: a and -conj(a) with opposite shifts, right: -a
+// and conj(a)), any modes, any envelope, any number of pairs per shift, at most BQ_GRID_MAXP;
+// sandwich terms with a static real coefficient that shift x and y alike, at most BQ_GRID_MAXS,
+// the secular ones included.  Anything else (time-dependent diagonal terms, jump operators of
+// several monomials) keeps the tiled kernels.  So do states with more points than the SMs'
+// shared memory holds.
+// ---------------------------------------------------------------------------------------
+static const int kGridMaxCtas = BQ_GRID_MAX_CTAS;
+static const int64_t kGridMaxPoints = 152 * 2500;
+
+// X or Y term t's weights over the flat index of its side; S terms: of side y's dimensions.
+static std::vector<double> flat_weights(const Compiled& C, const TermDesc& td, int wbase, bool y) {
+  std::vector<double> w(C.n_g, 1.0);
+  for (int k = 0; k < C.n_g; ++k) {
+    int idx[BQ_MAX_MODES], r = k;
+    for (int j = C.nm - 1; j >= 0; --j) { idx[j] = r % C.M[j]; r /= C.M[j]; }
+    for (int a = 0; a < td.n_act; ++a) {
+      const int d = td.dim[a];
+      if ((d >= C.nm) != y) continue;
+      const int i = idx[y ? d - C.nm : d];
+      // zero where the source leaves the grid
+      const int src = i + td.sh[a];
+      w[k] *= src < 0 || src >= C.M[y ? d - C.nm : d] ? 0.0 : C.wtab[td.wtab[a] - wbase + i];
+    }
+  }
+  return w;
+}
+
+static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wbase, int grad_off, bq::GridProb& G,
+                         std::vector<double>& tab, bool& herm) {
+  const int ng = C.n_g, nm = C.nm;
+  std::memset(&G, 0, sizeof(G));
+  G.ng = ng;
+  G.has_sep = C.has_sep; G.has_r = C.has_r; G.r_diag = C.r_diag;
+  G.n_params = C.n_params;
+  G.grad_off = grad_off;
+  std::vector<cplx> d[2];
+  for (int y = 0; y < 2; ++y) {
+    d[y].assign(ng, cplx(0, 0));
+    for (int k = 0; k < ng; ++k) {
+      int r = k;
+      for (int j = nm - 1; j >= 0; --j) {
+        int off = 0;
+        for (int q = 0; q < y * nm + j; ++q) off += C.M[q % nm];
+        d[y][k] += C.diag[off + r % C.M[j]];
+        r /= C.M[j];
+      }
+    }
+  }
+  std::vector<std::vector<double>> pw, sw;  // per pair xm xp ym yp, per sandwich term sx sy
+  std::vector<std::vector<cplx>> hw;        // per diagonal parameter hx hy
+  const int nt = (int)C.terms.size();
+  std::vector<char> used(nt, 0);
+  auto term = [&](int t) -> const TermDesc& { return P.terms[term_off + t]; };
+  for (int t = 0; t < nt; ++t) {
+    const TermDesc& td = term(t);
+    const cplx c(td.c_re, td.c_im);
+    if (td.side == bq::SIDE_S) {
+      if (td.ch >= 0 || td.param >= 0 || c.imag() != 0.0 || td.deltaGx != td.deltaGy || G.ns == BQ_GRID_MAXS) return false;
+      std::vector<double> wx = flat_weights(C, td, wbase, false), wy = flat_weights(C, td, wbase, true);
+      for (double& v : wx) v *= c.real();
+      G.ss[G.ns] = td.deltaGx;
+      if (td.diagp1) {
+        const int j = td.diagp1 - 1;
+        int st = 1;
+        for (int q = nm - 1; q > j; --q) st *= C.M[q];
+        G.sst[G.ns] = st;
+        G.sM[G.ns] = C.M[j];
+      }
+      ++G.ns;
+      sw.push_back(wx);
+      sw.push_back(wy);
+      used[t] = 1;
+      continue;
+    }
+    const bool y = td.side == bq::SIDE_Y;
+    bool shift0 = true;
+    for (int a = 0; a < td.n_act; ++a) shift0 = shift0 && td.sh[a] == 0;
+    if (shift0) {
+      if (td.ch >= 0) return false;
+      const std::vector<double> w = flat_weights(C, td, wbase, y);
+      for (int k = 0; k < ng; ++k) d[y][k] += c * w[k];
+      if (td.gslot_param >= 0) {
+        int q = 0;
+        while (q < G.nt && G.tpar[q] != td.gslot_param) ++q;
+        if (q == G.nt) {
+          if (G.nt == BQ_GRID_MAXT) return false;
+          G.tpar[G.nt++] = td.gslot_param;
+          hw.push_back(std::vector<cplx>(ng, cplx(0, 0)));
+          hw.push_back(std::vector<cplx>(ng, cplx(0, 0)));
+        }
+        for (int k = 0; k < ng; ++k) hw[2 * q + y][k] += cplx(td.cb_re, td.cb_im) * w[k];
+      }
+      used[t] = 1;
+    } else if ((y ? td.deltaGy : td.deltaGx) == 0) {
+      return false;  // shifts that cancel in the flat index
+    }
+  }
+  // conjugate pairs
+  for (int t = 0; t < nt; ++t) {
+    if (used[t] || term(t).side != bq::SIDE_X) continue;
+    const TermDesc& tm = term(t);
+    const cplx a(tm.c_re, tm.c_im);
+    const int dl = -tm.deltaGx;
+    auto find = [&](int side, int delta, cplx c, int conj) {
+      for (int q = 0; q < nt; ++q) {
+        const TermDesc& o = term(q);
+        if (used[q] || q == t || o.side != side || (side == bq::SIDE_X ? o.deltaGx : o.deltaGy) != delta) continue;
+        if (o.ch != tm.ch || o.param != tm.param || cplx(o.c_re, o.c_im) != c || (o.ch >= 0 && o.conj != conj)) continue;
+        // the same shifts per mode, up to the sign
+        return q;
+      }
+      return -1;
+    };
+    const int xp = find(bq::SIDE_X, dl, -std::conj(a), 1 - tm.conj);
+    if (xp < 0) return false;
+    used[t] = used[xp] = 1;
+    const int yp = find(bq::SIDE_Y, dl, -a, tm.conj);
+    if (yp < 0) return false;
+    used[yp] = 1;
+    const int ym = find(bq::SIDE_Y, -dl, std::conj(a), 1 - tm.conj);
+    if (ym < 0 || G.np == BQ_GRID_MAXP) return false;
+    used[ym] = 1;
+    const int j = G.np++;
+    G.dlt[j] = dl;
+    G.a_re[j] = tm.c_re; G.a_im[j] = tm.c_im;
+    G.cb_re[j] = tm.cb_re; G.cb_im[j] = tm.cb_im;
+    G.cj[j] = tm.conj;
+    G.gpar[j] = tm.gslot_param;
+    G.gpwc[j] = tm.gslot_pwc;
+    G.ch[j] = -1;
+    if (tm.ch >= 0) {
+      const ChanDesc& cd = P.chans[tm.ch];
+      int q = 0;
+      while (q < G.nch && !(G.cd[q].par_off == cd.par_off && G.cd[q].kind == cd.kind)) ++q;
+      if (q == G.nch) {
+        G.cd[G.nch] = cd;
+        G.chan[G.nch++] = pipe_chan(cd, P.chpar.data());
+      }
+      G.ch[j] = q;
+    }
+    for (int q : {t, xp}) pw.push_back(flat_weights(C, term(q), wbase, false));
+    for (int q : {ym, yp}) pw.push_back(flat_weights(C, term(q), wbase, true));
+  }
+  for (int t = 0; t < nt; ++t)
+    if (!used[t]) return false;
+  // Hermitian structure: mirrored weights
+  herm = C.has_r && !C.r_diag && ng >= 4;
+  for (int k = 0; k < ng && herm; ++k) {
+    herm = d[1][k] == std::conj(d[0][k]);
+    for (int j = 0; j < G.np && herm; ++j) herm = pw[4 * j][k] == pw[4 * j + 2][k] && pw[4 * j + 1][k] == pw[4 * j + 3][k];
+  }
+  for (int s = 0; s < G.ns && herm; ++s) herm = same_table(sw[2 * s], sw[2 * s + 1]);
+  // tables
+  auto putc = [&](const std::vector<cplx>& v) { for (const cplx& x : v) { tab.push_back(x.real()); tab.push_back(x.imag()); } };
+  auto putr = [&](const std::vector<double>& v) { tab.insert(tab.end(), v.begin(), v.end()); };
+  // w at the index from which a source shift of `shift` leads to k: the transposed weight
+  auto shifted = [&](const std::vector<double>& w, int shift) {
+    std::vector<double> o(ng, 0.0);
+    for (int k = 0; k < ng; ++k)
+      if (k - shift >= 0 && k - shift < ng) o[k] = w[k - shift];
+    return o;
+  };
+  while (tab.size() % 2) tab.push_back(0.0);
+  G.tab = (long long)tab.size();
+  putc(d[0]);
+  putc(d[1]);
+  for (auto& w : pw) putr(w);
+  for (auto& w : sw) putr(w);
+  for (int j = 0; j < G.np; ++j) {  // sources k - dlt, k + dlt, l - dlt, l + dlt
+    const int dl = G.dlt[j];
+    putr(shifted(pw[4 * j], -dl));
+    putr(shifted(pw[4 * j + 1], dl));
+    putr(shifted(pw[4 * j + 2], -dl));
+    putr(shifted(pw[4 * j + 3], dl));
+  }
+  for (int s = 0; s < G.ns; ++s) {
+    putr(shifted(sw[2 * s], G.ss[s]));
+    putr(shifted(sw[2 * s + 1], G.ss[s]));
+  }
+  for (auto& h : hw) putc(h);
+  return true;
+}
+
+// f(kind, points, points per piece) for every kind of point of system sd in list `list`.
+template <typename F>
+static void grid_kinds(const SysDesc& sd, const bq::GridProb& G, int list, F f) {
+  const bool hm = list == 0 && G.herm;
+  const int cols = sd.n_g | 1, len = list == 2 ? BQ_GRID_GLEN : 32;
+  if (sd.has_r) {
+    if (hm) f(bq::GRID_H, (cols / 2 + 1) * cols, 32);
+    else f(sd.r_diag ? bq::GRID_D : bq::GRID_R, sd.n_r, 32);
+  }
+  if (sd.has_sep) {
+    f(bq::GRID_X, sd.n_g, len);
+    if (!hm) f(bq::GRID_Y, sd.n_g, len);
+  }
+}
+static size_t grid_count(const std::vector<SysDesc>& sys, const std::vector<bq::GridProb>& probs, int list) {
+  size_t n = 0;
+  for (const SysDesc& sd : sys) grid_kinds(sd, probs[sd.prob], list, [&](int, int pts, int len) { n += (pts + len - 1) / len; });
+  return n;
+}
+
+static void make_grid_plan(Plan& P, const bq_problem* const* probs) {
+  const int B = (int)P.comp.size();
+  int64_t pts = 0;
+  for (const SysDesc& sd : P.sys) pts += sd.n_r + 2 * (sd.has_sep ? sd.n_g : 0);
+  if (P.total_elems >= ((int64_t)1 << 31) || pts > kGridMaxPoints || B > kGridMaxCtas) return;
+  std::vector<int> term_off(B, 0);
+  std::vector<char> herm(B, 1);
+  for (const SysDesc& sd : P.sys) {
+    term_off[sd.prob] = sd.term_off;
+    if (sd.has_sep && !(sd.p_flat >= 0 && sd.p_flat == sd.q_flat && sd.c_re == 0.0)) herm[sd.prob] = 0;
+  }
+  for (int b = 0; b < B; ++b) {
+    bq::GridProb G;
+    bool hm = false;
+    if (!grid_problem(P, P.comp[b], term_off[b], P.wbase[b], P.grad_offs[b], G, P.gtab, hm)) {
+      P.gprobs.clear();
+      P.gtab.clear();
+      return;
+    }
+    if (P.comp[b].method == BQ_METHOD_DIRECT)  // A(0) itself
+      for (auto& [kl, v] : probs[b]->measured) {
+        auto it = probs[b]->measured.find({kl.second, kl.first});
+        if (v != cplx(0, 0) && (it == probs[b]->measured.end() || it->second != std::conj(v))) hm = false;
+      }
+    herm[b] = herm[b] && hm;
+    G.herm = herm[b];
+    P.grid_herm = P.grid_herm || herm[b];
+    P.grid_np = std::max(P.grid_np, G.np);
+    P.grid_ns = std::max(P.grid_ns, G.ns);
+    P.gprobs.push_back(G);
+  }
+  for (int list = P.grid_herm ? 0 : 1; list < 3; ++list) P.grid_cap += grid_count(P.sys, P.gprobs, list);
+  P.grid_ok = 1;
+}
+
+// The pieces of a list (0: forward, Hermitian layout where possible; 1: forward, general layout; 2:
+// adjoint), spread over at most nsm CTAs with the smallest largest share, every CTA within one
+// problem (the adjoint: one system).  A unit's pieces are dealt out to its CTAs in turn, since the
+// kinds differ in cost.  gl.n_ctas is 0 where the list does not fit.
+static int build_grid_list(const std::vector<SysDesc>& sys, const std::vector<bq::GridProb>& probs, int list, int dtype,
+                           int np, int ns, std::vector<bq::GridPiece>& pieces, std::vector<bq::GridCta>& ctas, GridList& gl) {
+  int dev = 0, nsm = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  nsm = std::min(nsm, kGridMaxCtas);
+  gl.n_ctas = gl.smem = 0;
+  std::vector<std::vector<bq::GridPiece>> unit;
+  size_t total = 0;
+  int last = -1;
+  for (int i = 0; i < (int)sys.size(); ++i) {
+    const SysDesc& sd = sys[i];
+    const int u = list == 2 ? i : sd.prob;
+    if (u != last) {  // (a problem's systems are contiguous)
+      if ((int)unit.size() == nsm) return BQ_OK;
+      unit.emplace_back();
+      last = u;
+    }
+    grid_kinds(sd, probs[sd.prob], list, [&](int kind, int pts, int len) {
+      for (int s = 0; s < pts; s += len) {
+        bq::GridPiece g;
+        std::memset(&g, 0, sizeof(g));
+        g.sys = i; g.kind = kind; g.start = s; g.len = std::min(len, pts - s);
+        g.off_gx = (int)sd.off_gx; g.off_gy = (int)sd.off_gy; g.off_r = (int)sd.off_r;
+        g.c_re = sd.c_re; g.c_im = sd.c_im;
+        g.dc_off = sd.dc_off;
+        unit.back().push_back(g);
+      }
+      total += (pts + len - 1) / len;
+    });
+  }
+  int share = std::max(1, (int)((total + nsm - 1) / nsm));
+  for (;; ++share) {
+    size_t n = 0;
+    for (auto& v : unit) n += (v.size() + share - 1) / share;
+    if (n <= (size_t)nsm) break;
+  }
+  pieces.clear();
+  ctas.clear();
+  for (auto& v : unit) {
+    const int c = ((int)v.size() + share - 1) / share;
+    for (int q = 0; q < c; ++q) {
+      bq::GridCta cta{sys[v[0].sys].prob, (int)pieces.size(), 0, 0};
+      for (int i = q; i < (int)v.size(); i += c) pieces.push_back(v[i]);
+      cta.n = (int)pieces.size() - cta.p0;
+      ctas.push_back(cta);
+    }
+  }
+  size_t sm = 0;
+  for (const bq::GridProb& g : probs) sm = std::max(sm, bq::grid_smem(share, g, list == 2, dtype == BQ_F64 ? 16 : 8));
+  int most = 0;
+  if (sm <= BQ_GRID_SMEM_MAX) CUDA_TRY(bq::grid_max_ctas(dtype, np, ns, list == 2, (int)sm, &most));
+  if (most < (int)ctas.size()) return BQ_OK;
+  gl.n_ctas = (int)ctas.size();
+  gl.smem = (int)sm;
+  return BQ_OK;
 }
 
 static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o, Plan& P) {
@@ -1457,17 +1791,7 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
           for (int c = 0; c < 2; ++c) {
             if (chs[c] < 0) break;
             const ChanDesc& cd = P.chans[chs[c]];
-            bq::PipeChan pc;
-            std::memset(&pc, 0, sizeof(pc));
-            for (int i = 0; i < 4 && i < cd.n_par; ++i) pc.p[i] = P.chpar[cd.par_off + i];
-            pc.f[0] = (float)pc.p[0];
-            pc.f[1] = (float)pc.p[1];
-            pc.f[2] = cd.kind == BQ_CH_GAUSS ? (float)(1.0 / (2.0 * pc.p[3] * pc.p[3])) : 0.f;
-            pc.f[3] = cd.kind == BQ_CH_GAUSS ? (float)pc.p[2] : 0.f;
-            pc.c_lo = cd.kind == BQ_CH_GAUSS ? (float)(pc.p[2] - (double)pc.f[3]) : 0.f;
-            pc.kind = cd.kind;
-            pc.par_off = cd.par_off;
-            pc.n_par = cd.n_par;
+            const bq::PipeChan pc = pipe_chan(cd, P.chpar.data());
             blk.insert(blk.end(), (const unsigned char*)&pc, (const unsigned char*)&pc + sizeof(pc));
             ++n_ch;
           }
@@ -1621,6 +1945,8 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
     }
   }
 
+  make_grid_plan(P, probs);
+
   // ---- work items (tiles of R; the first tile of a system also updates G_x, G_y) ------
   for (SysDesc& sd : P.sys) {
     int ns = 0, cw = 0;
@@ -1674,6 +2000,11 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
   L.off_rgroups = seg(P.rgroups.size() * sizeof(bq::ResGroup));
   L.off_rbins = seg(P.rbins.size() * sizeof(bq::ResBin));
   L.off_rflags = seg(P.res_ok ? P.sys.size() : 0);
+  L.off_gprobs = seg(P.gprobs.size() * sizeof(bq::GridProb));
+  L.off_gtab = seg(P.gtab.size() * rs);
+  L.off_gpieces = seg(P.grid_cap * sizeof(bq::GridPiece));
+  L.off_gctas = seg(P.grid_ok ? 3 * kGridMaxCtas * sizeof(bq::GridCta) : 0);
+  L.off_gbar = seg(P.grid_ok ? sizeof(unsigned int) : 0);
   L.off_dc = seg(P.dc.size() * sizeof(double2));
   L.off_groups = seg(P.groups.size() * sizeof(EvalGroup));
   L.off_entries = seg(P.entries.size() * sizeof(EvalEntry));
@@ -1798,6 +2129,30 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
     for (size_t i = 0; i < d.size(); ++i) d[i] = make_float2((float)P.diag[i].real(), (float)P.diag[i].imag());
     CUDA_TRY(up(L.off_diag, d.data(), d.size() * sizeof(float2)));
   }
+  // (the adjoint's list, and a single-mode state's, are built by the first bq_grad: states that are
+  // only stepped do not pay for them)
+  GridList glist[3];
+  std::vector<bq::GridPiece> gpieces[2];
+  std::vector<bq::GridCta> gctas[2];
+  int grid_pieces = 0;
+  if (P.grid_ok) {
+    for (int q = P.use_m1 ? 2 : P.grid_herm ? 0 : 1; q < 2; ++q) {
+      r = build_grid_list(P.sys, P.gprobs, q, o->dtype, P.grid_np, P.grid_ns, gpieces[q], gctas[q], glist[q]);
+      if (r != BQ_OK) return r;
+      for (bq::GridCta& c : gctas[q]) c.p0 += grid_pieces;
+      CUDA_TRY(up(L.off_gpieces + grid_pieces * sizeof(bq::GridPiece), gpieces[q].data(), gpieces[q].size() * sizeof(bq::GridPiece)));
+      glist[q].c0 = q * kGridMaxCtas;
+      CUDA_TRY(up(L.off_gctas + glist[q].c0 * sizeof(bq::GridCta), gctas[q].data(), gctas[q].size() * sizeof(bq::GridCta)));
+      grid_pieces += (int)gpieces[q].size();
+    }
+    CUDA_TRY(up(L.off_gprobs, P.gprobs.data(), P.gprobs.size() * sizeof(bq::GridProb)));
+    if (o->dtype == BQ_F64) {
+      CUDA_TRY(up(L.off_gtab, P.gtab.data(), P.gtab.size() * sizeof(double)));
+    } else {
+      const auto t32 = to_real<float>(P.gtab);
+      CUDA_TRY(up(L.off_gtab, t32.data(), t32.size() * sizeof(float)));
+    }
+  }
   CUDA_TRY(cudaMemsetAsync(base + L.off_ctrl, 0, 64, s));
   CUDA_TRY(up(L.off_init, P.init.data(), P.init.size() * sizeof(InitEntry)));
   const size_t cs = o->dtype == BQ_F64 ? 16 : 8;
@@ -1852,6 +2207,13 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
   st->res_ns = P.res_ns;
   st->res_obs = P.res_obs;
   for (int q = 0; q < 3; ++q) st->rlist[q] = P.rlist[q];
+  for (int q = 0; q < 3; ++q) st->glist[q] = glist[q];
+  st->grid_np = P.grid_np;
+  st->grid_ns = P.grid_ns;
+  st->grid_herm = P.grid_herm;
+  st->grid_pieces = grid_pieces;
+  st->gprobs = P.gprobs;
+  if (!P.use_m1 && glist[1].n_ctas > 0) st->res_on = 1;
 
   st->grad_size = P.grad_size;
   st->adj_smem = P.adj_smem;
@@ -1986,6 +2348,103 @@ static cudaError_t launch_any_stage(bq_state* s, const bq::StageArgs& a, cudaStr
   return bq::launch_stage(a, s->dtype, s->nm, s->n_work, s->smem_bytes, st);
 }
 
+// The grid-resident kernel serves bq_step on the tiled path (res_on is the switch of both kinds).
+static bool grid_on(const bq_state* s) { return !s->use_m1 && s->res_on && s->glist[1].n_ctas > 0; }
+
+// Starts or continues a run of equal steps (see bq_state::run_tau0).
+static void run_begin(bq_state* s, double dt) {
+  if (s->tau != s->run_tau || dt != s->run_dt || s->run_steps == 0) {
+    s->run_tau0 = s->tau;
+    s->run_dt = dt;
+    s->run_steps = 0;
+  }
+}
+static void run_end(bq_state* s, double dt, int64_t n) {
+  s->run_steps += n;
+  s->tau = s->run_tau = s->run_tau0 + (double)s->run_steps * dt;
+}
+
+// Arguments of the grid-resident kernels for list q.
+static bq::GridArgs grid_args(bq_state* s, int q, double dt) {
+  char* b = s->pool;
+  const Layout& L = s->L;
+  bq::GridArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.ctas = (const bq::GridCta*)(b + L.off_gctas) + s->glist[q].c0;
+  a.pieces = (const bq::GridPiece*)(b + L.off_gpieces);
+  a.probs = (const bq::GridProb*)(b + L.off_gprobs);
+  a.tab = b + L.off_gtab;
+  a.chpar = (const double*)(b + L.off_chpar);
+  a.y = b + L.off_y;
+  a.comp = b + L.off_comp;
+  a.ua = b + L.off_ua;
+  a.ub = b + L.off_ub;
+  a.arr = (size_t)s->total_elems * (s->dtype == BQ_F64 ? 16 : 8);
+  a.bar = (unsigned int*)(b + L.off_gbar);
+  a.error = (unsigned int*)(b + L.off_ctrl + 32);
+  a.dc = (const double2*)(b + L.off_dc);
+  a.reverse = s->reverse;
+  a.herm = q == 0;
+  a.dt = dt;
+  a.horizon = s->horizon;
+  return a;
+}
+static cudaError_t launch_grid(bq_state* s, const bq::GridArgs& a, int q, cudaStream_t st) {
+  const auto launch = s->dtype == BQ_F64 ? bq::launch_grid_f64 : bq::launch_grid_f32;
+  return launch(a, s->grid_np, s->grid_ns, q == 2, s->glist[q].n_ctas, s->glist[q].smem, st);
+}
+
+// Builds and uploads the lists bq_grad needs, at its first call: the adjoint's, and in single-mode
+// states (whose steps take other kernels) the forward one.
+static int ensure_grid_adjoint(bq_state* s) {
+  if (s->grid_adj || s->gprobs.empty()) return BQ_OK;
+  for (int q = s->use_m1 ? 1 : 2; q < 3; ++q) {
+    if (q == 2 && s->glist[1].n_ctas == 0) break;
+    std::vector<bq::GridPiece> pieces;
+    std::vector<bq::GridCta> ctas;
+    GridList gl;
+    const int r = build_grid_list(s->sys, s->gprobs, q, s->dtype, s->grid_np, s->grid_ns, pieces, ctas, gl);
+    if (r != BQ_OK) return r;
+    gl.c0 = q * kGridMaxCtas;
+    for (bq::GridCta& c : ctas) c.p0 += s->grid_pieces;
+    if (gl.n_ctas > 0) {
+      CUDA_TRY(cudaMemcpy(s->pool + s->L.off_gpieces + s->grid_pieces * sizeof(bq::GridPiece), pieces.data(),
+                          pieces.size() * sizeof(bq::GridPiece), cudaMemcpyHostToDevice));
+      CUDA_TRY(cudaMemcpy(s->pool + s->L.off_gctas + gl.c0 * sizeof(bq::GridCta), ctas.data(),
+                          ctas.size() * sizeof(bq::GridCta), cudaMemcpyHostToDevice));
+      s->grid_pieces += (int)pieces.size();
+    }
+    s->glist[q] = gl;
+  }
+  s->grid_adj = 1;
+  return BQ_OK;
+}
+
+// n steps from s->tau with the grid-resident kernel in one launch; advances s->tau.
+static cudaError_t enqueue_grid(bq_state* s, double dt, int64_t n, cudaStream_t st, int* launches) {
+  run_begin(s, dt);
+  const int q = s->res_known && s->glist[0].n_ctas > 0 ? 0 : 1;
+  if (q == 1 && s->grid_herm) s->res_known = 0;  // (leaves Hermitian systems Hermitian to rounding)
+  bq::GridArgs a = grid_args(s, q, dt);
+  *launches = 0;
+  const int64_t most = 1 << 24;  // steps per launch (32-bit step and barrier counters)
+  for (int64_t done = 0; done < n;) {
+    const int64_t m = std::min(most, n - done);
+    a.n_steps = (int)m;
+    a.tau0 = s->run_tau0;
+    a.step0 = s->run_steps + done;
+    a.comp_zero = s->comp_zero;
+    const cudaError_t e = launch_grid(s, a, q, st);
+    if (e != cudaSuccess) return e;
+    s->comp_zero = 0;
+    ++*launches;
+    done += m;
+  }
+  run_end(s, dt, n);
+  s->obs_valid = 0;
+  return cudaSuccess;
+}
+
 // The resident kernel serves bq_step on the pipelined path and bq_solve's merged kernel.
 static bool res_on(const bq_state* s) { return s->res_ok && s->res_on && s->use_pipe; }
 
@@ -2014,11 +2473,7 @@ static cudaError_t enqueue_resident(bq_state* s, double dt, int64_t n, cudaStrea
   a.reverse = s->reverse;
   a.dt = dt;
   a.horizon = s->horizon;
-  if (s->tau != s->run_tau || dt != s->run_dt || s->run_steps == 0) {
-    s->run_tau0 = s->tau;
-    s->run_dt = dt;
-    s->run_steps = 0;
-  }
+  run_begin(s, dt);
   const int64_t most = 1 << 30;  // steps per launch (32-bit counter)
   for (int64_t done = 0; done < n;) {
     const int64_t m = std::min(most, n - done);
@@ -2040,17 +2495,15 @@ static cudaError_t enqueue_resident(bq_state* s, double dt, int64_t n, cudaStrea
     s->comp_zero = 0;  // every system's comp is written
     done += m;
   }
-  s->run_steps += n;
-  s->tau = s->run_tau = s->run_tau0 + (double)s->run_steps * dt;
+  run_end(s, dt, n);
   s->obs_valid = s->res_obs;
   return cudaSuccess;
 }
 
 static cudaError_t enqueue_steps(bq_state* s, double dt, int64_t n, cudaStream_t st) {
-  if (res_on(s)) {
-    int k = 0;
-    return enqueue_resident(s, dt, n, st, &k);
-  }
+  int k = 0;
+  if (res_on(s)) return enqueue_resident(s, dt, n, st, &k);
+  if (grid_on(s)) return enqueue_grid(s, dt, n, st, &k);
   s->res_known = 0;  // (these kernels may leave a Hermitian system Hermitian to rounding only)
   s->res_dirty = 1;
   if (pipe_fused_on(s)) {
@@ -2089,9 +2542,9 @@ extern "C" int bq_step(bq_state* s, double dt, int64_t n_steps, void* stream) {
   if (n_steps == 0) return BQ_OK;
   cudaStream_t st = (cudaStream_t)stream;
   char* b = s->pool;
-  if (res_on(s)) {
+  if (res_on(s) || grid_on(s)) {
     int k = 0;
-    CUDA_TRY(enqueue_resident(s, dt, n_steps, st, &k));
+    CUDA_TRY(res_on(s) ? enqueue_resident(s, dt, n_steps, st, &k) : enqueue_grid(s, dt, n_steps, st, &k));
     g_launches += k;
     return BQ_OK;
   }
@@ -2345,7 +2798,7 @@ extern "C" int bq_set_tune(bq_state* s, const bq_tune* t) {
   s->lanes = t->lanes == 0 ? default_lanes(s->sys) : t->lanes;
   s->grad_coop = t->grad_coop != 0;
   s->pipe_fused = t->pipe_fused != 0;
-  s->res_on = s->res_ok && t->resident != 0;
+  s->res_on = (s->res_ok || (!s->use_m1 && s->glist[1].n_ctas > 0)) && t->resident != 0;
   drop_graph(s);
   return BQ_OK;
 }
@@ -2426,6 +2879,8 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
       int launches = solve ? 1 : (int)(ns * kernels_per_step(s));
       if (solve ? solve_resident(s) : res_on(s))
         CUDA_TRY(enqueue_resident(s, dt, ns, st, &launches));
+      else if (!solve && grid_on(s))
+        CUDA_TRY(enqueue_grid(s, dt, ns, st, &launches));
       else
         CUDA_TRY(solve ? enqueue_solve(s, dt, ns, st) : enqueue_steps(s, dt, ns, st));
       g_launches += launches;
@@ -2450,6 +2905,7 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
     struct Cand { int path, slots, cap, lanes, gread, resident = 0; };
     std::vector<Cand> cands;
     if (s->res_ok) cands.push_back({BQ_PATH_PIPE, 2, 0, 1, 0, 1});
+    if (!s->use_m1 && s->glist[1].n_ctas > 0) cands.push_back({BQ_PATH_TILED, 0, s->tile, s->lanes, s->gread_sched, 1});
     if (s->pipe_ok) {
       for (int slots = 2; slots <= 4; ++slots) {
         if (pipe_configure(s, slots, 0) != BQ_OK) break;
@@ -2485,6 +2941,7 @@ extern "C" int bq_autotune(bq_state* s, double dt, int trial_steps, void* scratc
           continue;
         }
         s->lanes = c.lanes;
+        s->res_on = c.resident;
       } else {
         s->use_pipe = 0;
       }
@@ -2646,14 +3103,22 @@ extern "C" int bq_grad(bq_state* s, double dt, int64_t n_steps, int checkpoint_e
   // Cooperative segment kernels (tiled path): one launch per segment and direction, grids of
   // at most the resident CTAs and no more than the largest phase's items.
   int grid_f = 0, grid_b = 0;
-  if (s->grad_coop && !s->use_m1) {
+  {
+    const int rg = s->grad_coop && (s->res_on || s->use_m1) ? ensure_grid_adjoint(s) : BQ_OK;
+    if (rg != BQ_OK) return rg;
+  }
+  const bool grid_lists = s->glist[1].n_ctas > 0 && s->glist[2].n_ctas > 0;
+  if (s->grad_coop && !s->use_m1 && !(s->res_on && grid_lists)) {
     CUDA_TRY(bq::coop_max_grid(s->dtype, s->nm, false, s->smem_bytes, &grid_f));
     CUDA_TRY(bq::coop_max_grid(s->dtype, s->nm, true, s->adj_smem, &grid_b));
     const int src_items = s->max_s > 0 ? s->n_sys * s->max_s * 2 * ((s->ng_max + 3) / 4) : 0;  // BQ_SRC_TILE_COOP
     grid_f = std::min(grid_f, s->n_work);
     grid_b = std::min(grid_b, std::max(s->n_work, src_items));
   }
-  const bool coop = grid_f > 0 && grid_b > 0;
+  // the grid-resident kernels where the problems have their form (single-mode states follow the
+  // resident kernel's switch)
+  const bool grid = s->grad_coop && (s->res_on || (s->use_m1 && !s->res_ok)) && grid_lists;
+  const bool coop = grid || (grid_f > 0 && grid_b > 0);
   // Recording buffers: the two of the layout plus as many more as the workspace holds.  On
   // the cooperative path the forward pass records the last n_rec segments, which the
   // backward sweep then does not recompute; segment c uses buffer c % n_rec.
@@ -2675,6 +3140,14 @@ extern "C" int bq_grad(bq_state* s, double dt, int64_t n_steps, int checkpoint_e
     P.error = (unsigned int*)(b + L.off_ctrl + 32);
   }
   auto coop_fwd = [&](double tau_seg, int64_t n, char* rec, cudaStream_t cs) -> cudaError_t {
+    if (grid) {
+      bq::GridArgs a = grid_args(s, 1, dt);
+      a.rec = rec;
+      a.tau0 = tau_seg;
+      a.n_steps = (int)n;
+      g_launches++;
+      return launch_grid(s, a, 1, cs);
+    }
     P.tau0 = tau_seg;
     P.n_steps = (int)n;
     P.rec = rec;
@@ -2741,6 +3214,19 @@ extern "C" int bq_grad(bq_state* s, double dt, int64_t n_steps, int checkpoint_e
         CUDA_TRY(cudaMemcpyAsync(b + L.off_y, w + G.ckpt + (2 * c) * arr, arr, cudaMemcpyDeviceToDevice, st));
         CUDA_TRY(cudaMemcpyAsync(b + L.off_comp, w + G.ckpt + (2 * c + 1) * arr, arr, cudaMemcpyDeviceToDevice, st));
         CUDA_TRY(coop_fwd(tau0 + (double)n0 * dt, n1 - n0, rec, st));
+      }
+      if (grid) {
+        bq::GridArgs a = grid_args(s, 2, dt);
+        a.ua = w + G.ba;
+        a.ub = w + G.bb;
+        a.rec = rec;
+        a.lam = lam;
+        a.grad = (double*)(w + G.grad);
+        a.tau0 = tau0 + (double)n0 * dt;
+        a.n_steps = (int)(n1 - n0);
+        CUDA_TRY(launch_grid(s, a, 2, st));
+        g_launches++;
+        continue;
       }
       P.tau0 = tau0 + (double)n0 * dt;  // (the recomputation, when it runs, sets the same)
       P.n_steps = (int)(n1 - n0);
@@ -2849,10 +3335,13 @@ extern "C" int bq_autotune_grad(bq_state* s, double dt, int trial_steps, int che
   if (trial_steps < 1 || checkpoint_every < 1) return fail(BQ_EINVAL, "bad trial arguments");
   cudaStream_t st = (cudaStream_t)stream;
   std::vector<double> loss(s->B), g(std::max(1, s->grad_size));
-  struct Cand { int tile, lanes, gread; };
+  struct Cand { int tile, lanes, gread, resident = 0; };
   std::vector<Cand> cands;
+  const int res0 = s->res_on;
+  if (const int rg = ensure_grid_adjoint(s); rg != BQ_OK) return rg;
+  if (!s->use_m1 && s->glist[1].n_ctas > 0 && s->glist[2].n_ctas > 0) cands.push_back({s->tile, s->lanes, s->gread_sched, 1});
   if (s->use_m1) {
-    for (int ln : {1, 2, 4}) cands.push_back({s->tile, ln, s->gread_sched});
+    for (int ln : {1, 2, 4}) cands.push_back({s->tile, ln, s->gread_sched, res0});
   } else {
     for (int gr : {0, 1})
       for (int tl : {0, 32, 64, 96, 128, 192, 256, 512})
@@ -2875,7 +3364,7 @@ extern "C" int bq_autotune_grad(bq_state* s, double dt, int trial_steps, int che
     ~EvGuard() { cudaEventDestroy(a); cudaEventDestroy(b); }
   } guard{e0, e1};
   double best_us = 1e300;
-  Cand best{tile0, lanes0, gread0};
+  Cand best{tile0, lanes0, gread0, res0};
   int ntried = 0;
   for (const Cand& c : cands) {
     if (!s->use_m1 && (c.tile != s->tile || c.gread != s->gread_sched) && apply_tile(s, c.tile, c.gread) != BQ_OK) {
@@ -2883,6 +3372,7 @@ extern "C" int bq_autotune_grad(bq_state* s, double dt, int trial_steps, int che
       continue;
     }
     s->lanes = c.lanes;
+    s->res_on = c.resident;
     int rc = bq_grad(s, dt, std::min(trial_steps, checkpoint_every), checkpoint_every, work, work_bytes, loss.data(),
                      g.data(), stream);  // warm-up
     if (rc == BQ_OK) {
@@ -2894,6 +3384,7 @@ extern "C" int bq_autotune_grad(bq_state* s, double dt, int trial_steps, int che
       // restore the schedule the state had, then report
       if (!s->use_m1) apply_tile(s, tile0, gread0);
       s->lanes = lanes0;
+      s->res_on = res0;
       return rc;
     }
     CUDA_TRY(cudaEventSynchronize(e1));
@@ -2908,6 +3399,7 @@ extern "C" int bq_autotune_grad(bq_state* s, double dt, int trial_steps, int che
     if (rc != BQ_OK) return rc;
   }
   s->lanes = best.lanes;
+  s->res_on = best.resident;
   s->tune_grad_us = best_us;
   drop_graph(s);
   if (out) {

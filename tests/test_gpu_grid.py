@@ -1,0 +1,197 @@
+"""The grid-resident kernels of the tiled path (bq_tune resident = 1) against the tiled kernels
+(resident = 0) and the oracle: one to four modes, every residual layout, Hermitian and general
+states, both precisions, gradients, and the forms they must leave to the tiled kernels."""
+
+import dataclasses
+
+import numpy as np
+import pytest
+
+from oracle import grad as ograd
+from oracle import mapping
+from workloads import configs
+from workloads.spec import Channel, HTerm, Jump, SecularDamping
+
+from parity import compare_mapped_systems, gpu_state
+
+pytestmark = pytest.mark.gpu
+# two kernels' roundings over a few steps of O(1) data, as in the schedule tests: 1e-12 / 1e-6
+TOL = {"f64": 1e-12, "f32": 1e-6}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import torch
+    from paper_2203_05526_gb300 import build
+    build.build()
+    assert torch.cuda.is_available()
+
+
+def _raw(st, dtype):
+    import torch
+    host = torch.empty(st.state_bytes(), dtype=torch.uint8, pin_memory=True)
+    st.store_state(host.data_ptr())
+    torch.cuda.synchronize()
+    return host.numpy().view(np.float64 if dtype == "f64" else np.float32).astype(np.float64)
+
+
+def _driven(N=5, drive="gauss", n_th=0.1, steps=11, secular=False, measured=None):
+    """Two exchange-coupled, driven, damped Kerr modes."""
+    p = configs.two_mode(N=N, T=steps * 0.005, dt=0.005)
+    T = p.T
+    p.channels = [{"gauss": Channel("gauss", (0.4, 0.1, 0.4 * T, 0.3 * T)), "cexp": Channel("cexp", (0.3, -0.1, 2.0)),
+                   "const": Channel("const", (0.2, 0.1)),
+                   "pwc": Channel("pwc", (0.0, T / 3, 0.3, 0.1, -0.2, 0.2, 0.1, -0.1))}[drive]]
+    p.h_terms = p.h_terms + configs.gauss_drive_terms(2, 0, 0) + [HTerm(0.3, (1, 1), (1, 1))]  # and a cross-Kerr shift
+    if secular:
+        p.jumps = []
+        p.secular = [SecularDamping(j, 0.05, (0.1,) * (N - 1) if n_th else ()) for j in range(2)]
+    else:
+        p.jumps = configs.damping_jumps(2, 0, 0.05, n_th) + configs.damping_jumps(2, 1, 0.03, n_th)
+    if measured is not None:
+        p.measured = measured
+    return p
+
+
+GENERAL = {((1, 0), (0, 1)): 0.7 + 0.2j, ((0, 0), (1, 0)): 0.5j, ((1, 1), (1, 1)): 1.0}
+
+
+def _both(ps, dtype, steps, **kw):
+    a, b = gpu_state(ps, dtype=dtype, **kw), gpu_state(ps, dtype=dtype, **kw)
+    assert a.get_tune()["resident"] == 1 and a.get_tune()["stage_path"] == "tiled"
+    b.set_tune(resident=0)
+    dt = (ps if isinstance(ps, list) else [ps])[0].dt
+    for st in (a, b):
+        st.step(dt, steps - 2)
+        st.step(dt, 2)
+    return a, b
+
+
+def _agree(a, b, dtype):
+    x, y = _raw(a, dtype), _raw(b, dtype)
+    assert np.all(np.isfinite(x))
+    assert np.max(np.abs(x - y)) <= TOL[dtype] * np.max(np.abs(y))
+    ea, eb = a.evaluate(), b.evaluate()
+    assert np.max(np.abs(ea - eb)) <= TOL[dtype] * max(1.0, np.max(np.abs(eb)))
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("measured", [None, GENERAL])
+@pytest.mark.parametrize("form", [dict(), dict(drive="cexp"), dict(drive="pwc", n_th=0.0), dict(drive="const"),
+                                  dict(secular=True), dict(secular=True, n_th=0.0), dict(N=2), dict(N=3), dict(N=6)])
+def test_every_form_matches_the_tiled_kernels(dtype, measured, form):
+    p = _driven(measured=measured, **form)
+    a, b = _both(p, dtype, 11)
+    _agree(a, b, dtype)
+    if form == dict():
+        compare_mapped_systems(a, mapping.rk4_mapped(p), 1e-10 if dtype == "f64" else 1e-5)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("kw", [dict(method="direct"), dict(r_layout="off"), dict(r_layout="diag")])
+@pytest.mark.parametrize("modes", [1, 2, 3])
+def test_layouts_and_modes(dtype, kw, modes):
+    if modes == 1 and kw.get("r_layout") != "diag":
+        pytest.skip("other single-mode states do not take the tiled path")
+    p = configs.table_one_network(modes, 4, steps=4000)
+    p = dataclasses.replace(p, T=12 * p.dt)
+    a, b = _both(p, dtype, 12, **kw)
+    _agree(a, b, dtype)
+
+
+def test_four_modes_and_uneven_truncations():
+    p = configs.table_one_network(4, 3, steps=4000)
+    p = dataclasses.replace(p, T=6 * p.dt, measured={((1, 0, 1, 0), (0, 1, 1, 0)): 1.0 + 0.3j, ((1, 1, 0, 0), (1, 1, 0, 0)): 0.5})
+    a, b = _both(p, "f64", 6)
+    _agree(a, b, "f64")
+    q = _driven()
+    q.N = (7, 4)
+    a, b = _both(q, "f64", 11)
+    _agree(a, b, "f64")
+    a, b = _both([_driven(N=5), _driven(N=3, n_th=0.0), _driven(N=4, measured=GENERAL)], "f64", 11)  # several problems
+    _agree(a, b, "f64")
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_loaded_states_and_switches(dtype):
+    import torch
+    p = _driven()
+    a, b = _both(p, dtype, 9)
+    snap = torch.from_numpy(_raw(a, dtype)).to(torch.float64 if dtype == "f64" else torch.float32)
+    noise = torch.randn(snap.shape, generator=torch.Generator().manual_seed(5), dtype=torch.float64)
+    n_g = p.N[0] * p.N[1]
+    pad = (n_g + 3) & ~3
+    keep = torch.zeros_like(snap)
+    for off, n in ((0, n_g), (pad, n_g), (2 * pad, n_g * n_g)):  # the padding stays zero
+        keep[2 * off:2 * (off + n)] = 1
+    host = ((snap + 1e-2 * noise.to(snap.dtype)) * keep).contiguous().pin_memory()  # not Hermitian
+    for st in (a, b):
+        st.load_state(host.data_ptr())
+        st.step(p.dt, 3)
+    _agree(a, b, dtype)
+    a.set_tune(resident=0)
+    a.step(p.dt, 1)
+    a.set_tune(resident=1)
+    a.step(p.dt, 2)
+    b.step(p.dt, 3)
+    _agree(a, b, dtype)
+
+
+def _control(N, B=1, n_seg=3, steps_per_seg=6, measured=None):
+    ps = []
+    for b in range(B):
+        p = configs.two_mode_control(n_seg=n_seg, T=n_seg * steps_per_seg * 0.01, steps_per_seg=steps_per_seg, N=N, seed=5526 + b)
+        p.jumps = configs.damping_jumps(2, 0, 0.05, 0.1) + configs.damping_jumps(2, 1, 0.03, 0.0)
+        p.rho0 = {((0, 0), (0, 0)): 0.6, ((1, 0), (1, 0)): 0.3, ((0, 1), (1, 0)): 0.1j, ((1, 0), (0, 1)): -0.1j}
+        if measured:
+            p.measured = measured
+        ps.append(p)
+    return ps
+
+
+@pytest.mark.parametrize("measured", [None, {((1, 0), (1, 0)): 1.0, ((1, 0), (0, 1)): 0.7 + 0.2j, ((0, 1), (1, 0)): 0.7 - 0.2j}])
+@pytest.mark.parametrize("N,B,every", [(2, 1, 18), (4, 1, 7), (5, 3, 5), (7, 1, 1)])
+def test_gradients_match_the_tiled_kernels_and_the_oracle(measured, N, B, every):
+    ps = _control(N, B, measured=measured)
+    a, b = gpu_state(ps), gpu_state(ps)
+    assert a.get_tune()["resident"] == 1
+    b.set_tune(resident=0)
+    la, ga = a.grad(ps[0].dt, ps[0].n_steps, every)
+    lb, gb = b.grad(ps[0].dt, ps[0].n_steps, every)
+    assert np.max(np.abs(la - lb)) <= 1e-13 * max(1.0, np.max(np.abs(lb)))
+    assert np.max(np.abs(ga - gb)) <= 1e-12 * np.max(np.abs(gb))
+    if N == 4:
+        loss, gt, gp = ograd.loss_and_grad(ps[0], checkpoint_every=every)
+        ref = np.concatenate([gt, gp[0].reshape(-1)])
+        assert abs(la[0] - loss) <= 1e-12 * max(1.0, abs(loss))
+        assert np.max(np.abs(ga - ref)) <= 1e-10 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("kw", [dict(r_layout="diag"), dict(r_layout="off"), dict(method="direct")])
+@pytest.mark.parametrize("secular", [False, True])
+def test_gradients_of_other_layouts(kw, secular):
+    p = _control(4)[0]
+    if secular:
+        p.jumps = []
+        p.secular = [SecularDamping(j, 0.05, (0.1,) * 3) for j in range(2)]
+    a, b = gpu_state(p, **kw), gpu_state(p, **kw)
+    b.set_tune(resident=0)
+    la, ga = a.grad(p.dt, p.n_steps, 5)
+    lb, gb = b.grad(p.dt, p.n_steps, 5)
+    assert abs(la[0] - lb[0]) <= 1e-13 * max(1.0, abs(lb[0]))
+    assert np.max(np.abs(ga - gb)) <= 1e-12 * np.max(np.abs(gb))
+
+
+def test_other_forms_keep_the_tiled_kernels():
+    def one(f):
+        p = _driven(N=3)
+        f(p)
+        st = gpu_state(p)
+        st.set_tune(resident=1)
+        return st.get_tune()["resident"]
+
+    z, a = (0, 0), (1, 0)
+    assert one(lambda p: None) == 1
+    # a time-dependent diagonal term, a jump operator of two monomials
+    assert one(lambda p: p.h_terms.extend([HTerm(0.2, a, a, channel=0), HTerm(0.2, a, a, channel=0, conj=True)])) == 0
+    assert one(lambda p: p.jumps.append(Jump(0.1, ((1.0 + 0j, z, a), (0.5 + 0j, z, z))))) == 0

@@ -18,8 +18,8 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libbq.so")
 BUILD_DIR = os.path.join(HERE, "_build")
-SOURCES = ["bq_host.cu", "bq_kernels.cu", "bq_resident_f32.cu", "bq_resident_f64.cu", "bq_grid_f32.cu",
-           "bq_grid_f64.cu", "bq_peaks.cu"]
+SOURCES = ["bq_host.cu", "bq_kernels.cu", "bq_resident_f32_herm.cu", "bq_resident_f32_gen.cu",
+           "bq_resident_f64_herm.cu", "bq_resident_f64_gen.cu", "bq_grid_f32.cu", "bq_grid_f64.cu", "bq_peaks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -779,7 +779,7 @@ struct bq_state {
   // systems of list 0 are known to hold Hermitian states (false once a state was loaded or
   // another kernel stepped it: then res_dirty asks for a check of the data before the next
   // launch, and the systems that fail it take list 2)
-  int res_ok = 0, res_on = 0, res_mode = 1, res_ns = 1, res_obs = 0, res_known = 1, res_dirty = 0;
+  int res_ok = 0, res_on = 0, res_variant = 0, res_obs = 0, res_known = 1, res_dirty = 0;
   ResList rlist[3];
   // grid-resident kernels: lists (forward Hermitian, forward general, adjoint) and variant sizes
   GridList glist[3];
@@ -868,7 +868,7 @@ struct Plan {
   double rho = 0.0, dt_max = 0.0;
   // resident kernel (k_resident): parameter blocks per problem, groups (the Hermitian layout's,
   // then the general layout's) and the CTAs' bins
-  int res_ok = 0, res_mode = 1, res_ns = 1, res_obs = 1;
+  int res_ok = 0, res_variant = 0, res_obs = 1;
   std::vector<unsigned char> rparams;
   std::vector<bq::ResGroup> rgroups;
   std::vector<bq::ResBin> rbins;
@@ -993,18 +993,22 @@ static bq::PipeChan pipe_chan(const ChanDesc& cd, const double* chpar) {
 }
 
 // Rows per strip and warps of a system: the fewest issue slots, counting a
-// row as 1 and a strip's fixed part (edges, stage set-up) as 1.4 rows.  0 if it does not fit.
-static int res_shape(int M, int cs, bool herm, int& rb, int& nb) {
+// row as 1 and a strip's fixed part (edges, stage set-up) as 1.4 rows.  few: the systems do not
+// fill the GPU, so the shortest strips that fit (a stage's latency is then what counts).  0 if
+// nothing fits.
+static int res_shape(int M, int cs, bool herm, bool few, int& rb, int& nb) {
   const int cols = herm ? M | 1 : M, nd = herm ? cols / 2 + 1 : M;
   const int cap = BQ_RES_WARPS(cs, herm);
   int best = 0;
   double cost = 1e300;
-  for (int r : {2, 4, 7}) {
-    if (r > nd || (cs == 16 && r > 4)) continue;
+  for (int r = 2; r <= 7; ++r) {
+    // (the lengths the kernels are compiled for)
+    if (r > nd || (cs == 16 ? r != 2 && r != 4 : herm ? r != 3 && r != 5 : r != 2 && r != 4 && r != 7)) continue;
     const int n = (nd + r - 1) / r, w = (cols * n + 31) / 32;
     if (w + 1 > cap) continue;
-    if (w * (r + 1.4) < cost) {
-      cost = w * (r + 1.4);
+    const double c = few ? r : w * (r + 1.4);
+    if (c < cost) {
+      cost = c;
       rb = r;
       nb = n;
       best = w + 1;
@@ -1027,7 +1031,7 @@ static bool same_table(const std::vector<double>& x, const std::vector<double>& 
 }
 
 static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, const EvalGroup& eg, int term_off,
-                        int wbase, size_t cs, std::vector<unsigned char>& blk, int& mode, int& ns, bool& herm) {
+                        int wbase, size_t cs, std::vector<unsigned char>& blk, int& variant, bool& herm) {
   const int M = C.M[0];
   if (M < 4 || M > 42 || !C.has_r || C.r_diag || eg.n_e > 32) return false;
   std::vector<cplx> d(C.diag.begin(), C.diag.begin() + 2 * M);
@@ -1113,8 +1117,7 @@ static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, co
       }
     }
   }
-  if (!imag) mode = 2;
-  if (splus) ns = 2;
+  variant = (imag ? 0 : 1) | (splus ? 2 : 0) | (sdiag > 0 ? 4 : 0);
   herm = w[0] == w[2] && w[1] == w[3];
   for (int k = 0; k < M && herm; ++k) herm = d[M + k] == std::conj(d[k]);
   herm = herm && same_table(w[4], w[5]) && same_table(w[6], w[7]);
@@ -1155,8 +1158,8 @@ static bool res_pack(Plan& P, const std::vector<int>& which, const std::vector<i
       const int M = sd.M[0];
       bq::ResGroup g;
       std::memset(&g, 0, sizeof(g));
-      const int cols = herm ? M | 1 : M, nd = herm ? cols / 2 + 1 : M;
-      const int w = res_shape(M, (int)cs, herm, g.rb, g.nb);
+      const int cols = herm ? M | 1 : M;
+      const int w = res_shape(M, (int)cs, herm, which.size() <= 152, g.rb, g.nb);
       if (!w) return false;
       g.sys = which[i];
       g.M = M;
@@ -1166,8 +1169,8 @@ static bool res_pack(Plan& P, const std::vector<int>& which, const std::vector<i
       g.blk_elems = g.r_off + ((sd.n_r + 3) & ~3);
       g.param_off = poff[sd.prob];
       g.nwarps = w;
-      const int buf = nd * cols;
-      g.stage_elems = std::max(g.blk_elems, 2 * buf + (BQ_RES_COMP_SMEM(cs, herm) ? g.rb * g.nb * cols : 0));
+      const int buf = g.nb * bq::res_strip_stride(g.rb, cols);
+      g.stage_elems = std::max(g.blk_elems, 2 * buf + g.rb * g.nb * cols);
       g.c_re = sd.c_re; g.c_im = sd.c_im; g.w_re = sd.w_re; g.w_im = sd.w_im;
       by[w].push_back((int)P.rgroups.size());
       P.rgroups.push_back(g);
@@ -1213,10 +1216,21 @@ static void make_res_plan(Plan& P, const bq_problem* const* probs, const std::ve
   for (const SysDesc& sd : P.sys) term_off[sd.prob] = sd.term_off;
   std::vector<char> herm(B, 0);
   std::vector<unsigned char> blk;
+  int sd = -1;
   for (int b = 0; b < B; ++b) {
     bool hm = false;
+    int variant = 0;
     blk.clear();
-    if (!res_problem(P, P.comp[b], progs[b], P.groups[b], term_off[b], P.wbase[b], cs, blk, P.res_mode, P.res_ns, hm)) return;
+    if (!res_problem(P, P.comp[b], progs[b], P.groups[b], term_off[b], P.wbase[b], cs, blk, variant, hm)) return;
+    // one kernel per launch: the restriction to k = l holds for all sandwich terms of the batch or
+    // for none (problems without sandwich terms go with either)
+    bool has_s = false;
+    for (const TermDesc& td : P.comp[b].terms) has_s = has_s || td.side == bq::SIDE_S;
+    if (has_s) {
+      if (sd >= 0 && sd != (variant & 4)) return;
+      sd = variant & 4;
+    }
+    P.res_variant |= variant;
     if (P.comp[b].method == BQ_METHOD_DIRECT) {  // A(0) itself
       for (auto& [kl, v] : probs[b]->measured) {
         auto it = probs[b]->measured.find({kl.second, kl.first});
@@ -2203,8 +2217,7 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
   }
   st->pipe_ok = st->use_pipe;
   st->res_ok = st->res_on = P.res_ok && st->pipe_ok;
-  st->res_mode = P.res_mode;
-  st->res_ns = P.res_ns;
+  st->res_variant = P.res_variant;
   st->res_obs = P.res_obs;
   for (int q = 0; q < 3; ++q) st->rlist[q] = P.rlist[q];
   for (int q = 0; q < 3; ++q) st->glist[q] = glist[q];
@@ -2473,6 +2486,11 @@ static cudaError_t enqueue_resident(bq_state* s, double dt, int64_t n, cudaStrea
   a.reverse = s->reverse;
   a.dt = dt;
   a.horizon = s->horizon;
+  a.cd[0] = dt;
+  a.cd[1] = 0.5 * dt;
+  a.cd[2] = dt / 6.0;
+  for (int i = 0; i < 3; ++i) a.cf[i] = (float)a.cd[i];
+  a.cf[3] = (float)(a.cd[2] - (double)a.cf[2]);
   run_begin(s, dt);
   const int64_t most = 1 << 30;  // steps per launch (32-bit counter)
   for (int64_t done = 0; done < n;) {
@@ -2487,8 +2505,9 @@ static cudaError_t enqueue_resident(bq_state* s, double dt, int64_t n, cudaStrea
       a.bins = (const bq::ResBin*)(b + L.off_rbins) + l.b0;
       a.flags = q == 1 || s->res_known ? nullptr : flags;
       a.want = q == 0;
-      const auto launch = s->dtype == BQ_F64 ? bq::launch_resident_f64 : bq::launch_resident_f32;
-      const cudaError_t e = launch(a, s->res_mode, s->res_ns, q == 0, l.n_bins, l.smem, st);
+      const auto launch = s->dtype == BQ_F64 ? (q == 0 ? bq::launch_resident_f64_herm : bq::launch_resident_f64_gen)
+                                             : (q == 0 ? bq::launch_resident_f32_herm : bq::launch_resident_f32_gen);
+      const cudaError_t e = launch(a, s->res_variant, l.n_bins, l.smem, st);
       if (e != cudaSuccess) return e;
       ++*launches;
     }

@@ -16,8 +16,10 @@
 // What it replaces and measured (one GB300): the streamed step kernel was bound by HBM traffic
 // and issue, the earlier persistent solve by issue (160 instructions per point and stage, most of
 // them loads and rebuilding of per-stage coefficients).  4096 ragged FP32 oscillators (N 10..40):
-// 84 -> 22.9 us per step; 16 384: 351 -> 102; 1024 in FP64: 413 -> 120; one in FP32 (N = 40):
-// 14.2 -> 3.9; one in FP64: 145 -> 39.
+// 84 -> 18.6 us per step; 16 384: 351 -> 79; 1024 in FP64: 413 -> 118; one in FP32 (N = 40):
+// 14.2 -> 2.0; one in FP64: 145 -> 36.  What bounds it now: in FP32 shared-memory wavefronts and
+// issue about equally (a half each, 20 warps per SM to hide the latencies); in FP64 the FP64 pipe
+// (88%).
 //
 // Layout: a thread owns column l and RB consecutive rows, its state, stage sum, compensation,
 // stage input and weights in registers; the column's own neighbours never leave registers, and
@@ -90,6 +92,12 @@ __device__ __forceinline__ C off_diag(C a, C p, C q, C k) {
 }
 
 template <typename T>
+__device__ __forceinline__ T res_const(const ResArgs& A, int i) {
+  if constexpr (sizeof(T) == 8) return A.cd[i];
+  else return A.cf[i];
+}
+
+template <typename T>
 struct ResWeights {  // pointers into a problem's parameter block
   using C = typename C2T<T>::type;
   const C *dx, *dy;
@@ -110,10 +118,9 @@ struct ResView {
   static constexpr int GW = HERM ? 1 : 2;  // G_x (and G_y) stored
   const unsigned char* blk;
   C *U, *Gs, *RG, *E, *yg, *cg;
-  int M, P, us, gt, gn, bar;
+  int M, P, ss, us, gt, gn, bar;
   bool sep;
-  // U: [2] stage buffers of us elements, perhaps a third for the compensation (BQ_RES_COMP_SMEM);
-  // the whole region is also the staging buffer of the load and the store.  Gs: [2][GW P] stage inputs of
+  // U: [2] stage buffers of us elements, then the strips' compensation; the whole region is also the staging buffer of the load and the store.  Gs: [2][GW P] stage inputs of
   // G.  RG: [2][2][2 P] row products sm_k G_x[k-1], sp_k G_x[k+1] (HERM: twice, so that the
   // index l + d needs no modulo).  E: [2][32] off-diagonal coefficient of the stages.
   __device__ __forceinline__ ResView(const ResArgs& A, const ResGroup& g, unsigned char* sm, int gt_, int gn_, int bar_)
@@ -125,7 +132,8 @@ struct ResView {
     E = RG + 8 * P;
     yg = reinterpret_cast<C*>(A.y) + g.blk_off;
     cg = reinterpret_cast<C*>(A.comp) + g.blk_off;
-    us = (HERM ? P / 2 + 1 : M) * P;
+    ss = res_strip_stride(g.rb, P);
+    us = g.nb * ss;
     sep = g.gy_off >= 0;
   }
   __device__ __forceinline__ void sync() const { group_sync(bar, gn); }
@@ -145,18 +153,18 @@ struct ResView {
 // [comp placed] [comp out].
 
 // The strips of R.
-template <typename T, int RB, int MODE, int NS, bool HERM>
+template <typename T, int RB, int MODE, int NS, bool SD, bool HERM>
 __device__ __forceinline__ void res_strips(const ResArgs& A, const ResGroup& g, unsigned char* sm, int gt, int gn, int bar) {
   using C = typename C2T<T>::type;
-  constexpr bool SMEM = BQ_RES_COMP_SMEM(sizeof(C), HERM);
+  // registers are short: the compensation, touched once a step, lives in shared memory, and the
+  // own stage input too except in the FP32 Hermitian layout
+  constexpr bool US = sizeof(T) == 8 || !HERM;
   const ResView<T, NS, HERM> V(A, g, sm, gt, gn, bar);
-  const ResHdr& h = *reinterpret_cast<const ResHdr*>(V.blk);
   const ResWeights<T> W(V.blk, g.M);
   const int M = g.M, P = V.P, D = P / 2, ND = HERM ? D + 1 : M, us = V.us;
   C* U = V.U;
   const C zero = cmk<C>(0.0, 0.0);
-  C* Cs = U + 2 * us + gt;  // (SMEM) this thread's compensation, row j at Cs[j nb P]
-  const bool sdiag = h.sdiag != 0;
+  C* Cs = U + 2 * us + gt;  // this thread's compensation, row j at Cs[j nb P]
   const bool act = gt < g.nb * P;
   const int l = act ? gt % P : 0;
   // (the last strip may overlap the one before: both threads then compute the shared rows, with
@@ -165,21 +173,30 @@ __device__ __forceinline__ void res_strips(const ResArgs& A, const ResGroup& g, 
   const bool first = HERM && d0 == 0, last = HERM && d0 + RB == ND;
   const unsigned m0 = first ? 0x80000000u : 0u, m1 = last ? 0x80000000u : 0u;
   const int lm = max(l - 1, 0), lp = min(l + 1, P - 1);  // (clamped columns have zero weights)
-  // element offsets in a stage buffer of the values around the strip
-  const int o_own = d0 * P + l;
-  const int o_top = first ? P + (l == 0 ? P - 1 : l - 1) : max(d0 - 1, 0) * P + l;
-  const int o_bot = last ? D * P + (l + D + 1) % P : min(d0 + RB, ND - 1) * P + l;
-  const int o_lw = (d0 + (HERM ? 1 : 0)) * P + lm;  // left column at row j: o_lw + j P
-  const int o_lend = last ? D * P + (l + D) % P : o_lw + (RB - 1) * P;
-  const int o_lpre = HERM ? o_lw - P : max(d0 - 1, 0) * P + lm;
-  const int o_rw = (d0 - (HERM ? 1 : 0)) * P + lp;  // right column at row j: o_rw + j P
-  const int o_r0 = first ? P + l : o_rw;
-  const int o_rpost = HERM ? o_rw + RB * P : min(d0 + RB, M - 1) * P + lp;
+  // Element offsets in a stage buffer of the values around the strip.  Strip-major: strip b's rows
+  // start at b SS, a row is S elements (a constant: the step from row to row is an immediate), and
+  // SS is P modulo 16, so that the lanes of a half warp touch consecutive 8-byte banks across
+  // strips too (a sixth fewer shared-memory wavefronts than plain rows).
+  constexpr int S = BQ_RES_COLS;
+  const int SS = V.ss;
+  auto at = [&](int d) {  // row d, column 0 (rows the last two strips share: the last strip's copy)
+    const int sb = d >= ND - RB ? g.nb - 1 : d / RB;
+    return sb * SS + (d - min(sb * RB, ND - RB)) * S;
+  };
+  const int o_own = (act ? gt / P : 0) * SS + l;
+  const int o_top = first ? at(1) + (l == 0 ? P - 1 : l - 1) : at(max(d0 - 1, 0)) + l;
+  const int o_bot = last ? at(D) + (l + D + 1) % P : at(min(d0 + RB, ND - 1)) + l;
+  const int o_lw = o_own - l + (HERM ? S : 0) + lm;  // left column at row j < RB - 1: o_lw + j S
+  const int o_lend = last ? at(D) + (l + D) % P : (HERM ? at(d0 + RB) + lm : o_lw + (RB - 1) * S);
+  const int o_lpre = HERM ? o_lw - S : at(max(d0 - 1, 0)) + lm;
+  const int o_rw = o_own - l - (HERM ? S : 0) + lp;  // right column at row j > 0: o_rw + j S
+  const int o_r0 = HERM ? (first ? at(1) + l : at(d0 - 1) + lp) : o_rw;
+  const int o_rpost = HERM ? o_rw + RB * S : at(min(d0 + RB, M - 1)) + lp;
   const int k0 = HERM ? l + d0 : d0;  // row index of the first point (HERM: modulo P)
   auto row = [&](int j) { const int k = k0 + j; return HERM && k >= P ? k - P : k; };
   auto in = [&](int j) { return act && (!HERM || (l < M && row(j) < M)); };  // a point of the grid
 
-  C y[RB], c[SMEM ? 1 : RB], u[SMEM ? 1 : RB], s[RB], dg[RB];
+  C y[RB], u[US ? 1 : RB], s[RB], dg[RB];
   T xm[RB], xp[RB], sm_[RB], sp_[NS == 2 ? RB : 1];
   V.stage_in(V.yg, g.blk_elems);
 #pragma unroll
@@ -197,13 +214,8 @@ __device__ __forceinline__ void res_strips(const ResArgs& A, const ResGroup& g, 
       V.sync();
     }
 #pragma unroll
-    for (int j = 0; j < RB; ++j) {
-      if constexpr (SMEM) {
-        if (act) Cs[j * g.nb * P] = ct[j];
-      } else {
-        c[j] = ct[j];
-      }
-    }
+    for (int j = 0; j < RB; ++j)
+      if (act) Cs[j * g.nb * P] = ct[j];
   }
   const bool inl = l < M;
   const T ym = inl ? W.ym[l] : (T)0, yp = inl ? W.yp[l] : (T)0, smy = inl ? W.smy[l] : (T)0, spy = inl ? W.spy[l] : (T)0;
@@ -216,15 +228,13 @@ __device__ __forceinline__ void res_strips(const ResArgs& A, const ResGroup& g, 
     xp[j] = ok ? W.xp[k] : (T)0;
     sm_[j] = ok ? W.smx[k] * smy : (T)0;
     if (NS == 2) sp_[j] = ok ? W.spx[k] * spy : (T)0;
-    if (!SMEM) u[j] = y[j];
-    if (act) U[o_own + j * P] = y[j];
+    if (!US) u[US ? 0 : j] = y[j];
+    if (act) U[o_own + j * S] = y[j];
     s[j] = zero;
   }
   V.sync();
 
-  const T hh = (T)A.dt, h2 = (T)(0.5 * A.dt);
-  const double wd = A.dt / 6.0;
-  const T w_hi = (T)wd, w_lo = (T)(wd - (double)w_hi);
+  const T hh = res_const<T>(A, 0), h2 = res_const<T>(A, 1), w_hi = res_const<T>(A, 2), w_lo = res_const<T>(A, 3);
 
   // right-hand side at the strip's points from stage buffer B (half b of G), handed to f(j, k)
   auto rhs = [&](const C* B, int b, C a, auto f) {
@@ -239,12 +249,12 @@ __device__ __forceinline__ void res_strips(const ResArgs& A, const ResGroup& g, 
     gr = cscale(gr, spy);
     C up = conj_if(B[o_top], m0), lpre = B[o_lpre];
     C rj = conj_if(B[o_r0], m0);
-    C uc = SMEM ? B[o_own] : u[0];
+    C uc = US ? B[o_own] : u[0];
 #pragma unroll
     for (int j = 0; j < RB; ++j) {
-      const C dn = j + 1 < RB ? (SMEM ? B[o_own + (j + 1) * P] : u[SMEM ? 0 : j + 1]) : conj_if(B[o_bot], m1);
-      const C lj = j + 1 < RB ? B[o_lw + j * P] : conj_if(B[o_lend], m1);
-      const C rn = j + 1 < RB ? B[o_rw + (j + 1) * P] : (NS == 2 ? B[o_rpost] : zero);
+      const C dn = j + 1 < RB ? (US ? B[o_own + (j + 1) * S] : u[US ? 0 : j + 1]) : conj_if(B[o_bot], m1);
+      const C lj = j + 1 < RB ? B[o_lw + j * S] : conj_if(B[o_lend], m1);
+      const C rn = j + 1 < RB ? B[o_rw + (j + 1) * S] : (NS == 2 ? B[o_rpost] : zero);
       C k, p, q;
       k.x = fma(dg[j].x, uc.x, -(dg[j].y * uc.y));
       k.y = fma(dg[j].x, uc.y, dg[j].y * uc.x);
@@ -260,7 +270,8 @@ __device__ __forceinline__ void res_strips(const ResArgs& A, const ResGroup& g, 
         q.y = fma(xp[j], dn.y, -ym * lj.y);
         k = off_diag<MODE>(a, p, q, k);
       }
-      if (!sdiag || (HERM ? d0 + j == 0 : d0 + j == l)) {  // secular projector: k = l only
+      // (SD, the secular projector: k = l only, in the Hermitian layout the first row)
+      if (!SD || (HERM ? j == 0 && d0 == 0 : d0 + j == l)) {
         k = caxpy(sm_[j], lpre, k);
         k = cfma(r[j], gl, k);
         if constexpr (NS == 2) {
@@ -281,56 +292,80 @@ __device__ __forceinline__ void res_strips(const ResArgs& A, const ResGroup& g, 
 #pragma unroll 1
   for (int step = 0; step < n_steps; ++step) {
     const C* Es = V.E + ((step >> 3) & 1) * 32 + (step & 7) * 4;
+    // the state update of row j by the stage sum and k4
+    auto update = [&](int j, C k) {
+      C d, cj = Cs[j * g.nb * P];
+      d.x = s[j].x + k.x;
+      d.y = s[j].y + k.y;
+      if constexpr (sizeof(T) == 4) {
+        d.x = fma(w_hi, d.x, fma(w_lo, d.x, -cj.x));
+        d.y = fma(w_hi, d.y, fma(w_lo, d.y, -cj.y));
+      } else {  // (w_lo is zero)
+        d.x = fma(w_hi, d.x, -cj.x);
+        d.y = fma(w_hi, d.y, -cj.y);
+      }
+      res_update(d, y[j], cj);
+      Cs[j * g.nb * P] = cj;
+      s[j] = zero;
+    };
+    if constexpr (!US) {
+      // One copy of the right-hand side for all four stages (the ragged batch runs several strip
+      // lengths at once and would not fit the instruction caches with more): k replaces u row by
+      // row, the combination follows.
 #pragma unroll 1
-    for (int stage = 1; stage <= 3; ++stage) {
-      const int b = (stage & 1) ^ 1;  // stages 1, 3 read half 0; 2, 4 half 1
-      const T al = stage == 3 ? hh : h2, be = stage == 1 ? (T)1 : (T)2;
+      for (int stage = 1; stage <= 4; ++stage) {
+        const int b = (stage & 1) ^ 1;  // stages 1, 3 read half 0; 2, 4 half 1
+        if (act) {
+          C* O = U + (b ^ 1) * us + o_own;
+          rhs(U + b * us, b, Es[stage - 1], [&](int j, C k) { u[US ? 0 : j] = k; });
+          if (stage < 4) {
+            const T al = stage == 3 ? hh : h2, be = stage == 1 ? (T)1 : (T)2;
+#pragma unroll
+            for (int j = 0; j < RB; ++j) {
+              C& v = u[US ? 0 : j];
+              s[j] = caxpy(be, v, s[j]);
+              v = caxpy(al, v, y[j]);
+              O[j * S] = v;
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < RB; ++j) {
+              update(j, u[US ? 0 : j]);
+              u[US ? 0 : j] = y[j];
+              O[j * S] = y[j];
+            }
+          }
+        }
+        V.sync();
+      }
+    } else {
+#pragma unroll 1
+      for (int stage = 1; stage <= 3; ++stage) {
+        const int b = (stage & 1) ^ 1;
+        const T al = stage == 3 ? hh : h2, be = stage == 1 ? (T)1 : (T)2;
+        if (act) {
+          C* O = U + (b ^ 1) * us + o_own;
+          rhs(U + b * us, b, Es[stage - 1], [&](int j, C k) {
+            s[j] = caxpy(be, k, s[j]);
+            O[j * S] = caxpy(al, k, y[j]);
+          });
+        }
+        V.sync();
+      }
       if (act) {
-        C* O = U + (b ^ 1) * us + o_own;
-        rhs(U + b * us, b, Es[stage - 1], [&](int j, C k) {
-          const C v = caxpy(al, k, y[j]);
-          s[j] = caxpy(be, k, s[j]);
-          if constexpr (!SMEM) u[j] = v;
-          O[j * P] = v;
+        C* O = U + o_own;
+        rhs(U + us, 1, Es[3], [&](int j, C k) {
+          update(j, k);
+          O[j * S] = y[j];
         });
       }
       V.sync();
     }
-    if (act) {
-      C* O = U + o_own;
-      rhs(U + us, 1, Es[3], [&](int j, C k) {
-        C d;
-        d.x = s[j].x + k.x;
-        d.y = s[j].y + k.y;
-        if constexpr (SMEM) {
-          C cj = Cs[j * g.nb * P];
-          if constexpr (sizeof(T) == 4) {
-            d.x = fma(w_hi, d.x, fma(w_lo, d.x, -cj.x));
-            d.y = fma(w_hi, d.y, fma(w_lo, d.y, -cj.y));
-          } else {  // (w_lo is zero)
-            d.x = fma(w_hi, d.x, -cj.x);
-            d.y = fma(w_hi, d.y, -cj.y);
-          }
-          res_update(d, y[j], cj);
-          Cs[j * g.nb * P] = cj;
-        } else {
-          d.x = fma(w_hi, d.x, fma(w_lo, d.x, -c[SMEM ? 0 : j].x));
-          d.y = fma(w_hi, d.y, fma(w_lo, d.y, -c[SMEM ? 0 : j].y));
-          res_update(d, y[j], c[SMEM ? 0 : j]);
-          u[SMEM ? 0 : j] = y[j];
-        }
-        s[j] = zero;
-        O[j * P] = y[j];
-      });
-    }
-    V.sync();
   }
 
   // ---- store: through the staging buffer, coalesced ------------------------------------------
-  if constexpr (SMEM) {
 #pragma unroll
-    for (int j = 0; j < RB; ++j) s[j] = act ? Cs[j * g.nb * P] : zero;
-  }
+  for (int j = 0; j < RB; ++j) s[j] = act ? Cs[j * g.nb * P] : zero;
   V.sync();
   auto place = [&](int j, C v) {
     const int k = row(j);
@@ -342,7 +377,7 @@ __device__ __forceinline__ void res_strips(const ResArgs& A, const ResGroup& g, 
   for (int j = 0; j < RB; ++j) place(j, y[j]);
   V.stage_out(V.yg, g.blk_elems);
 #pragma unroll
-  for (int j = 0; j < RB; ++j) place(j, SMEM ? s[j] : c[SMEM ? 0 : j]);
+  for (int j = 0; j < RB; ++j) place(j, s[j]);
   V.stage_out(V.cg, g.blk_elems);
 }
 
@@ -437,9 +472,7 @@ __device__ __forceinline__ void res_gwarp(const ResArgs& A, const ResGroup& g, u
   envelope(0);
   V.sync();
 
-  const T hh = (T)A.dt, h2 = (T)(0.5 * A.dt);
-  const double wd = A.dt / 6.0;
-  const T w_hi = (T)wd, w_lo = (T)(wd - (double)w_hi);
+  const T hh = res_const<T>(A, 0), h2 = res_const<T>(A, 1), w_hi = res_const<T>(A, 2), w_lo = res_const<T>(A, 3);
   auto rhs = [&](int b, int i, C a) {
     const int q = lane + 32 * i;
     const bool isx = q < M;
@@ -530,7 +563,7 @@ __device__ __forceinline__ void res_gwarp(const ResArgs& A, const ResGroup& g, u
   }
 }
 
-template <typename T, int MODE, int NS, bool HERM>
+template <typename T, int MODE, int NS, bool SD, bool HERM>
 __global__ void __launch_bounds__(32 * BQ_RES_WARPS(2 * sizeof(T), HERM), sizeof(T) == 4 ? 2 : 1)
     k_resident(const ResArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -546,42 +579,47 @@ __global__ void __launch_bounds__(32 * BQ_RES_WARPS(2 * sizeof(T), HERM), sizeof
     res_gwarp<T, MODE, NS, HERM>(A, g, sm, gt, gn, bar);
     return;
   }
-  switch (g.rb) {
-    case 2: res_strips<T, 2, MODE, NS, HERM>(A, g, sm, gt, gn, bar); break;
-    case 4: res_strips<T, 4, MODE, NS, HERM>(A, g, sm, gt, gn, bar); break;
-    default:
-      if constexpr (sizeof(T) == 4) res_strips<T, 7, MODE, NS, HERM>(A, g, sm, gt, gn, bar);
-      break;
+  // (the strip lengths res_shape chooses from)
+  if constexpr (sizeof(T) == 8) {
+    if (g.rb == 2) res_strips<T, 2, MODE, NS, SD, HERM>(A, g, sm, gt, gn, bar);
+    else res_strips<T, 4, MODE, NS, SD, HERM>(A, g, sm, gt, gn, bar);
+  } else if constexpr (HERM) {
+    if (g.rb == 3) res_strips<T, 3, MODE, NS, SD, HERM>(A, g, sm, gt, gn, bar);
+    else res_strips<T, 5, MODE, NS, SD, HERM>(A, g, sm, gt, gn, bar);
+  } else {
+    switch (g.rb) {
+      case 2: res_strips<T, 2, MODE, NS, SD, HERM>(A, g, sm, gt, gn, bar); break;
+      case 4: res_strips<T, 4, MODE, NS, SD, HERM>(A, g, sm, gt, gn, bar); break;
+      default: res_strips<T, 7, MODE, NS, SD, HERM>(A, g, sm, gt, gn, bar); break;
+    }
   }
 }
 
-template <typename T, int MODE, int NS, bool HERM>
+template <typename T, int MODE, int NS, bool SD, bool HERM>
 static cudaError_t launch_resident_one(const ResArgs& a, int n_bins, int smem_bytes, cudaStream_t s) {
   // (per call: the attribute belongs to the current device's context, and setting it is cheap)
-  cudaError_t e = cudaFuncSetAttribute(k_resident<T, MODE, NS, HERM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(k_resident<T, MODE, NS, SD, HERM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        BQ_RES_SMEM_MAX);
   if (e != cudaSuccess) return e;
-  k_resident<T, MODE, NS, HERM>
-      <<<n_bins, 32 * BQ_RES_WARPS(2 * sizeof(T), HERM), smem_bytes, s>>>(a);
+  k_resident<T, MODE, NS, SD, HERM><<<n_bins, 32 * BQ_RES_WARPS(2 * sizeof(T), HERM), smem_bytes, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T>
-static cudaError_t launch_resident_t(const ResArgs& a, int mode, int ns, int herm, int n_bins, int smem_bytes,
-                                     cudaStream_t s) {
+// variant: bit 0 = a general off-diagonal coefficient, bit 1 = a sandwich term with source (k + 1, l + 1),
+// bit 2 = sandwich terms restricted to k = l
+template <typename T, bool HERM>
+static cudaError_t launch_resident_t(const ResArgs& a, int variant, int n_bins, int smem_bytes, cudaStream_t s) {
   if (n_bins <= 0) return cudaSuccess;
-  if (mode == 1) {
-    if (ns == 1)
-      return herm ? launch_resident_one<T, 1, 1, true>(a, n_bins, smem_bytes, s)
-                  : launch_resident_one<T, 1, 1, false>(a, n_bins, smem_bytes, s);
-    return herm ? launch_resident_one<T, 1, 2, true>(a, n_bins, smem_bytes, s)
-                : launch_resident_one<T, 1, 2, false>(a, n_bins, smem_bytes, s);
+  switch (variant) {
+    case 0: return launch_resident_one<T, 1, 1, false, HERM>(a, n_bins, smem_bytes, s);
+    case 1: return launch_resident_one<T, 2, 1, false, HERM>(a, n_bins, smem_bytes, s);
+    case 2: return launch_resident_one<T, 1, 2, false, HERM>(a, n_bins, smem_bytes, s);
+    case 3: return launch_resident_one<T, 2, 2, false, HERM>(a, n_bins, smem_bytes, s);
+    case 4: return launch_resident_one<T, 1, 1, true, HERM>(a, n_bins, smem_bytes, s);
+    case 5: return launch_resident_one<T, 2, 1, true, HERM>(a, n_bins, smem_bytes, s);
+    case 6: return launch_resident_one<T, 1, 2, true, HERM>(a, n_bins, smem_bytes, s);
+    default: return launch_resident_one<T, 2, 2, true, HERM>(a, n_bins, smem_bytes, s);
   }
-  if (ns == 1)
-    return herm ? launch_resident_one<T, 2, 1, true>(a, n_bins, smem_bytes, s)
-                : launch_resident_one<T, 2, 1, false>(a, n_bins, smem_bytes, s);
-  return herm ? launch_resident_one<T, 2, 2, true>(a, n_bins, smem_bytes, s)
-              : launch_resident_one<T, 2, 2, false>(a, n_bins, smem_bytes, s);
 }
 
 }  // namespace bq

@@ -8,10 +8,10 @@
 
 // warps of a CTA: FP32 two CTAs per SM (128 registers a thread; 112 in the general layout, whose
 // largest systems take nine warps), FP64 one
-#define BQ_RES_WARPS(cs, herm) ((cs) == 16 ? 16 : (herm) ? 8 : 9)
-// whether a strip's compensation and own stage input live in shared memory (registers are short)
-#define BQ_RES_COMP_SMEM(cs, herm) ((cs) == 16 || !(herm))
+#define BQ_RES_WARPS(cs, herm) ((cs) == 16 ? 16 : (herm) ? 10 : 9)
 #define BQ_RES_MAXW 16
+// elements from one row of a stage buffer to the next (P <= 43)
+#define BQ_RES_COLS 44
 #define BQ_RES_SMEM_MAX (200 * 1024)
 
 namespace bq {
@@ -71,18 +71,27 @@ struct ResArgs {
   int n_steps;
   long long step0;             // the launch's first step is at tau0 + step0 dt
   double dt, tau0, horizon;
+  // dt, dt / 2 and the pair w_hi + w_lo = dt / 6 in the state's precision (converted on the host: in
+  // the kernel the compiler repeats the conversions every stage, on the scarce FP64 pipe)
+  double cd[4];
+  float cf[4];
 };
 
-// Steps every system of the bins' groups by a.n_steps RK4 steps in one launch.  mode 1: the
-// off-diagonal coefficient is purely imaginary at all times, 2: any; ns: 1 = no sandwich term
-// with source (k + 1, l + 1), 2 = some; herm: the groups are laid out for Hermitian systems.
-cudaError_t launch_resident_f32(const ResArgs& a, int mode, int ns, int herm, int n_bins, int smem_bytes, cudaStream_t s);
-cudaError_t launch_resident_f64(const ResArgs& a, int mode, int ns, int herm, int n_bins, int smem_bytes, cudaStream_t s);
+// Steps every system of the bins' groups by a.n_steps RK4 steps in one launch; the groups are laid
+// out for Hermitian systems (herm) or for any (gen).  variant: bit 0 = the off-diagonal coefficient
+// is not purely imaginary at all times, bit 1 = there are sandwich terms with source (k + 1, l + 1),
+// bit 2 = the sandwich terms are restricted to k = l.
+cudaError_t launch_resident_f32_herm(const ResArgs& a, int variant, int n_bins, int smem_bytes, cudaStream_t s);
+cudaError_t launch_resident_f32_gen(const ResArgs& a, int variant, int n_bins, int smem_bytes, cudaStream_t s);
+cudaError_t launch_resident_f64_herm(const ResArgs& a, int variant, int n_bins, int smem_bytes, cudaStream_t s);
+cudaError_t launch_resident_f64_gen(const ResArgs& a, int variant, int n_bins, int smem_bytes, cudaStream_t s);
 // flags[sys] = 1 where the system's G_x, G_y, R (and their compensation) are exactly Hermitian
 // (G_y = conj G_x, R = R^dagger) for the n groups given.
 cudaError_t launch_res_check(const ResGroup* groups, int n, const void* y, const void* comp, int comp_zero, int dtype,
                              unsigned char* flags, cudaStream_t s);
 
+// Elements from one strip of a stage buffer to the next: its rows, rounded up to P modulo 16.
+__host__ __device__ inline int res_strip_stride(int rb, int P) { return rb * BQ_RES_COLS + (((P - rb * BQ_RES_COLS) % 16 + 16) % 16); }
 // Shared memory (bytes) of a group: stage buffers, G stage inputs, row products, envelope table.
 inline size_t res_group_smem(int stage_elems, int M, size_t cs) {
   const int cols = M | 1;  // (the Hermitian layout's columns)

@@ -1,10 +1,10 @@
-// FP64 instantiations of the resident single-mode kernel, and the Hermitian check of both types.
+// FP64 instantiations of the resident single-mode kernel, general layout, and the Hermitian check of both types.
 #include "bq_resident.cuh"
 
 namespace bq {
 
-cudaError_t launch_resident_f64(const ResArgs& a, int mode, int ns, int herm, int n_bins, int smem_bytes, cudaStream_t s) {
-  return launch_resident_t<double>(a, mode, ns, herm, n_bins, smem_bytes, s);
+cudaError_t launch_resident_f64_gen(const ResArgs& a, int variant, int n_bins, int smem_bytes, cudaStream_t s) {
+  return launch_resident_t<double, false>(a, variant, n_bins, smem_bytes, s);
 }
 
 // One warp per system: exact comparison of every element with its mirror (a NaN compares

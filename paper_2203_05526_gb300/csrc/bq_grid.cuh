@@ -5,17 +5,20 @@
 // descriptors, on building coefficient tables and on integer work per term; the FP64 pipe was
 // busy a third of the time.  Here every point stays with one lane for the whole call, its
 // state, stage sum, compensation and stage input in shared memory; only the stage input is
-// exchanged, through L2, with one grid barrier per stage.  Per point (k, l), k and l flat over the modes,
+// exchanged, through L2, in numbered slots that the readers poll (below: slots_wait).  Per point
+// (k, l), k and l flat over the modes,
 //   (dx_k + dy_l) u + sum_j a_j (xm_k u(k-d,l) - yp_l u(k,l+d)) - conj(a_j) (xp_k u(k+d,l) - ym_l u(k,l-d))
 //   + sum_q sx_k sy_l (u(k+s,l+s) + G_x[k+s] G_y[l+s])
 // with real static weights in tables of n_g entries (products over the modes, zero where the
 // source leaves the grid) and one complex coefficient per pair of a Hermitian H's terms: two
 // to three times fewer FP64 operations than term by term.  Hermitian states (see
 // bq_resident.cuh for the layout) hold half the points.
-// Measured (one GB300, FP64, per RK4 step): two modes at N = 12 45 -> 20 us, three modes at N = 6
-// direct 183 -> 68, mapped with R(xy) (125 systems) 279 -> 66; the 131-parameter control gradient
-// 201 -> 76.  What bounds a stage now: the barrier (1.3 us), one round trip to L2, and the FP64
-// pipe (one warp instruction per 16 cycles and SM).
+// Measured (one GB300, FP64, per RK4 step; one launch per stage / a grid barrier per stage / slots):
+// two modes at N = 12 45 / 20 / 11.0 us, three modes at N = 6 direct 183 / 68 / 32, mapped with R(xy)
+// (125 systems) 279 / 66 / 53; the 131-parameter control gradient 201 / 76 / 52; one oscillator at N =
+// 40, which the resident kernel keeps on one SM in 36 us, 10.  What bounds a stage now: small states
+// the chain store, L2, poll, arithmetic of one warp (2.2 us); large ones the FP64 pipe (one warp
+// instruction per 16 cycles and SM).
 #pragma once
 
 #include "bq_device.cuh"
@@ -29,23 +32,19 @@ template <typename C> __device__ __forceinline__ C ld_cg(const C* p);
 template <> __device__ __forceinline__ float2 ld_cg<float2>(const float2* p) { return __ldcg(p); }
 template <> __device__ __forceinline__ double2 ld_cg<double2>(const double2* p) { return __ldcg(p); }
 
-// Grid barrier number `round` (1, 2, ...) of a launch: one counter, zero before the launch, that
-// every CTA adds one to; one thread per CTA waits for round x CTAs arrivals.  Measured on 152
-// CTAs: 1.3 us; a word per CTA polled by everybody (no atomics) takes 6.5 us, the polls of 152 x
-// 152 words delaying the stores they wait for.  The wait is bounded; on timeout the error word is
-// set and the caller returns.  The CTA's earlier writes are visible to the others after it.
-__device__ __forceinline__ bool grid_sync(unsigned int* bar, unsigned int round, unsigned int* error) {
+// A launch's first grid barrier: one counter, zero before the launch, that every CTA adds one to; one
+// thread per CTA waits for all.  The wait is bounded; on timeout the error word is set and the caller
+// returns.  The CTA's earlier writes are visible to the others after it.
+__device__ __forceinline__ bool grid_sync(unsigned int* bar, unsigned int* error) {
   __syncthreads();
   int bad = 0;
   if (threadIdx.x == 0) {
-    __threadfence();
     unsigned int v;
-    asm volatile("atom.release.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(bar) : "memory");
-    const unsigned int want = round * gridDim.x;  // (wraps with the counter: compared as a difference)
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     const long long t0 = clock64();
     for (;;) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-      if ((int)(v - want) >= 0) break;
+      if (v >= gridDim.x) break;
       if (clock64() - t0 > BQ_GRID_WAIT_CYCLES2) {
         atomicOr(error, 4u);
         bad = 1;
@@ -105,13 +104,9 @@ __device__ __forceinline__ C pair_sum(C a, C p, C q, C k) {
   return k;
 }
 
-// g += u v, summed in FP64 (an FP32 product is rounded to FP32 first, as in the other kernels).
-__device__ __forceinline__ void grad_add(double2& g, double2 u, double2 v) { g = cfma(u, v, g); }
-__device__ __forceinline__ void grad_add(double2& g, float2 u, float2 v) {
-  const float2 p = cmul(u, v);
-  g.x += (double)p.x;
-  g.y += (double)p.y;
-}
+// g += a b + c d, summed in FP64 (FP32 products are rounded to FP32 first, as in the other kernels).
+__device__ __forceinline__ void grad_add(double& g, double a, double b, double c, double d) { g = fma(a, b, fma(c, d, g)); }
+__device__ __forceinline__ void grad_add(double& g, float a, float b, float c, float d) { g += (double)fmaf(a, b, c * d); }
 
 // Envelopes of the problem's pairs for the eight steps from s0 on (32 stages, one per lane), into
 // half (s0 / 8) & 1 of E[2][32][MAXP].
@@ -202,35 +197,138 @@ struct GridSlots {
   }
 };
 
-template <typename C>
-__device__ __forceinline__ C ld_at(const C* b, int o) {  // the value at a program offset
-  return conj_bit(ld_cg(b + (o & 0x7fffffff)), (unsigned)o & 0x80000000u);
+// ---- the exchange of stage inputs ----------------------------------------------------------------
+// A slot is a value together with the number of the stage it is for, in 16-byte words {value,
+// number} (FP64: one word per component; FP32: the value fits in one), each written and read as a
+// whole (b128 accesses are single-copy atomic).  A reader polls the slots it needs until they carry
+// its stage's number: no fence, no barrier, no flag between the writer's store and the reader's
+// load.  A grid barrier per stage took four dependent trips to L2 (fence, counter, poll, load),
+// this takes one and a half, and warps without a stage's last neighbours wait alone.
+// (slot_get returns zero if the slot carries the number.)  Slot i of a place: FP64 in two planes of n words (a warp's 16-byte accesses are then consecutive),
+// base the place's first word.
+__device__ __forceinline__ void slot_put(double2* base, size_t n, int i, double2 v, unsigned int no) {
+  double2* p = base + i;
+  asm volatile(
+      "{\n.reg .b128 a, b;\nmov.b128 a, {%1, %3};\nmov.b128 b, {%2, %3};\n"
+      "st.relaxed.gpu.global.b128 [%0], a;\nst.relaxed.gpu.global.b128 [%4], b;\n}" ::"l"(p),
+      "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "l"((unsigned long long)no), "l"(p + n)
+      : "memory");
+}
+__device__ __forceinline__ void slot_put(float2* base, size_t, int i, float2 v, unsigned int no) {
+  float2* p = base + 2 * (size_t)i;
+  const unsigned long long w = (unsigned long long)__float_as_uint(v.y) << 32 | __float_as_uint(v.x);
+  asm volatile("{\n.reg .b128 a;\nmov.b128 a, {%1, %2};\nst.relaxed.gpu.global.b128 [%0], a;\n}" ::"l"(p), "l"(w),
+               "l"((unsigned long long)no)
+               : "memory");
+}
+__device__ __forceinline__ unsigned int slot_get(const double2* base, size_t n, int i, unsigned int no, double2& v) {
+  const double2* p = base + i;
+  unsigned long long x, y, n0, n1;
+  asm volatile(
+      "{\n.reg .b128 a, b;\nld.relaxed.gpu.global.b128 a, [%4];\nld.relaxed.gpu.global.b128 b, [%5];\n"
+      "mov.b128 {%0, %1}, a;\nmov.b128 {%2, %3}, b;\n}"
+      : "=l"(x), "=l"(n0), "=l"(y), "=l"(n1)
+      : "l"(p), "l"(p + n)
+      : "memory");
+  v.x = __longlong_as_double((long long)x);
+  v.y = __longlong_as_double((long long)y);
+  return ((unsigned int)n0 ^ no) | ((unsigned int)n1 ^ no);
+}
+__device__ __forceinline__ unsigned int slot_get(const float2* base, size_t, int i, unsigned int no, float2& v) {
+  const float2* p = base + 2 * (size_t)i;
+  unsigned long long w, n0;
+  asm volatile("{\n.reg .b128 a;\nld.relaxed.gpu.global.b128 a, [%2];\nmov.b128 {%0, %1}, a;\n}"
+               : "=l"(w), "=l"(n0)
+               : "l"(p)
+               : "memory");
+  v.x = __uint_as_float((unsigned int)w);
+  v.y = __uint_as_float((unsigned int)(w >> 32));
+  return (unsigned int)n0 ^ no;
 }
 
-template <typename T, int NP, int NS>
-__global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_fwd(const GridArgs A) {
+// off(j): program offset of value j (sign bit: conjugate); on: bit j set where value j is wanted (the
+// others come back zero).  The whole warp calls it and stays together in the loop: when lanes left it
+// one by one the arithmetic behind it was issued for several parts of the warp in turn (the FP64 pipe
+// 93% busy for 44% of useful lanes, three modes direct).  The wait is bounded: a thread that gives up
+// sets the error word and *dead, does not wait again, and the launch ends without storing.
+template <int N, typename C, typename F>
+__device__ __forceinline__ void slots_wait(const C* base, size_t n, F off, unsigned int on, unsigned int no, C (&v)[N],
+                                           unsigned int* error, int* dead) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) v[j] = cmk<C>(0.0, 0.0);
+  long long t0 = 0;
+  for (;;) {
+    unsigned int bad = 0u;
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+      if (on >> j & 1u) bad |= slot_get(base, n, off(j) & 0x7fffffff, no, v[j]);
+    if (!__any_sync(0xffffffffu, bad)) break;
+    if (!t0) t0 = clock64();
+    const bool stop = clock64() - t0 > BQ_GRID_WAIT_CYCLES2 || *(volatile int*)dead;
+    if (stop && bad) atomicOr(error, 4u);
+    if (__any_sync(0xffffffffu, stop)) {
+      *(volatile int*)dead = 1;
+      break;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j)
+    if (on >> j & 1u) v[j] = conj_bit(v[j], (unsigned)off(j) & 0x80000000u);
+}
+
+// Slots are used in turn: stage number `no` has place no % ring.  On entering a block of `block`
+// steps (block h = 1, 2, ...) a CTA counts itself and waits until all have entered block h - 1; every
+// read of block h - 2 is then over, and its places (and one) may be written again: ring = 8 block +
+// 1.  The wait is almost always over before it begins.  bar[0] is the launch's first barrier; block h
+// counts in bar[1 + h % 4] (CTAs are never more than two blocks apart, so a word's counts of
+// different blocks do not mix; one counter for all blocks would let fast CTAs stand in for slow ones).
+__device__ __forceinline__ bool block_sync(unsigned int* bar, unsigned int h, unsigned int* error, int* dead) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar + 1 + (h & 3u)) : "memory");
+    const unsigned int b = h - 1, want = ((b + 3u) >> 2) * gridDim.x;  // (wraps with the counter: compared as a difference)
+    const long long t0 = clock64();
+    while (b > 0) {
+      unsigned int v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar + 1 + (b & 3u)) : "memory");
+      if ((int)(v - want) >= 0) break;
+      if (clock64() - t0 > BQ_GRID_WAIT_CYCLES2) {
+        atomicOr(error, 4u);
+        *(volatile int*)dead = 1;
+        break;
+      }
+    }
+  }
+  return __syncthreads_or(threadIdx.x == 0 && *(volatile int*)dead) == 0;
+}
+
+// SMALL (GRID_ONE): at most two pairs and two sandwich terms and a piece per warp: its state and its
+// neighbours' offsets stay in registers and every value comes in one batch of loads.  Else the
+// program is read from shared memory and the pairs go in batches of two or, with 256 threads (no
+// more than eight pieces a CTA, 255 registers), four.
+template <typename T, bool SMALL, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
   using C = typename C2T<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ GridProb P;
+  __shared__ int dead;
   const GridCta cta = A.ctas[blockIdx.x];
-  for (int i = threadIdx.x; i < (int)(sizeof(GridProb) / 4); i += BQ_GRID_THREADS)
+  for (int i = threadIdx.x; i < (int)(sizeof(GridProb) / 4); i += THREADS)
     reinterpret_cast<int*>(&P)[i] = reinterpret_cast<const int*>(A.probs + cta.prob)[i];
+  if (threadIdx.x == 0) dead = 0;
   __syncthreads();
   const int ng = P.ng, np = P.np, ns = P.ns;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = BQ_GRID_THREADS / 32;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = THREADS / 32;
   const GridSlots<T> S(smem_raw, cta.n, 4 * np + ns, 4 * np + 3 * ns);
   const int n = S.n;
   C* const E = S.E;
   const C zero = cmk<C>(0.0, 0.0);
-  for (int i = tid; i < cta.n * (int)(sizeof(GridPiece) / 4); i += BQ_GRID_THREADS)
+  for (int i = tid; i < cta.n * (int)(sizeof(GridPiece) / 4); i += THREADS)
     reinterpret_cast<int*>(S.pc)[i] = reinterpret_cast<const int*>(A.pieces + cta.p0)[i];
   __syncthreads();
-  C* ua = reinterpret_cast<C*>(A.ua);
-  C* ub = reinterpret_cast<C*>(A.ub);
-  auto slot = [&](long long i, int stage) -> C* {
-    if (A.rec) return reinterpret_cast<C*>(A.rec + ((size_t)i * 4 + stage - 1) * A.arr);
-    return (stage & 1) ? ua : ub;
-  };
+  C* const ring = reinterpret_cast<C*>(A.ring);
+  const size_t slots = A.arr / sizeof(C), place = 2 * slots;  // of a place of the ring; its elements
+  auto recorded = [&](long long i, int stage) { return reinterpret_cast<C*>(A.rec + ((size_t)i * 4 + stage - 1) * A.arr); };
   const int Pc = ng | 1;
   auto position = [&](const GridPiece& g) {
     GridPos p;
@@ -317,122 +415,230 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_fwd(const GridArgs 
     S.v1[pi] = zero;
     S.v2[pi] = cv;
     S.dg[pi] = dg;
-    if (lane < g.len) slot(0, 1)[self] = yv;
+    if (g.kind <= GRID_D) {  // (terms restricted to the diagonal of a mode are absent from most warps)
+      unsigned int any = 0u;
+      for (int s = 0; s < ns; ++s)
+        if (__any_sync(0xffffffffu, S.w[(4 * np + s) * n + pi] != (T)0)) any |= (P.has_sep ? 7u : 1u) << (3 * s);
+      if (lane == 0) S.pc[q].pad = (int)any;
+    }
+    if (lane < g.len) {
+      for (int r = 0; r < A.ring_places; ++r)
+        if (r != 1) slot_put(ring + r * place, slots, self, zero, 0u);
+      slot_put(ring + place, slots, self, yv, 1u);
+      if (A.rec) recorded(0, 1)[self] = yv;
+    }
   }
   if (warp == nw - 1) grid_envelope<T>(A, P, E, 0);
-  unsigned int epoch = 1;
-  if (!grid_sync(A.bar, epoch, A.error)) return;
+  unsigned int block = 0;
+  if (!grid_sync(A.bar, A.error)) return;
 
   const T hh = (T)A.dt, h2 = (T)(0.5 * A.dt);
   const double wd = A.dt / 6.0;
   const T w_hi = (T)wd, w_lo = (T)(wd - (double)w_hi);
+  unsigned int no = 1;       // number and place of the stage's input
+  const C* in = ring + place;
+  int turn = 1;
+  // the state after a step: y + (sum + k) dt / 6 with its rounding error carried along
+  auto update = [&](C sum, C k, C yv, C& cv) {
+    const C s = cadd(sum, k);
+    C d, e, nu;
+    if constexpr (sizeof(T) == 4) {
+      d.x = fma(w_hi, s.x, fma(w_lo, s.x, -cv.x));
+      d.y = fma(w_hi, s.y, fma(w_lo, s.y, -cv.y));
+      two_sum(yv, d, nu, e);
+      cv = cneg(e);
+    } else {  // (w_lo is zero)
+      d.x = fma(w_hi, s.x, -cv.x);
+      d.y = fma(w_hi, s.y, -cv.y);
+      nu.x = yv.x + d.x;
+      nu.y = yv.y + d.y;
+      cv.x = (nu.x - yv.x) - d.x;
+      cv.y = (nu.y - yv.y) - d.y;
+    }
+    return nu;
+  };
+  // SMALL: a warp's one piece, its offsets, state, sum and compensation in registers
+  int of[SMALL ? 14 : 1];
+  unsigned int on = 0u;
+  C y1 = zero, s1 = zero, c1 = zero, u1 = zero, dg1 = zero;
+  int kind1 = 0, xi1 = -1;
+  bool real1 = false;
+  if (SMALL && warp < cta.n) {
+    const GridPiece& g = S.pc[warp];
+    const int pi = 32 * warp + lane;
+    kind1 = g.kind;
+    if (lane < g.len) xi1 = xidx(g);
+    const unsigned int any = (unsigned int)g.pad;
+#pragma unroll
+    for (int i = 0; i < (SMALL ? 14 : 1); ++i) {
+      // values 0..7: pairs (points of G have two of each four); 8..13: sandwich terms
+      const bool want = i < 8 ? i < 4 * np && kind1 != GRID_D && (kind1 <= GRID_H || (i & 3) < 2) : any >> (i - 8) & 1u;
+      of[i] = want ? S.off[(i < 8 ? i : 4 * np + ((i - 8) % 3) * ns + (i - 8) / 3) * n + pi] : 0;
+      on |= (want ? 1u : 0u) << i;
+    }
+    y1 = u1 = S.v0[pi];
+    c1 = S.v2[pi];
+    dg1 = S.dg[pi];
+    real1 = S.fl[pi] & 2;
+  }
 #pragma unroll 1
   for (int step = 0; step < A.n_steps; ++step) {
+    if (step > 0 && (step & (A.block - 1)) == 0) {
+      if (!block_sync(A.bar, ++block, A.error, &dead)) return;
+    }
+    // (the next eight steps' envelopes: behind a block boundary, ahead of the one before their use)
+    if ((step & 7) == 4 && (step | 7) + 1 < A.n_steps && warp == nw - 1) grid_envelope<T>(A, P, E, (step | 7) + 1);
 #pragma unroll 1
     for (int stage = 1; stage <= 4; ++stage) {
-      const C* in = slot(step, stage);
-      const bool more = step + 1 < A.n_steps;
-      C* out = stage < 4 ? slot(step, stage + 1) : more ? slot(step + 1, 1) : nullptr;
+      const bool send = stage < 4 || step + 1 < A.n_steps;
+      turn = turn + 1 == A.ring_places ? 0 : turn + 1;
+      C* out = ring + turn * place;
       const C* Es = E + (((step >> 3) & 1) * 32 + (step & 7) * 4 + stage - 1) * BQ_GRID_MAXP;
+      if constexpr (SMALL) {
+        if (on || warp < cta.n) {
+          const T* w = S.w + 32 * warp + lane;
+          C v[14];
+          slots_wait<14>(in, slots, [&](int i) { return of[i]; }, on, no, v, A.error, &dead);
+          C k = cmul(dg1, u1);
+          const unsigned int yc = kind1 == GRID_Y ? 0x80000000u : 0u;
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            if (on >> (4 * j) & 1u) {  // (points of G: values and weights 2, 3 are zero)
+              const T w0 = w[(4 * j) * n], w1 = w[(4 * j + 1) * n], w2 = w[(4 * j + 2) * n], w3 = w[(4 * j + 3) * n];
+              const C a = conj_bit(Es[j], yc);
+              C p;
+              p.x = fma(w0, v[4 * j].x, -w3 * v[4 * j + 3].x);
+              p.y = fma(w0, v[4 * j].y, -w3 * v[4 * j + 3].y);
+              if (a.x == 0) {  // a = i b: the sum in one chain
+                p.x = fma(w1, v[4 * j + 1].x, fma(-w2, v[4 * j + 2].x, p.x));
+                p.y = fma(w1, v[4 * j + 1].y, fma(-w2, v[4 * j + 2].y, p.y));
+                k.x = fma(-a.y, p.y, k.x);
+                k.y = fma(a.y, p.x, k.y);
+              } else {
+                C b;
+                b.x = fma(w1, v[4 * j + 1].x, -w2 * v[4 * j + 2].x);
+                b.y = fma(w1, v[4 * j + 1].y, -w2 * v[4 * j + 2].y);
+                k = pair_sum(a, p, b, k);
+              }
+            }
+#pragma unroll
+          for (int s = 0; s < 2; ++s)
+            if (on >> (8 + 3 * s) & 1u) {
+              const C z = on >> (9 + 3 * s) & 1u ? cfma(v[9 + 3 * s], v[10 + 3 * s], v[8 + 3 * s]) : v[8 + 3 * s];
+              k = caxpy(w[(4 * np + s) * n], z, k);
+            }
+          if (real1) k.y = (T)0;  // the diagonal of a Hermitian system is real
+          if (stage < 4) {
+            u1 = caxpy(stage == 3 ? hh : h2, k, y1);
+            s1 = stage == 1 ? k : caxpy((T)2, k, s1);
+          } else {
+            y1 = u1 = update(s1, k, y1, c1);
+          }
+          if (send && xi1 >= 0) {
+            slot_put(out, slots, xi1, u1, no + 1);
+            if (A.rec) (stage < 4 ? recorded(step, stage + 1) : recorded(step + 1, 1))[xi1] = u1;
+          }
+        }
+      } else {
 #pragma unroll 1
       for (int q = warp; q < cta.n; q += nw) {
         const int kind = S.pc[q].kind, len = S.pc[q].len;
+        const unsigned int any = (unsigned int)S.pc[q].pad;
         const int pi = 32 * q + lane;
         const T* w = S.w + pi;
         const int* off = S.off + pi;
         const C u = S.v3[pi];
         C k = cmul(S.dg[pi], u);
-        if (kind <= GRID_H) {
-          // every load first: they are independent and come from L2
-          C nb[4 * NP];
-#pragma unroll
-          for (int j = 0; j < 4 * NP; ++j)
-            if (j < 4 * np) nb[j] = ld_at(in, off[j * n]);
-#pragma unroll
-          for (int j = 0; j < NP; ++j) {
-            if (j >= np) break;
-            const T w0 = w[(4 * j) * n], w1 = w[(4 * j + 1) * n], w2 = w[(4 * j + 2) * n], w3 = w[(4 * j + 3) * n];
-            C a, b;
-            a.x = fma(w0, nb[4 * j].x, -w3 * nb[4 * j + 3].x);
-            a.y = fma(w0, nb[4 * j].y, -w3 * nb[4 * j + 3].y);
-            b.x = fma(w1, nb[4 * j + 1].x, -w2 * nb[4 * j + 2].x);
-            b.y = fma(w1, nb[4 * j + 1].y, -w2 * nb[4 * j + 2].y);
-            k = pair_sum(Es[j], a, b, k);
+        // pair j of R with its four neighbours, and a sandwich term with its three
+        auto pair = [&](int j, C n0, C n1, C n2, C n3) {
+          const T w0 = w[(4 * j) * n], w1 = w[(4 * j + 1) * n], w2 = w[(4 * j + 2) * n], w3 = w[(4 * j + 3) * n];
+          const C a = Es[j];
+          C p;
+          p.x = fma(w0, n0.x, -w3 * n3.x);
+          p.y = fma(w0, n0.y, -w3 * n3.y);
+          if (a.x == 0) {  // a = i b: the sum in one chain
+            p.x = fma(w1, n1.x, fma(-w2, n2.x, p.x));
+            p.y = fma(w1, n1.y, fma(-w2, n2.y, p.y));
+            k.x = fma(-a.y, p.y, k.x);
+            k.y = fma(a.y, p.x, k.y);
+          } else {
+            C b;
+            b.x = fma(w1, n1.x, -w2 * n2.x);
+            b.y = fma(w1, n1.y, -w2 * n2.y);
+            k = pair_sum(a, p, b, k);
           }
-        } else if (kind >= GRID_X) {
-          C lo[NP], hi[NP];
+        };
+        auto sand = [&](int s, C v, C x, C y) {
+          k = caxpy(w[(4 * np + s) * n], P.has_sep ? cfma(x, y, v) : v, k);
+        };
+        auto soff = [&](int i) { return off[(4 * np + (i % 3) * ns + i / 3) * n]; };  // value i of the sandwich terms
+        if (kind >= GRID_X) {
+#pragma unroll 1
+          for (int j0 = 0; j0 < np; j0 += 4) {
+            const int m = min(4, np - j0);
+            C v[8];
+            slots_wait<8>(in, slots, [&](int i) { return off[(4 * (j0 + i / 2) + (i & 1)) * n]; }, (1u << (2 * m)) - 1u, no, v,
+                          A.error, &dead);
 #pragma unroll
-          for (int j = 0; j < NP; ++j)
-            if (j < np) {
-              lo[j] = ld_at(in, off[(4 * j) * n]);
-              hi[j] = ld_at(in, off[(4 * j + 1) * n]);
-            }
-#pragma unroll
-          for (int j = 0; j < NP; ++j) {
-            if (j >= np) break;
-            k = pair_sum(conj_bit(Es[j], kind == GRID_X ? 0u : 0x80000000u), cscale(lo[j], w[(4 * j) * n]),
-                         cscale(hi[j], w[(4 * j + 1) * n]), k);
-          }
-        }
-        if (kind <= GRID_D) {
-          C sv[NS], sx[NS], sy[NS];
-          T sw[NS];
-          unsigned any = 0u;
-#pragma unroll
-          for (int s = 0; s < NS; ++s) {
-            if (s >= ns) break;
-            sw[s] = w[(4 * np + s) * n];
-            // (terms restricted to the diagonal of a mode are absent from most warps)
-            if (__any_sync(0xffffffffu, sw[s] != (T)0)) {
-              any |= 1u << s;
-              sv[s] = ld_at(in, off[(4 * np + s) * n]);
-              if (P.has_sep) {
-                sx[s] = ld_at(in, off[(4 * np + ns + s) * n]);
-                sy[s] = ld_at(in, off[(4 * np + 2 * ns + s) * n]);
-              }
+            for (int i = 0; i < 4; ++i) {
+              if (i >= m) break;
+              const int j = j0 + i;
+              k = pair_sum(conj_bit(Es[j], kind == GRID_X ? 0u : 0x80000000u), cscale(v[2 * i], w[(4 * j) * n]),
+                           cscale(v[2 * i + 1], w[(4 * j + 1) * n]), k);
             }
           }
+        } else {
+          constexpr int PB = THREADS == 256 ? 4 : 2;
+          if (kind <= GRID_H) {
+#pragma unroll 1
+            for (int j0 = 0; j0 < np; j0 += PB) {
+              const int m = min(PB, np - j0);
+              C v[4 * PB];
+              slots_wait<4 * PB>(in, slots, [&](int i) { return off[(4 * j0 + i) * n]; }, (1u << (4 * m)) - 1u, no, v, A.error, &dead);
 #pragma unroll
-          for (int s = 0; s < NS; ++s) {
-            if (s >= ns) break;
-            if (any >> s & 1) k = caxpy(sw[s], P.has_sep ? cfma(sx[s], sy[s], sv[s]) : sv[s], k);
+              for (int i = 0; i < PB; ++i)
+                if (i < m) pair(j0 + i, v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            }
+          }
+#pragma unroll 1
+          for (int s0 = 0; s0 < ns; s0 += 2) {
+            const unsigned int on = any >> (3 * s0) & 63u;
+            if (!on) continue;
+            C v[6];
+            slots_wait<6>(in, slots, [&](int i) { return soff(3 * s0 + i); }, on, no, v, A.error, &dead);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+              if (on >> (3 * s) & 1u) sand(s0 + s, v[3 * s], v[3 * s + 1], v[3 * s + 2]);
           }
         }
-        const int fl = S.fl[pi];
-        if (fl & 2) k.y = (T)0;  // the diagonal of a Hermitian system is real
+        if (S.fl[pi] & 2) k.y = (T)0;  // the diagonal of a Hermitian system is real
         C nu;
         if (stage < 4) {
           nu = caxpy(stage == 3 ? hh : h2, k, S.v0[pi]);
           S.v1[pi] = stage == 1 ? k : caxpy((T)2, k, S.v1[pi]);
         } else {
-          const C yv = S.v0[pi];
-          const C s = cadd(S.v1[pi], k), cv = S.v2[pi];
-          C d, e;
-          if constexpr (sizeof(T) == 4) {
-            d.x = fma(w_hi, s.x, fma(w_lo, s.x, -cv.x));
-            d.y = fma(w_hi, s.y, fma(w_lo, s.y, -cv.y));
-            two_sum(yv, d, nu, e);
-            S.v2[pi] = cneg(e);
-          } else {  // (w_lo is zero)
-            d.x = fma(w_hi, s.x, -cv.x);
-            d.y = fma(w_hi, s.y, -cv.y);
-            nu.x = yv.x + d.x;
-            nu.y = yv.y + d.y;
-            e.x = (nu.x - yv.x) - d.x;
-            e.y = (nu.y - yv.y) - d.y;
-            S.v2[pi] = e;
-          }
+          C cv = S.v2[pi];
+          nu = update(S.v1[pi], k, S.v0[pi], cv);
+          S.v2[pi] = cv;
           S.v0[pi] = nu;
         }
         S.v3[pi] = nu;
-        if (out && lane < len) out[xidx(S.pc[q])] = nu;
+        if (send && lane < len) {
+          const int i = xidx(S.pc[q]);
+          slot_put(out, slots, i, nu, no + 1);
+          if (A.rec) (stage < 4 ? recorded(step, stage + 1) : recorded(step + 1, 1))[i] = nu;
+        }
       }
-      if (stage == 1 && (step & 7) == 4 && (step | 7) + 1 < A.n_steps && warp == nw - 1)
-        grid_envelope<T>(A, P, E, (step | 7) + 1);
-      if (stage < 4 || more) {
-        if (!grid_sync(A.bar, ++epoch, A.error)) return;
       }
+      ++no;
+      in = out;
     }
+  }
+  __syncthreads();
+  if (*(volatile int*)&dead) return;
+  if (SMALL && warp < cta.n) {
+    S.v0[32 * warp + lane] = y1;
+    S.v2[32 * warp + lane] = c1;
   }
   for (int q = warp; q < cta.n; q += nw) {
     const GridPiece g = S.pc[q];
@@ -467,32 +673,37 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_fwd(const GridArgs 
 // passed: a warp per G point sums it directly, in the same phase as the points of R (no
 // reduction phase of its own).  Parameter sums stay in registers: per pair u P^T b and u Q^T b,
 // reduced into the gradient slots when an envelope changes its value and at the end.
-template <typename T, int NP, int NS>
-__global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs A) {
+// ONE (at most two pairs, two sandwich terms, eight pieces a CTA and ten row values a lane): a warp's one piece with its
+// offsets and state in registers and every value it needs in one batch of loads.
+template <typename T, int NP, int THREADS, bool ONE>
+__global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
   using C = typename C2T<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[BQ_GRID_THREADS / 32][4 * NP + BQ_GRID_MAXT + 2];
+  __shared__ double red[THREADS / 32][2 * NP + BQ_GRID_MAXT + 2];
   __shared__ int segs[2 * 8 * BQ_GRID_MAXP];
   __shared__ GridProb P;
+  __shared__ int dead;
   const GridCta cta = A.ctas[blockIdx.x];
-  for (int i = threadIdx.x; i < (int)(sizeof(GridProb) / 4); i += BQ_GRID_THREADS)
+  for (int i = threadIdx.x; i < (int)(sizeof(GridProb) / 4); i += THREADS)
     reinterpret_cast<int*>(&P)[i] = reinterpret_cast<const int*>(A.probs + cta.prob)[i];
+  if (threadIdx.x == 0) dead = 0;
   __syncthreads();
   const int ng = P.ng, np = P.np, ns = P.ns, nt = P.nt;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = BQ_GRID_THREADS / 32;
-  const GridSlots<T> S(smem_raw, cta.n, 4 * np + ns + 2 * nt, 4 * np + ns);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = THREADS / 32;
+  const int wrow = 4 * np + ns + 2 * nt;  // weights of the row values (ONE)
+  const GridSlots<T> S(smem_raw, cta.n, wrow + (ONE ? BQ_GRID_ROWS : 0), 4 * np + ns);
   const int n = S.n;
   C* const E = S.E;
   // weights of the sandwich terms over the flat index (the sums over rows and columns of b_R)
   T* swt = reinterpret_cast<T*>(S.fl + n);
   const C zero = cmk<C>(0.0, 0.0);
-  for (int i = tid; i < cta.n * (int)(sizeof(GridPiece) / 4); i += BQ_GRID_THREADS)
+  for (int i = tid; i < cta.n * (int)(sizeof(GridPiece) / 4); i += THREADS)
     reinterpret_cast<int*>(S.pc)[i] = reinterpret_cast<const int*>(A.pieces + cta.p0)[i];
   const GridTab<T> W(P, reinterpret_cast<const T*>(A.tab) + P.tab);
-  for (int i = tid; i < 2 * ns * ng; i += BQ_GRID_THREADS) swt[i] = W.sand(0, 0)[i];
+  for (int i = tid; i < 2 * ns * ng; i += THREADS) swt[i] = W.sand(0, 0)[i];
   __syncthreads();
-  C* ba = reinterpret_cast<C*>(A.ua);
-  C* bb = reinterpret_cast<C*>(A.ub);
+  C* const ring = reinterpret_cast<C*>(A.ring);
+  const size_t slots = A.arr / sizeof(C), place = 2 * slots;
   auto xidx = [&](const GridPiece& g) {
     return (g.kind <= GRID_D ? g.off_r : g.kind == GRID_X ? g.off_gx : g.off_gy) + g.start + lane;
   };
@@ -511,7 +722,9 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
     C v = zero, dg = zero;
     if (ok) {
       v = reinterpret_cast<const C*>(A.lam)[self];
-      ba[self] = cscale(v, w6);
+      for (int r = 0; r < A.ring_places; ++r)
+        if (r != 1) slot_put(ring + r * place, slots, self, zero, 0u);
+      slot_put(ring + place, slots, self, cscale(v, w6), 1u);
       if (g.kind <= GRID_D) dg = cadd(W.dx[k], W.dy[l]);
       else if (g.kind == GRID_X) dg = cadd(W.dx[k], cmk<C>(g.c_re, g.c_im));
       else dg = cadd(W.dy[k], cmk<C>(-g.c_re, -g.c_im));
@@ -553,33 +766,194 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
     S.v0[pi] = S.v1[pi] = v;
     S.v3[pi] = cscale(v, w6);
     S.dg[pi] = dg;
+    unsigned int any = 0u;
+    for (int s = 0; s < ns; ++s)
+      if (__any_sync(0xffffffffu, S.w[(4 * np + s) * n + pi] != (T)0)) any |= 1u << s;
+    if (lane == 0) S.pc[q].pad = (int)any;
   }
-  // parameter sums of this thread
-  double2 ga[NP], gb[NP], dcs = make_double2(0.0, 0.0);
+  // parameter sums of this thread: per pair Re sum u (a - b) and Im sum u (a + b), which are all
+  // that Re(da S_a - conj(da) S_b) needs
+  double gx[NP], gy[NP];
+  double2 dcs = make_double2(0.0, 0.0);
   double gt[BQ_GRID_MAXT];
 #pragma unroll
-  for (int j = 0; j < NP; ++j) ga[j] = gb[j] = make_double2(0.0, 0.0);
+  for (int j = 0; j < NP; ++j) gx[j] = gy[j] = 0.0;
 #pragma unroll
   for (int t = 0; t < BQ_GRID_MAXT; ++t) gt[t] = 0.0;
   const long long last = A.n_steps - 1;
   if (warp == nw - 1) grid_envelope<T>(A, P, E, last & ~7LL, segs);
-  unsigned int epoch = 1;
-  if (!grid_sync(A.bar, epoch, A.error)) return;
+  unsigned int block = 0;
+  if (!grid_sync(A.bar, A.error)) return;
 
   auto seg_of = [&](long long i, int j) { return segs[(((i >> 3) & 1) * 8 + (i & 7)) * BQ_GRID_MAXP + j]; };
 
+  unsigned int no = 1;
+  const C* in = ring + place;
+  int turn = 1;
+  // value of pair j at this point: a from sources x.lo, y.lo, b from x.hi, y.hi (see pair_sum)
+  int of[ONE ? 14 : 1], go[ONE ? BQ_GRID_ROWS : 1];
+  unsigned int on = 0u;
+  C l1 = zero, a1 = zero, b1 = zero, dg1 = zero;
+  int kind1 = 0, xi1 = -1, rows = 0;
+  if (ONE && warp < cta.n) {
+    const GridPiece& g = S.pc[warp];
+    const int pi = 32 * warp + lane;
+    const bool isx = g.kind == GRID_X;
+    kind1 = g.kind;
+    if (lane < g.len) xi1 = xidx(g);
+    l1 = a1 = S.v0[pi];
+    b1 = S.v3[pi];
+    dg1 = S.dg[pi];
+    if (kind1 <= GRID_D) {  // values 0..7: pairs, 8, 9: sandwich terms
+#pragma unroll
+      for (int i = 0; i < (ONE ? 14 : 1); ++i) {
+        const bool want = i < 8 ? i < 4 * np && kind1 == GRID_R : (unsigned int)g.pad >> (i - 8) & 1u;
+        of[i] = want ? S.off[(i < 8 ? i : 4 * np + i - 8) * n + pi] : 0;
+        on |= (want ? 1u : 0u) << i;
+      }
+    } else {  // values 0..3: lo and hi of the pairs, 4..13: elements of the rows or columns of b_R
+      const int nj = P.r_diag ? 1 : (ng + 31) / 32;
+      rows = P.has_r ? ns * nj : 0;
+#pragma unroll
+      for (int i = 0; i < (ONE ? 14 : 1); ++i) {
+        of[i] = 0;
+        if (i < 4) {
+          if (i < 2 * np && xi1 >= 0) {
+            of[i] = S.off[(4 * (i >> 1) + (i & 1)) * n + pi];
+            on |= 1u << i;
+          }
+          continue;
+        }
+        const int t = i - 4;
+        go[t] = 0;
+        T wt = (T)0;
+        if (t < rows) {
+          const int s = t / nj, kk = g.start - P.ss[s], j = P.r_diag ? kk : lane + 32 * (t - s * nj);
+          if (kk >= 0 && kk < ng && j < ng && !(P.r_diag && lane)) {
+            wt = swt[(2 * s + (isx ? 0 : 1)) * ng + kk] * swt[(2 * s + (isx ? 1 : 0)) * ng + j];
+            if (!P.r_diag && P.sst[s] && (j / P.sst[s]) % P.sM[s] != (kk / P.sst[s]) % P.sM[s]) wt = (T)0;
+          }
+          if (wt != (T)0) {
+            of[i] = g.off_r + (P.r_diag ? kk : isx ? kk * ng + j : j * ng + kk);
+            go[t] = (isx ? g.off_gy : g.off_gx) + P.ss[s] + j;
+            on |= 1u << i;
+          }
+          S.w[(wrow + t) * n + pi] = wt;
+        }
+      }
+    }
+  }
+  auto grad_pair = [&](int j, C u, C a, C b) {
+    if (P.gpar[j] < 0 && P.gpwc[j] < 0) return;
+    C s = cadd(a, b), d;
+    d.x = a.x - b.x;
+    d.y = a.y - b.y;
+#pragma unroll
+    for (int i = 0; i < NP; ++i)
+      if (i == j) {
+        grad_add(gx[i], u.x, d.x, -u.y, d.y);
+        grad_add(gy[i], u.x, s.y, u.y, s.x);
+      }
+  };
+
 #pragma unroll 1
   for (long long it = last; it >= 0; --it) {
+    if (it != last && ((it + 1) & (A.block - 1)) == 0) {
+      if (!block_sync(A.bar, ++block, A.error, &dead)) return;
+    }
+    // the eight steps below this batch, in its first step (a block boundary, with one before their use)
+    if (((it & 7) == 7 || it == last) && it > 7 && warp == nw - 1) grid_envelope<T>(A, P, E, (it & ~7LL) - 8, segs);
 #pragma unroll 1
     for (int stage = 4; stage >= 1; --stage) {
-      const C* in = (stage & 1) ? bb : ba;
-      C* out = (stage & 1) ? ba : bb;
+      turn = turn + 1 == A.ring_places ? 0 : turn + 1;
+      C* out = ring + turn * place;
       const C* U = reinterpret_cast<const C*>(A.rec + ((size_t)it * 4 + stage - 1) * A.arr);
       const C* Es = E + (((it >> 3) & 1) * 32 + (it & 7) * 4 + stage - 1) * BQ_GRID_MAXP;
+      if constexpr (ONE) {
+        if (warp < cta.n) {
+          const T* w = S.w + 32 * warp + lane;
+          const C u = xi1 >= 0 ? U[xi1] : zero;
+          C h[BQ_GRID_ROWS];
+          if (kind1 >= GRID_X) {
+#pragma unroll
+            for (int t = 0; t < BQ_GRID_ROWS; ++t)
+              if (t < rows) h[t] = on >> (4 + t) & 1u ? cscale(U[go[t]], w[(wrow + t) * n]) : zero;
+          }
+          C v[14];
+          slots_wait<14>(in, slots, [&](int i) { return of[i]; }, on, no, v, A.error, &dead);
+          C qv = cmul(dg1, b1);
+          if (kind1 <= GRID_D) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+              if (on >> (4 * j) & 1u) {
+                const T w0 = w[(4 * j) * n], w1 = w[(4 * j + 1) * n], w2 = w[(4 * j + 2) * n], w3_ = w[(4 * j + 3) * n];
+                C a, c;
+                a.x = fma(w0, v[4 * j].x, -w3_ * v[4 * j + 3].x);
+                a.y = fma(w0, v[4 * j].y, -w3_ * v[4 * j + 3].y);
+                c.x = fma(w1, v[4 * j + 1].x, -w2 * v[4 * j + 2].x);
+                c.y = fma(w1, v[4 * j + 1].y, -w2 * v[4 * j + 2].y);
+                qv = pair_sum(Es[j], a, c, qv);
+                grad_pair(j, u, a, c);
+              }
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+              if (on >> (8 + s) & 1u) qv = caxpy(w[(4 * np + s) * n], v[8 + s], qv);
+          } else {
+            const bool isx = kind1 == GRID_X;
+            C r0 = zero, r1 = zero;
+#pragma unroll
+            for (int t = 0; t < BQ_GRID_ROWS; ++t)
+              if (t < rows) {
+                if (t & 1) r1 = cfma(v[4 + t], h[t], r1);
+                else r0 = cfma(v[4 + t], h[t], r0);
+              }
+            r0 = cadd(r0, r1);
+            // lanes 0..15 sum the real parts, 16..31 the imaginary ones
+            const bool up = lane & 16;
+            T x = up ? r0.y : r0.x;
+            x += __shfl_xor_sync(0xffffffffu, up ? r0.x : r0.y, 16);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            const T xi = __shfl_sync(0xffffffffu, x, 16);
+            if (lane == 0) {
+              qv.x += x;
+              qv.y += xi;
+            }
+            // (lanes without a point hold zeros throughout)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+              if (j < np) {
+                const C lo = cscale(v[2 * j], w[(4 * j) * n]), hi = cscale(v[2 * j + 1], w[(4 * j + 1) * n]);
+                qv = pair_sum(conj_bit(Es[j], isx ? 0u : 0x80000000u), lo, hi, qv);
+                // X: a lo - conj(a) hi;  Y: conj(a) lo - a hi = a (-hi) - conj(a) (-lo)
+                grad_pair(j, u, isx ? lo : cneg(hi), isx ? hi : cneg(lo));
+              }
+            const C z = cmul(u, b1);
+            const double sg = isx ? 1.0 : -1.0;
+            dcs.x += sg * (double)z.x;
+            dcs.y += sg * (double)z.y;
+          }
+          if (nt) {  // Re sum u b dD/dtheta of the parameters on diagonal terms
+            const C z = cmul(u, b1);
+#pragma unroll
+            for (int t = 0; t < BQ_GRID_MAXT; ++t)
+              if (t < nt) grad_add(gt[t], z.x, w[(4 * np + ns + 2 * t) * n], -z.y, w[(4 * np + ns + 2 * t + 1) * n]);
+          }
+          a1 = cadd(a1, qv);  // (the step's sum starts as lam)
+          if (stage > 1) {
+            b1 = caxpy(stage == 4 ? hh : h2, qv, cscale(l1, stage == 2 ? w6 : w3));
+          } else {
+            l1 = a1;
+            b1 = cscale(a1, w6);
+          }
+          if (xi1 >= 0 && (it > 0 || stage > 1)) slot_put(out, slots, xi1, b1, no + 1);
+        }
+      } else {
 #pragma unroll 1
       for (int q = warp; q < cta.n; q += nw) {
         const GridPiece& g = S.pc[q];
         const int kind = g.kind, len = g.len;
+        const unsigned int any = (unsigned int)g.pad;
         const int pi = 32 * q + lane;
         const T* w = S.w + pi;
         const int* off = S.off + pi;
@@ -588,41 +962,36 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
         const C u = ok ? U[xidx(g)] : zero;
         C qv = cmul(S.dg[pi], b);
         if (kind == GRID_R) {
-          C nb[4 * NP], sv[NS];
-#pragma unroll
-          for (int j = 0; j < 4 * NP; ++j)
-            if (j < 4 * np) nb[j] = ld_cg(in + off[j * n]);
-          unsigned any = 0u;
-#pragma unroll
-          for (int s = 0; s < NS; ++s) {
-            if (s >= ns) break;
-            if (__any_sync(0xffffffffu, w[(4 * np + s) * n] != (T)0)) {
-              any |= 1u << s;
-              sv[s] = ld_cg(in + off[(4 * np + s) * n]);
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < NP; ++j) {
-            if (j >= np) break;
+          C sv[4];
+          auto pair = [&](int j, C n0, C n1, C n2, C n3) {
             const T w0 = w[(4 * j) * n], w1 = w[(4 * j + 1) * n], w2 = w[(4 * j + 2) * n], w3_ = w[(4 * j + 3) * n];
             C a, c;
-            a.x = fma(w0, nb[4 * j].x, -w3_ * nb[4 * j + 3].x);
-            a.y = fma(w0, nb[4 * j].y, -w3_ * nb[4 * j + 3].y);
-            c.x = fma(w1, nb[4 * j + 1].x, -w2 * nb[4 * j + 2].x);
-            c.y = fma(w1, nb[4 * j + 1].y, -w2 * nb[4 * j + 2].y);
+            a.x = fma(w0, n0.x, -w3_ * n3.x);
+            a.y = fma(w0, n0.y, -w3_ * n3.y);
+            c.x = fma(w1, n1.x, -w2 * n2.x);
+            c.y = fma(w1, n1.y, -w2 * n2.y);
             qv = pair_sum(Es[j], a, c, qv);
-            if (P.gpar[j] >= 0 || P.gpwc[j] >= 0) {
-              grad_add(ga[j], u, a);
-              grad_add(gb[j], u, c);
-            }
-          }
+            grad_pair(j, u, a, c);
+          };
+#pragma unroll 1
+            for (int j0 = 0; j0 < np; j0 += 2) {
+              const int m = min(2, np - j0);
+              C v[8];
+              slots_wait<8>(in, slots, [&](int i) { return off[(4 * j0 + i) * n]; }, (1u << (4 * m)) - 1u, no, v, A.error, &dead);
 #pragma unroll
-          for (int s = 0; s < NS; ++s) {
-            if (s >= ns) break;
-            if (any >> s & 1) qv = caxpy(w[(4 * np + s) * n], sv[s], qv);
-          }
+              for (int i = 0; i < 2; ++i)
+                if (i < m) pair(j0 + i, v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            }
+            slots_wait<4>(in, slots, [&](int i) { return off[(4 * np + i) * n]; }, any, no, sv, A.error, &dead);
+#pragma unroll
+          for (int s = 0; s < 4; ++s)
+            if (any >> s & 1u) qv = caxpy(w[(4 * np + s) * n], sv[s], qv);
         } else if (kind == GRID_D) {
-          for (int s = 0; s < ns; ++s) qv = caxpy(w[(4 * np + s) * n], ld_cg(in + off[(4 * np + s) * n]), qv);
+          C sv[4];
+          slots_wait<4>(in, slots, [&](int i) { return off[(4 * np + i) * n]; }, any, no, sv, A.error, &dead);
+#pragma unroll
+          for (int s = 0; s < 4; ++s)
+            if (any >> s & 1u) qv = caxpy(w[(4 * np + s) * n], sv[s], qv);
         } else {
           // points of G, BQ_GRID_GLEN per piece, the whole warp on each: the transposed source's
           // sum over a row (G_x) or column (G_y) of b_R, then the point's own lane the rest
@@ -640,19 +1009,32 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
               const C* go = U + (isx ? g.off_gy : g.off_gx) + P.ss[s];
               C v = zero;
               if (P.r_diag) {
-                if (lane == 0 && wo[kk] != (T)0) v = cmul(ld_cg(in + g.off_r + kk), cscale(go[kk], wo[kk]));
+                const T wj = lane == 0 ? wo[kk] : (T)0;  // (the whole warp calls slots_wait)
+                C x[1];
+                slots_wait<1>(in, slots, [&](int) { return g.off_r + kk; }, wj != (T)0 ? 1u : 0u, no, x, A.error, &dead);
+                if (wj != (T)0) v = cmul(x[0], cscale(go[kk], wj));
               } else {
-                const C* br = in + g.off_r + (isx ? kk * ng : kk);
-                const int st = isx ? 1 : ng;
                 const int mk = P.sst[s] ? (kk / P.sst[s]) % P.sM[s] : 0;
-                for (int j = lane; j < ng; j += 32) {
-                  const T wj = wo[j];
-                  if (wj == (T)0 || (P.sst[s] && (j / P.sst[s]) % P.sM[s] != mk)) continue;
-                  v = cfma(ld_cg(br + j * st), cscale(go[j], wj), v);
+                const int br = g.off_r + (isx ? kk * ng : kk), st = isx ? 1 : ng;
+#pragma unroll 1
+                for (int jb = 0; jb < ng; jb += 192) {
+                  const int j0 = jb + lane;
+                  unsigned int on = 0u;
+                  C x[6];
+#pragma unroll
+                  for (int i = 0; i < 6; ++i) {
+                    const int j = j0 + 32 * i;
+                    if (j < ng && wo[j] != (T)0 && !(P.sst[s] && (j / P.sst[s]) % P.sM[s] != mk)) on |= 1u << i;
+                  }
+                  slots_wait<6>(in, slots, [&](int i) { return br + (j0 + 32 * i) * st; }, on, no, x, A.error, &dead);
+#pragma unroll
+                  for (int i = 0; i < 6; ++i)
+                    if (on >> i & 1u) v = cfma(x[i], cscale(go[j0 + 32 * i], wo[j0 + 32 * i]), v);
                 }
               }
               src = caxpy(wt, v, src);
             }
+            __syncwarp();
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
               src.x += __shfl_xor_sync(0xffffffffu, src.x, o);
@@ -661,33 +1043,37 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
             if (lane == gi) mine = src;
           }
           qv = cadd(qv, mine);
-          if (ok) {
+#pragma unroll 1
+          for (int j0 = 0; j0 < np; j0 += 2) {
+            const int m = min(2, np - j0);
+            C v[4];
+            slots_wait<4>(in, slots, [&](int i) { return off[(4 * (j0 + i / 2) + (i & 1)) * n]; },
+                          ok ? (1u << (2 * m)) - 1u : 0u, no, v, A.error, &dead);
+            if (ok) {
 #pragma unroll
-            for (int j = 0; j < NP; ++j) {
-              if (j >= np) break;
-              const C lo = cscale(ld_cg(in + off[(4 * j) * n]), w[(4 * j) * n]);
-              const C hi = cscale(ld_cg(in + off[(4 * j + 1) * n]), w[(4 * j + 1) * n]);
-              qv = pair_sum(conj_bit(Es[j], isx ? 0u : 0x80000000u), lo, hi, qv);
-              if (P.gpar[j] >= 0 || P.gpwc[j] >= 0) {
+              for (int i = 0; i < 2; ++i) {
+                if (i >= m) break;
+                const int j = j0 + i;
+                const C lo = cscale(v[2 * i], w[(4 * j) * n]), hi = cscale(v[2 * i + 1], w[(4 * j + 1) * n]);
+                qv = pair_sum(conj_bit(Es[j], isx ? 0u : 0x80000000u), lo, hi, qv);
                 // X: a lo - conj(a) hi;  Y: conj(a) lo - a hi = a (-hi) - conj(a) (-lo)
-                const C pa = isx ? lo : cneg(hi), pb = isx ? hi : cneg(lo);
-                grad_add(ga[j], u, pa);
-                grad_add(gb[j], u, pb);
+                grad_pair(j, u, isx ? lo : cneg(hi), isx ? hi : cneg(lo));
               }
             }
+          }
+          if (ok) {
             const C z = cmul(u, b);
             const double sg = isx ? 1.0 : -1.0;
             dcs.x += sg * (double)z.x;
             dcs.y += sg * (double)z.y;
           }
+          __syncwarp();
         }
         if (nt) {  // Re sum u b dD/dtheta of the parameters on diagonal terms
           const C z = cmul(u, b);
-          for (int t = 0; t < BQ_GRID_MAXT; ++t) {
-            if (t >= nt) break;
-            const T hx = w[(4 * np + ns + 2 * t) * n], hy = w[(4 * np + ns + 2 * t + 1) * n];
-            gt[t] += (double)(z.x * hx - z.y * hy);
-          }
+#pragma unroll
+          for (int t = 0; t < BQ_GRID_MAXT; ++t)
+            if (t < nt) grad_add(gt[t], z.x, w[(4 * np + ns + 2 * t) * n], -z.y, w[(4 * np + ns + 2 * t + 1) * n]);
         }
         if (ok) {
           const C lv = S.v0[pi];
@@ -701,12 +1087,12 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
             bn = cscale(av, w6);
           }
           S.v3[pi] = bn;
-          out[xidx(g)] = bn;
+          if (it > 0 || stage > 1) slot_put(out, slots, xidx(g), bn, no + 1);
         }
       }
-      // the eight steps below this batch, in its first step
-      if (stage == 4 && ((it & 7) == 7 || it == last) && it > 7 && warp == nw - 1)
-        grid_envelope<T>(A, P, E, (it & ~7LL) - 8, segs);
+      }
+      ++no;
+      in = out;
       // ---- parameter sums: reduced when a factor changes before the next stage, and at the end --
       bool flush = it == 0 && stage == 1;
       for (int j = 0; j < np && !flush; ++j) {
@@ -725,23 +1111,24 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
           if (j >= np) break;
-          const double x0 = sum(ga[j].x), x1 = sum(ga[j].y), x2 = sum(gb[j].x), x3 = sum(gb[j].y);
+          const double x = sum(gx[j]), y = sum(gy[j]);
           if (lane == 0) {
-            red[warp][4 * j] = x0; red[warp][4 * j + 1] = x1; red[warp][4 * j + 2] = x2; red[warp][4 * j + 3] = x3;
+            red[warp][2 * j] = x;
+            red[warp][2 * j + 1] = y;
           }
-          ga[j] = gb[j] = make_double2(0.0, 0.0);
+          gx[j] = gy[j] = 0.0;
         }
 #pragma unroll
         for (int t = 0; t < BQ_GRID_MAXT; ++t) {
           const double x = sum(gt[t]);
-          if (lane == 0) red[warp][4 * NP + t] = x;
+          if (lane == 0) red[warp][2 * NP + t] = x;
           gt[t] = 0.0;
         }
         {
           const double x = sum(dcs.x), y = sum(dcs.y);
           if (lane == 0) {
-            red[warp][4 * NP + BQ_GRID_MAXT] = x;
-            red[warp][4 * NP + BQ_GRID_MAXT + 1] = y;
+            red[warp][2 * NP + BQ_GRID_MAXT] = x;
+            red[warp][2 * NP + BQ_GRID_MAXT + 1] = y;
           }
           dcs = make_double2(0.0, 0.0);
         }
@@ -753,7 +1140,7 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
         };
         if (tid < np && (P.gpar[tid] >= 0 || P.gpwc[tid] >= 0)) {
           const int j = tid;
-          const double2 sa = make_double2(col(4 * j), col(4 * j + 1)), sb = make_double2(col(4 * j + 2), col(4 * j + 3));
+          const double x = col(2 * j), y = col(2 * j + 1);
           double2 e = make_double2(1.0, 0.0);
           if (P.ch[j] >= 0) {
             const double tau = A.tau0 + (double)(A.step0 + it) * A.dt;
@@ -764,9 +1151,7 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
             if (P.cj[j]) e.y = -e.y;
           }
           // d Re(da S_a - conj(da) S_b) for a coefficient derivative da
-          auto dre = [&](double2 da) {
-            return da.x * sa.x - da.y * sa.y - (da.x * sb.x + da.y * sb.y);
-          };
+          auto dre = [&](double2 da) { return da.x * x - da.y * y; };
           if (P.gpar[j] >= 0) atomicAdd(A.grad + P.gpar[j], dre(cmul(make_double2(P.cb_re[j], P.cb_im[j]), e)));
           if (P.gpwc[j] >= 0) {
             const int sg = seg_of(it, j);
@@ -778,23 +1163,23 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
             }
           }
         }
-        if (tid >= 32 && tid < 32 + nt) atomicAdd(A.grad + P.tpar[tid - 32], col(4 * NP + tid - 32));
+        if (tid >= 32 && tid < 32 + nt) atomicAdd(A.grad + P.tpar[tid - 32], col(2 * NP + tid - 32));
         __syncthreads();
         // the separation constant's dependence on the parameters (an adjoint CTA holds one system)
         if (P.has_sep) {
-          const double x = col(4 * NP + BQ_GRID_MAXT), y = col(4 * NP + BQ_GRID_MAXT + 1);
-          for (int i = tid; i < P.n_params; i += BQ_GRID_THREADS) {
+          const double x = col(2 * NP + BQ_GRID_MAXT), y = col(2 * NP + BQ_GRID_MAXT + 1);
+          for (int i = tid; i < P.n_params; i += THREADS) {
             const double2 v = A.dc[S.pc[0].dc_off + i];
             if (v.x != 0.0 || v.y != 0.0) atomicAdd(A.grad + P.grad_off + i, v.x * x - v.y * y);
           }
         }
         __syncthreads();
       }
-      if (!(it == 0 && stage == 1)) {
-        if (!grid_sync(A.bar, ++epoch, A.error)) return;
-      }
     }
   }
+  __syncthreads();
+  if (*(volatile int*)&dead) return;
+  if (ONE && warp < cta.n) S.v0[32 * warp + lane] = l1;
   for (int q = warp; q < cta.n; q += nw) {
     const GridPiece& g = S.pc[q];
     if (lane < g.len) reinterpret_cast<C*>(A.lam)[xidx(g)] = S.v0[32 * q + lane];
@@ -802,23 +1187,26 @@ __global__ void __launch_bounds__(BQ_GRID_THREADS, 1) k_grid_adj(const GridArgs 
 }
 
 template <typename T>
-static const void* grid_func_t(int np, int ns, bool adj) {
-#define BQ_GRID_PICK(NPX, NSX) (adj ? (const void*)k_grid_adj<T, NPX, NSX> : (const void*)k_grid_fwd<T, NPX, NSX>)
-  if (np <= 2) return ns <= 2 ? BQ_GRID_PICK(2, 2) : BQ_GRID_PICK(2, 4);
-  if (np <= 4) return BQ_GRID_PICK(4, 4);
-  return np <= BQ_GRID_MAXP && !adj ? (const void*)k_grid_fwd<T, 8, 4> : nullptr;
-#undef BQ_GRID_PICK
+static const void* grid_func_t(int np, int ns, bool adj, int form) {
+  if (adj) {
+    if (form == GRID_ONE) return (const void*)k_grid_adj<T, 2, 256, true>;
+    if (np <= 2) return form == GRID_FEW ? (const void*)k_grid_adj<T, 2, 256, false> : (const void*)k_grid_adj<T, 2, 512, false>;
+    if (np <= 4) return form == GRID_FEW ? (const void*)k_grid_adj<T, 4, 256, false> : (const void*)k_grid_adj<T, 4, 512, false>;
+    return nullptr;
+  }
+  if (form == GRID_ONE) return (const void*)k_grid_fwd<T, true, 256>;
+  return form == GRID_FEW ? (const void*)k_grid_fwd<T, false, 256> : (const void*)k_grid_fwd<T, false, 512>;
 }
 
-static cudaError_t launch_grid_any(const void* f, const GridArgs& a, int ctas, int smem_bytes, cudaStream_t s) {
+static cudaError_t launch_grid_any(const void* f, const GridArgs& a, int ctas, int form, int smem_bytes, cudaStream_t s) {
   if (!f || ctas < 1) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, BQ_GRID_SMEM_MAX);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(a.bar, 0, sizeof(unsigned int), s);
+  e = cudaMemsetAsync(a.bar, 0, BQ_GRID_BAR_WORDS * sizeof(unsigned int), s);
   if (e != cudaSuccess) return e;
   GridArgs p = a;
   void* args[] = {(void*)&p};
-  return cudaLaunchCooperativeKernel(f, dim3(ctas), dim3(BQ_GRID_THREADS), args, (size_t)smem_bytes, s);
+  return cudaLaunchCooperativeKernel(f, dim3(ctas), dim3(grid_threads(form)), args, (size_t)smem_bytes, s);
 }
 
 }  // namespace bq

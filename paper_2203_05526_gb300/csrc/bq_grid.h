@@ -6,12 +6,13 @@
 
 #include "bq_internal.h"
 
-#define BQ_GRID_THREADS 256
 #define BQ_GRID_MAX_CTAS 256
 #define BQ_GRID_MAXP 8   // off-diagonal pairs of a problem
 #define BQ_GRID_MAXS 4   // sandwich terms
 #define BQ_GRID_MAXT 4   // parameters that multiply diagonal terms
 #define BQ_GRID_SMEM_MAX (200 * 1024)
+#define BQ_GRID_ROWS 10   // row values a lane of an adjoint piece of G may need (GRID_ONE)
+#define BQ_GRID_BAR_WORDS 5
 #define BQ_GRID_GLEN 1   // G points of an adjoint piece
 
 namespace bq {
@@ -60,11 +61,11 @@ struct GridArgs {
   const double* chpar;
   void* y;
   void* comp;
-  void* ua;       // stage inputs 1 and 3; adjoint: b of stages 4 and 2
-  void* ub;       // stage inputs 2 and 4; adjoint: b of stages 3 and 1
+  void* ring;     // exchange of stage inputs (adjoint: of b): ring_places x 2 arr bytes
+  int ring_places, block;  // places; steps (a power of two) between the CTAs' block counts
   char* rec;      // recorded stage inputs (4 per step) or null
   size_t arr;     // bytes of one state array
-  unsigned int* bar;    // the barrier's counter, zeroed before the launch
+  unsigned int* bar;    // BQ_GRID_BAR_WORDS counters, zeroed before the launch
   unsigned int* error;  // bit 2 is set when a barrier wait gives up
   void* lam;      // adjoint: cotangent of the state, in and out
   double* grad;
@@ -76,16 +77,25 @@ struct GridArgs {
 };
 
 // Largest grid whose CTAs are all resident (0: no cooperative launch), and the launches.
-cudaError_t grid_max_ctas(int dtype, int np, int ns, bool adj, int smem_bytes, int* out);
-cudaError_t launch_grid_f32(const GridArgs& a, int np, int ns, bool adj, int ctas, int smem_bytes, cudaStream_t s);
-cudaError_t launch_grid_f64(const GridArgs& a, int np, int ns, bool adj, int ctas, int smem_bytes, cudaStream_t s);
-const void* grid_func_f32(int np, int ns, bool adj);
-const void* grid_func_f64(int np, int ns, bool adj);
+cudaError_t grid_max_ctas(int dtype, int np, int ns, bool adj, int form, int smem_bytes, int* out);
+cudaError_t launch_grid_f32(const GridArgs& a, int np, int ns, bool adj, int ctas, int form, int smem_bytes, cudaStream_t s);
+cudaError_t launch_grid_f64(const GridArgs& a, int np, int ns, bool adj, int ctas, int form, int smem_bytes, cudaStream_t s);
+const void* grid_func_f32(int np, int ns, bool adj, int form);
+const void* grid_func_f64(int np, int ns, bool adj, int form);
+
+// Forms of the kernels, by the largest number n of pieces in a CTA: a piece per warp in registers (small
+// problems), eight warps, sixteen warps.
+enum GridForm : int { GRID_ONE = 0, GRID_FEW = 1, GRID_MANY = 2 };
+inline int grid_threads(int form) { return form == GRID_MANY ? 512 : 256; }
+// Whether a problem is small enough for GRID_ONE.
+inline bool grid_small(const GridProb& p, bool adj) {
+  return p.np <= 2 && p.ns <= 2 && (!adj || !p.has_r || p.r_diag || p.ns * ((p.ng + 31) / 32) <= BQ_GRID_ROWS);
+}
 
 // Dynamic shared memory of a CTA with n pieces (cs: complex size): per point five complex values,
 // the weights, the offsets and a flag word; envelopes; in the adjoint the sandwich tables.
-inline size_t grid_smem(int n, const GridProb& p, bool adj, size_t cs) {
-  const int nw = 4 * p.np + p.ns + (adj ? 2 * p.nt : 0), no = 4 * p.np + (adj ? 1 : 3) * p.ns;
+inline size_t grid_smem(int n, const GridProb& p, bool adj, int form, size_t cs) {
+  const int nw = 4 * p.np + p.ns + (adj ? 2 * p.nt + (form == GRID_ONE ? BQ_GRID_ROWS : 0) : 0), no = 4 * p.np + (adj ? 1 : 3) * p.ns;
   return (size_t)n * sizeof(GridPiece) + (size_t)n * 32 * (5 * cs + nw * (cs / 2) + (no + 1) * 4) +
          (size_t)2 * 32 * BQ_GRID_MAXP * cs + (adj ? (size_t)2 * p.ns * p.ng * (cs / 2) : 0) + 16;
 }

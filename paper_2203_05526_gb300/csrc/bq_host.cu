@@ -744,7 +744,7 @@ static int compile_problem(const bq_problem* p, const bq_map_opts& o, Compiled& 
 // State.
 // ---------------------------------------------------------------------------------------
 struct Layout {
-  size_t off_sys, off_terms, off_chans, off_chpar, off_work, off_m1, off_order, off_dc, off_pparams, off_precs, off_obs, off_rparams, off_rgroups, off_rbins, off_rflags, off_gprobs, off_gtab, off_gpieces, off_gctas, off_gbar, off_groups, off_entries, off_out, off_wtab, off_diag,
+  size_t off_sys, off_terms, off_chans, off_chpar, off_work, off_m1, off_order, off_dc, off_pparams, off_precs, off_obs, off_rparams, off_rgroups, off_rbins, off_rflags, off_gprobs, off_gtab, off_gpieces, off_gctas, off_gbar, off_gring, off_groups, off_entries, off_out, off_wtab, off_diag,
       off_ctrl, off_init, off_y, off_comp, off_ua, off_ub, off_acc, total;
 };
 
@@ -758,7 +758,7 @@ struct ResList {
 
 // A launch of the grid-resident kernels: CTAs [c0, c0 + n_ctas), none where the list does not fit.
 struct GridList {
-  int c0 = 0, n_ctas = 0, smem = 0;
+  int c0 = 0, n_ctas = 0, form = 0, smem = 0;
 };
 
 struct bq_state {
@@ -784,6 +784,7 @@ struct bq_state {
   // grid-resident kernels: lists (forward Hermitian, forward general, adjoint) and variant sizes
   GridList glist[3];
   int grid_np = 0, grid_ns = 0, grid_herm = 0;
+  int grid_few = 0;  // single-mode: bq_step and bq_solve take the grid-resident kernel
   int grid_pieces = 0, grid_adj = 0;  // pieces in the pool so far; the adjoint's list has been built
   std::vector<bq::GridProb> gprobs;
   // steps of equal length taken by the resident kernels since tau was run_tau0: their times are
@@ -874,7 +875,7 @@ struct Plan {
   std::vector<bq::ResBin> rbins;
   ResList rlist[3];
   // grid-resident kernels (k_grid_fwd, k_grid_adj): problems, tables, capacity of the lists' pieces
-  int grid_ok = 0, grid_np = 0, grid_ns = 0, grid_herm = 0;
+  int grid_ok = 0, grid_np = 0, grid_ns = 0, grid_herm = 0, grid_few = 0;
   size_t grid_cap = 0;
   std::vector<bq::GridProb> gprobs;
   std::vector<double> gtab;
@@ -1266,6 +1267,16 @@ static void make_res_plan(Plan& P, const bq_problem* const* probs, const std::ve
 // ---------------------------------------------------------------------------------------
 static const int kGridMaxCtas = BQ_GRID_MAX_CTAS;
 static const int64_t kGridMaxPoints = 152 * 2500;
+// Few single-mode systems in FP64 take the grid-resident kernel: the resident kernel keeps a system on
+// one SM, whose FP64 pipe then takes longer for a stage than the exchange between SMs does.  Measured
+// (us per step, resident / grid): one system N = 16 10.0 / 8.8, N = 20 10.8 / 9.0, N = 40 34.9 / 9.7;
+// 4 systems N = 12 20.9 / 8.9, N = 40 33.3 / 9.0; 64 systems N = 12 26.1 / 9.1, N = 40 34.9 / 12.7
+// (growing with the number from there; the resident kernel's 35 hold up to two systems per SM).
+static const int kGridFewSystems = 128;
+static const int kGridFewM = 20;  // of a single system: below, both are at their latencies
+// Steps between the block counts of the grid-resident kernels: two while the ring stays small
+// beside L2, one for larger states.
+static int grid_block(size_t arr) { return arr <= ((size_t)1 << 20) ? 2 : 1; }
 
 // X or Y term t's weights over the flat index of its side; S terms: of side y's dimensions.
 static std::vector<double> flat_weights(const Compiled& C, const TermDesc& td, int wbase, bool y) {
@@ -1461,7 +1472,7 @@ static size_t grid_count(const std::vector<SysDesc>& sys, const std::vector<bq::
   return n;
 }
 
-static void make_grid_plan(Plan& P, const bq_problem* const* probs) {
+static void make_grid_plan(Plan& P, const bq_problem* const* probs, const bq_map_opts& o) {
   const int B = (int)P.comp.size();
   int64_t pts = 0;
   for (const SysDesc& sd : P.sys) pts += sd.n_r + 2 * (sd.has_sep ? sd.n_g : 0);
@@ -1494,6 +1505,9 @@ static void make_grid_plan(Plan& P, const bq_problem* const* probs) {
   }
   for (int list = P.grid_herm ? 0 : 1; list < 3; ++list) P.grid_cap += grid_count(P.sys, P.gprobs, list);
   P.grid_ok = 1;
+  int m = 0;
+  for (const bq::GridProb& g : P.gprobs) m = std::max(m, g.ng);
+  P.grid_few = P.res_ok && o.dtype == BQ_F64 && B <= kGridFewSystems && (B > 1 || m >= kGridFewM);
 }
 
 // The pieces of a list (0: forward, Hermitian layout where possible; 1: forward, general layout; 2:
@@ -1548,13 +1562,17 @@ static int build_grid_list(const std::vector<SysDesc>& sys, const std::vector<bq
       ctas.push_back(cta);
     }
   }
+  int form = share <= 8 ? bq::GRID_ONE : bq::GRID_MANY;
+  for (const bq::GridProb& g : probs)
+    if (form == bq::GRID_ONE && !bq::grid_small(g, list == 2)) form = bq::GRID_FEW;
   size_t sm = 0;
-  for (const bq::GridProb& g : probs) sm = std::max(sm, bq::grid_smem(share, g, list == 2, dtype == BQ_F64 ? 16 : 8));
+  for (const bq::GridProb& g : probs) sm = std::max(sm, bq::grid_smem(share, g, list == 2, form, dtype == BQ_F64 ? 16 : 8));
   int most = 0;
-  if (sm <= BQ_GRID_SMEM_MAX) CUDA_TRY(bq::grid_max_ctas(dtype, np, ns, list == 2, (int)sm, &most));
+  if (sm <= BQ_GRID_SMEM_MAX) CUDA_TRY(bq::grid_max_ctas(dtype, np, ns, list == 2, form, (int)sm, &most));
   if (most < (int)ctas.size()) return BQ_OK;
   gl.n_ctas = (int)ctas.size();
   gl.smem = (int)sm;
+  gl.form = form;
   return BQ_OK;
 }
 
@@ -1959,7 +1977,7 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
     }
   }
 
-  make_grid_plan(P, probs);
+  make_grid_plan(P, probs, *o);
 
   // ---- work items (tiles of R; the first tile of a system also updates G_x, G_y) ------
   for (SysDesc& sd : P.sys) {
@@ -2018,7 +2036,8 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
   L.off_gtab = seg(P.gtab.size() * rs);
   L.off_gpieces = seg(P.grid_cap * sizeof(bq::GridPiece));
   L.off_gctas = seg(P.grid_ok ? 3 * kGridMaxCtas * sizeof(bq::GridCta) : 0);
-  L.off_gbar = seg(P.grid_ok ? sizeof(unsigned int) : 0);
+  L.off_gbar = seg(P.grid_ok ? BQ_GRID_BAR_WORDS * sizeof(unsigned int) : 0);
+  L.off_gring = seg(P.grid_ok ? 2 * (size_t)P.total_elems * cs * (8 * grid_block((size_t)P.total_elems * cs) + 1) : 0);
   L.off_dc = seg(P.dc.size() * sizeof(double2));
   L.off_groups = seg(P.groups.size() * sizeof(EvalGroup));
   L.off_entries = seg(P.entries.size() * sizeof(EvalEntry));
@@ -2150,7 +2169,7 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
   std::vector<bq::GridCta> gctas[2];
   int grid_pieces = 0;
   if (P.grid_ok) {
-    for (int q = P.use_m1 ? 2 : P.grid_herm ? 0 : 1; q < 2; ++q) {
+    for (int q = P.use_m1 && !P.grid_few ? 2 : P.grid_herm ? 0 : 1; q < 2; ++q) {
       r = build_grid_list(P.sys, P.gprobs, q, o->dtype, P.grid_np, P.grid_ns, gpieces[q], gctas[q], glist[q]);
       if (r != BQ_OK) return r;
       for (bq::GridCta& c : gctas[q]) c.p0 += grid_pieces;
@@ -2224,6 +2243,7 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
   st->grid_np = P.grid_np;
   st->grid_ns = P.grid_ns;
   st->grid_herm = P.grid_herm;
+  st->grid_few = P.grid_few && glist[1].n_ctas > 0 && (!P.grid_herm || glist[0].n_ctas > 0);
   st->grid_pieces = grid_pieces;
   st->gprobs = P.gprobs;
   if (!P.use_m1 && glist[1].n_ctas > 0) st->res_on = 1;
@@ -2390,9 +2410,10 @@ static bq::GridArgs grid_args(bq_state* s, int q, double dt) {
   a.chpar = (const double*)(b + L.off_chpar);
   a.y = b + L.off_y;
   a.comp = b + L.off_comp;
-  a.ua = b + L.off_ua;
-  a.ub = b + L.off_ub;
   a.arr = (size_t)s->total_elems * (s->dtype == BQ_F64 ? 16 : 8);
+  a.ring = b + L.off_gring;
+  a.block = grid_block(a.arr);
+  a.ring_places = 8 * a.block + 1;
   a.bar = (unsigned int*)(b + L.off_gbar);
   a.error = (unsigned int*)(b + L.off_ctrl + 32);
   a.dc = (const double2*)(b + L.off_dc);
@@ -2404,14 +2425,14 @@ static bq::GridArgs grid_args(bq_state* s, int q, double dt) {
 }
 static cudaError_t launch_grid(bq_state* s, const bq::GridArgs& a, int q, cudaStream_t st) {
   const auto launch = s->dtype == BQ_F64 ? bq::launch_grid_f64 : bq::launch_grid_f32;
-  return launch(a, s->grid_np, s->grid_ns, q == 2, s->glist[q].n_ctas, s->glist[q].smem, st);
+  return launch(a, s->grid_np, s->grid_ns, q == 2, s->glist[q].n_ctas, s->glist[q].form, s->glist[q].smem, st);
 }
 
 // Builds and uploads the lists bq_grad needs, at its first call: the adjoint's, and in single-mode
 // states (whose steps take other kernels) the forward one.
 static int ensure_grid_adjoint(bq_state* s) {
   if (s->grid_adj || s->gprobs.empty()) return BQ_OK;
-  for (int q = s->use_m1 ? 1 : 2; q < 3; ++q) {
+  for (int q = s->use_m1 && s->glist[1].n_ctas == 0 ? 1 : 2; q < 3; ++q) {
     if (q == 2 && s->glist[1].n_ctas == 0) break;
     std::vector<bq::GridPiece> pieces;
     std::vector<bq::GridCta> ctas;
@@ -2437,7 +2458,10 @@ static int ensure_grid_adjoint(bq_state* s) {
 static cudaError_t enqueue_grid(bq_state* s, double dt, int64_t n, cudaStream_t st, int* launches) {
   run_begin(s, dt);
   const int q = s->res_known && s->glist[0].n_ctas > 0 ? 0 : 1;
-  if (q == 1 && s->grid_herm) s->res_known = 0;  // (leaves Hermitian systems Hermitian to rounding)
+  if (q == 1 && (s->grid_herm || s->use_m1)) {  // (leaves Hermitian systems Hermitian to rounding)
+    s->res_known = 0;
+    s->res_dirty = 1;
+  }
   bq::GridArgs a = grid_args(s, q, dt);
   *launches = 0;
   const int64_t most = 1 << 24;  // steps per launch (32-bit step and barrier counters)
@@ -2463,6 +2487,7 @@ static bool res_on(const bq_state* s) { return s->res_ok && s->res_on && s->use_
 
 // n steps from s->tau with the resident kernel, one launch per non-empty list; advances s->tau.
 static cudaError_t enqueue_resident(bq_state* s, double dt, int64_t n, cudaStream_t st, int* launches) {
+  if (s->grid_few) return enqueue_grid(s, dt, n, st, launches);
   char* b = s->pool;
   const Layout& L = s->L;
   unsigned char* flags = (unsigned char*)(b + L.off_rflags);
@@ -3236,8 +3261,6 @@ extern "C" int bq_grad(bq_state* s, double dt, int64_t n_steps, int checkpoint_e
       }
       if (grid) {
         bq::GridArgs a = grid_args(s, 2, dt);
-        a.ua = w + G.ba;
-        a.ub = w + G.bb;
         a.rec = rec;
         a.lam = lam;
         a.grad = (double*)(w + G.grad);

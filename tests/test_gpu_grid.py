@@ -195,3 +195,29 @@ def test_other_forms_keep_the_tiled_kernels():
     # a time-dependent diagonal term, a jump operator of two monomials
     assert one(lambda p: p.h_terms.extend([HTerm(0.2, a, a, channel=0), HTerm(0.2, a, a, channel=0, conj=True)])) == 0
     assert one(lambda p: p.jumps.append(Jump(0.1, ((1.0 + 0j, z, a), (0.5 + 0j, z, z))))) == 0
+
+
+def test_independent_systems_drift_apart_without_losing_slots():
+    """125 systems that no exchange couples, many blocks of steps and several calls: CTAs run ahead of
+    one another as far as the slots' reuse lets them."""
+    p = configs.table_one_network(3, 6, steps=4000)
+    a, b = gpu_state(p, dtype="f64", r_layout="diag"), gpu_state(p, dtype="f64", r_layout="diag")
+    b.set_tune(resident=0)
+    for n in (61, 1, 2, 96):
+        a.step(p.dt, n)
+        b.step(p.dt, n)
+    _agree(a, b, "f64")
+
+
+@pytest.mark.parametrize("instances,N", [(1, 19), (1, 20), (1, 42), (2, 8), (31, 41), (128, 9), (129, 9)])
+def test_few_single_mode_systems(instances, N):
+    """FP64 single-mode states on both sides of the rule that sends few systems to the grid kernels."""
+    ps = [configs.kerr_driven(N=max(4, N - i % 3), dt=0.002, T=0.05, n_th=0.1 if i % 2 else 0.0) for i in range(instances)]
+    a, b = gpu_state(ps, dtype="f64"), gpu_state(ps, dtype="f64")
+    b.set_tune(resident=0)
+    for n in (1, 13):
+        a.step(ps[0].dt, n)
+        b.step(ps[0].dt, n)
+    a.solve(ps[0].dt, 5)
+    b.step(ps[0].dt, 5)
+    _agree(a, b, "f64")

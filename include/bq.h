@@ -178,16 +178,16 @@ int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* opts, void*
 /* Advances every system of the state by n_steps RK4 steps of size dt (the mapped value
  * of dt must not exceed the bound checked at bq_map).  Single-mode states of the resident form
  * (bq_tune resident): all n_steps in one launch, every system on chip.  Tiled states of that
- * form that fit the SMs' shared memory: all n_steps in one cooperative launch with a bounded grid
- * barrier per stage (one that waits longer than about 2 s sets the error word: BQ_ETIMEOUT from
- * the next synchronising call).  Else fused stage kernels: on the pipelined single-mode path the four stages of a step run in one launch
+ * form that fit the SMs' shared memory, and FP64 states of up to 128 single-mode systems: all
+ * n_steps in one cooperative launch that exchanges stage inputs through L2 (the waits are bounded:
+ * one longer than a few seconds sets the error word, BQ_ETIMEOUT from the next synchronising call).  Else fused stage kernels: on the pipelined single-mode path the four stages of a step run in one launch
  * (bq_tune pipe_fused), otherwise one launch per stage; replayed from a CUDA graph.
  * Asynchronous on stream. */
 int bq_step(bq_state* s, double dt, int64_t n_steps, void* stream);
 
 /* Batched persistent solve (one launch for all steps of all systems of the batch; the
  * paper's independent initial conditions, main text after Eq. 13, processed as a work
- * queue).  Single-mode states of the resident form run bq_step's resident kernel (bq_tune
+ * queue).  Single-mode states of the resident form run bq_step's kernel (bq_tune
  * resident); in the others every CTA takes systems from an atomic queue, largest first, and
  * keeps the system on chip for all n_steps steps (the RK4 stage buffers, stage sums and compensation
  * in shared memory, the state in registers).  The same arithmetic as bq_step (classical
@@ -247,8 +247,8 @@ typedef struct bq_tune {
   int resident;          /* 1 (the default where the state has the form they take): the resident
                           * kernels, all steps of a call in one launch with the state on chip,
                           * whatever the other schedule fields say: BQ_PATH_PIPE (one system per
-                          * group of warps; also BQ_SOLVE_MERGED with solve_ctas_per_sm = 0) and
-                          * BQ_PATH_TILED (the state spread over the SMs, one cooperative launch;
+                          * group of warps; few FP64 systems over all SMs; also BQ_SOLVE_MERGED
+                          * with solve_ctas_per_sm = 0) and BQ_PATH_TILED (the state spread over the SMs, one cooperative launch;
                           * also bq_grad's segments with grad_coop).  0 = the kernels that the
                           * other fields describe */
 } bq_tune;

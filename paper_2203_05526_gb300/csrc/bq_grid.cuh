@@ -14,11 +14,11 @@
 // to three times fewer FP64 operations than term by term.  Hermitian states (see
 // bq_resident.cuh for the layout) hold half the points.
 // Measured (one GB300, FP64, per RK4 step; one launch per stage / a grid barrier per stage / slots):
-// two modes at N = 12 45 / 20 / 11.0 us, three modes at N = 6 direct 183 / 68 / 32, mapped with R(xy)
-// (125 systems) 279 / 66 / 53; the 131-parameter control gradient 201 / 76 / 52; one oscillator at N =
-// 40, which the resident kernel keeps on one SM in 36 us, 10.  What bounds a stage now: small states
-// the chain store, L2, poll, arithmetic of one warp (2.2 us); large ones the FP64 pipe (one warp
-// instruction per 16 cycles and SM).
+// two modes at N = 12 45 / 20 / 9.8 us, three modes at N = 6 direct 183 / 68 / 28, mapped with R(xy)
+// (125 systems) 279 / 66 / 37; the 131-parameter control gradient 201 / 76 / 46; one oscillator at N =
+// 40, which the resident kernel keeps on one SM in 36 us, 9.  What bounds a stage now: small states
+// the chain store, L2, poll, arithmetic of one warp (about 2 us); large ones the FP64 pipe (one warp
+// instruction per 16 cycles and SM: 65% busy).
 #pragma once
 
 #include "bq_device.cuh"
@@ -27,10 +27,6 @@
 namespace bq {
 
 #define BQ_GRID_WAIT_CYCLES2 (4000000000LL)  // about 2 s at the maximum SM clock
-
-template <typename C> __device__ __forceinline__ C ld_cg(const C* p);
-template <> __device__ __forceinline__ float2 ld_cg<float2>(const float2* p) { return __ldcg(p); }
-template <> __device__ __forceinline__ double2 ld_cg<double2>(const double2* p) { return __ldcg(p); }
 
 // A launch's first grid barrier: one counter, zero before the launch, that every CTA adds one to; one
 // thread per CTA waits for all.  The wait is bounded; on timeout the error word is set and the caller
@@ -86,12 +82,16 @@ __device__ __forceinline__ double2 conj_bit(double2 v, unsigned m) {
   return v;
 }
 
+// x == 0 on the integer pipe.
+__device__ __forceinline__ bool zero_bits(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool zero_bits(float x) { return (__float_as_uint(x) << 1) == 0; }
+
 // a p - conj(a) q added to k; a purely imaginary a (uniform over the CTA) takes two
 // multiply-adds per component less.
 template <typename C>
 __device__ __forceinline__ C pair_sum(C a, C p, C q, C k) {
   const C s = cadd(p, q);
-  if (a.x == 0) {
+  if (zero_bits(a.x)) {
     k.x = fma(-a.y, s.y, k.x);
     k.y = fma(a.y, s.x, k.y);
   } else {
@@ -107,6 +107,8 @@ __device__ __forceinline__ C pair_sum(C a, C p, C q, C k) {
 // g += a b + c d, summed in FP64 (FP32 products are rounded to FP32 first, as in the other kernels).
 __device__ __forceinline__ void grad_add(double& g, double a, double b, double c, double d) { g = fma(a, b, fma(c, d, g)); }
 __device__ __forceinline__ void grad_add(double& g, float a, float b, float c, float d) { g += (double)fmaf(a, b, c * d); }
+__device__ __forceinline__ void grad_add(double& g, double a, double b) { g = fma(a, b, g); }
+__device__ __forceinline__ void grad_add(double& g, float a, float b) { g += (double)(a * b); }
 
 // Envelopes of the problem's pairs for the eight steps from s0 on (32 stages, one per lane), into
 // half (s0 / 8) & 1 of E[2][32][MAXP].
@@ -204,38 +206,37 @@ struct GridSlots {
 // its stage's number: no fence, no barrier, no flag between the writer's store and the reader's
 // load.  A grid barrier per stage took four dependent trips to L2 (fence, counter, poll, load),
 // this takes one and a half, and warps without a stage's last neighbours wait alone.
-// (slot_get returns zero if the slot carries the number.)  Slot i of a place: FP64 in two planes of n words (a warp's 16-byte accesses are then consecutive),
-// base the place's first word.
-__device__ __forceinline__ void slot_put(double2* base, size_t n, int i, double2 v, unsigned int no) {
-  double2* p = base + i;
+// Word of slot i in a place.  FP64: 32 slots' real words, then their imaginary words, so that a
+// warp's 16-byte accesses are consecutive (a slot's two words side by side took twice the sectors:
+// two modes 11.1 -> 12.9 us per step) and the second word is an immediate offset away.
+template <typename C> __device__ __forceinline__ int slot_of(int i) { return sizeof(C) == 16 ? (i >> 5 << 6) | (i & 31) : i; }
+__device__ __forceinline__ void slot_put(uint4* p, double2 v, unsigned int no) {
   asm volatile(
       "{\n.reg .b128 a, b;\nmov.b128 a, {%1, %3};\nmov.b128 b, {%2, %3};\n"
-      "st.relaxed.gpu.global.b128 [%0], a;\nst.relaxed.gpu.global.b128 [%4], b;\n}" ::"l"(p),
-      "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "l"((unsigned long long)no), "l"(p + n)
+      "st.relaxed.gpu.global.b128 [%0], a;\nst.relaxed.gpu.global.b128 [%0+512], b;\n}" ::"l"(p),
+      "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "l"((unsigned long long)no)
       : "memory");
 }
-__device__ __forceinline__ void slot_put(float2* base, size_t, int i, float2 v, unsigned int no) {
-  float2* p = base + 2 * (size_t)i;
+__device__ __forceinline__ void slot_put(uint4* p, float2 v, unsigned int no) {
   const unsigned long long w = (unsigned long long)__float_as_uint(v.y) << 32 | __float_as_uint(v.x);
   asm volatile("{\n.reg .b128 a;\nmov.b128 a, {%1, %2};\nst.relaxed.gpu.global.b128 [%0], a;\n}" ::"l"(p), "l"(w),
                "l"((unsigned long long)no)
                : "memory");
 }
-__device__ __forceinline__ unsigned int slot_get(const double2* base, size_t n, int i, unsigned int no, double2& v) {
-  const double2* p = base + i;
+// Zero if the slot carries the number.
+__device__ __forceinline__ unsigned int slot_get(const uint4* p, unsigned int no, double2& v) {
   unsigned long long x, y, n0, n1;
   asm volatile(
-      "{\n.reg .b128 a, b;\nld.relaxed.gpu.global.b128 a, [%4];\nld.relaxed.gpu.global.b128 b, [%5];\n"
+      "{\n.reg .b128 a, b;\nld.relaxed.gpu.global.b128 a, [%4];\nld.relaxed.gpu.global.b128 b, [%4+512];\n"
       "mov.b128 {%0, %1}, a;\nmov.b128 {%2, %3}, b;\n}"
       : "=l"(x), "=l"(n0), "=l"(y), "=l"(n1)
-      : "l"(p), "l"(p + n)
+      : "l"(p)
       : "memory");
   v.x = __longlong_as_double((long long)x);
   v.y = __longlong_as_double((long long)y);
   return ((unsigned int)n0 ^ no) | ((unsigned int)n1 ^ no);
 }
-__device__ __forceinline__ unsigned int slot_get(const float2* base, size_t, int i, unsigned int no, float2& v) {
-  const float2* p = base + 2 * (size_t)i;
+__device__ __forceinline__ unsigned int slot_get(const uint4* p, unsigned int no, float2& v) {
   unsigned long long w, n0;
   asm volatile("{\n.reg .b128 a;\nld.relaxed.gpu.global.b128 a, [%2];\nmov.b128 {%0, %1}, a;\n}"
                : "=l"(w), "=l"(n0)
@@ -246,31 +247,37 @@ __device__ __forceinline__ unsigned int slot_get(const float2* base, size_t, int
   return (unsigned int)n0 ^ no;
 }
 
-// off(j): program offset of value j (sign bit: conjugate); on: bit j set where value j is wanted (the
+// off(j): word of value j's slot; on: bit j set where value j is wanted (the
 // others come back zero).  The whole warp calls it and stays together in the loop: when lanes left it
 // one by one the arithmetic behind it was issued for several parts of the warp in turn (the FP64 pipe
 // 93% busy for 44% of useful lanes, three modes direct).  The wait is bounded: a thread that gives up
 // sets the error word and *dead, does not wait again, and the launch ends without storing.
 template <int N, typename C, typename F>
-__device__ __forceinline__ void slots_wait(const C* base, size_t n, F off, unsigned int on, unsigned int no, C (&v)[N],
+__device__ __forceinline__ void slots_wait(const uint4* base, F off, unsigned int on, unsigned int no, C (&v)[N],
                                            unsigned int* error, int* dead) {
 #pragma unroll
   for (int j = 0; j < N; ++j) v[j] = cmk<C>(0.0, 0.0);
-  long long t0 = 0;
-  for (;;) {
+  for (unsigned int tries = 1;; ++tries) {
     unsigned int bad = 0u;
 #pragma unroll
     for (int j = 0; j < N; ++j)
-      if (on >> j & 1u) bad |= slot_get(base, n, off(j) & 0x7fffffff, no, v[j]);
+      if (on >> j & 1u) bad |= slot_get(base + (unsigned)off(j), no, v[j]);
     if (!__any_sync(0xffffffffu, bad)) break;
-    if (!t0) t0 = clock64();
-    const bool stop = clock64() - t0 > BQ_GRID_WAIT_CYCLES2 || *(volatile int*)dead;
-    if (stop && bad) atomicOr(error, 4u);
-    if (__any_sync(0xffffffffu, stop)) {
-      *(volatile int*)dead = 1;
-      break;
+    if (!(tries & 1023u)) {  // (a try takes a trip to L2: 2^22 of them about 2 s)
+      const bool stop = tries >> 22;
+      if (stop && bad) atomicOr(error, 4u);
+      if (__any_sync(0xffffffffu, stop || *(volatile int*)dead)) {
+        *(volatile int*)dead = 1;
+        break;
+      }
     }
   }
+}
+// The same for program offsets with the conjugation in their sign bit.
+template <int N, typename C, typename F>
+__device__ __forceinline__ void slots_wait_conj(const uint4* base, F off, unsigned int on, unsigned int no, C (&v)[N],
+                                                unsigned int* error, int* dead) {
+  slots_wait<N>(base, [&](int j) { return off(j) & 0x7fffffff; }, on, no, v, error, dead);
 #pragma unroll
   for (int j = 0; j < N; ++j)
     if (on >> j & 1u) v[j] = conj_bit(v[j], (unsigned)off(j) & 0x80000000u);
@@ -302,13 +309,16 @@ __device__ __forceinline__ bool block_sync(unsigned int* bar, unsigned int h, un
   return __syncthreads_or(threadIdx.x == 0 && *(volatile int*)dead) == 0;
 }
 
-// SMALL (GRID_ONE): at most two pairs and two sandwich terms and a piece per warp: its state and its
-// neighbours' offsets stay in registers and every value comes in one batch of loads.  Else the
+// NPS > 0 (GRID_ONE): at most NPS pairs and NSS sandwich terms, a piece per warp: its state and its
+// neighbours' slots stay in registers and every value comes in one batch of loads without a branch
+// (a value that a point lacks is its own slot with a zero weight).  Else the
 // program is read from shared memory and the pairs go in batches of two or, with 256 threads (no
 // more than eight pieces a CTA, 255 registers), four.
-template <typename T, bool SMALL, int THREADS>
+template <typename T, int NPS, int NSS, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
   using C = typename C2T<T>::type;
+  constexpr bool SMALL = NPS > 0;
+  constexpr int NV = SMALL ? 4 * NPS + 3 * NSS : 1;  // values of a point
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ GridProb P;
   __shared__ int dead;
@@ -318,6 +328,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
   if (threadIdx.x == 0) dead = 0;
   __syncthreads();
   const int ng = P.ng, np = P.np, ns = P.ns;
+  // pairs with a static imaginary coefficient i b: b is part of the weights
+  unsigned int fold = 0u;
+  for (int j = 0; j < np; ++j)
+    if (P.ch[j] < 0 && P.a_re[j] == 0.0) fold |= 1u << j;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = THREADS / 32;
   const GridSlots<T> S(smem_raw, cta.n, 4 * np + ns, 4 * np + 3 * ns);
   const int n = S.n;
@@ -326,8 +340,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
   for (int i = tid; i < cta.n * (int)(sizeof(GridPiece) / 4); i += THREADS)
     reinterpret_cast<int*>(S.pc)[i] = reinterpret_cast<const int*>(A.pieces + cta.p0)[i];
   __syncthreads();
-  C* const ring = reinterpret_cast<C*>(A.ring);
-  const size_t slots = A.arr / sizeof(C), place = 2 * slots;  // of a place of the ring; its elements
+  uint4* const ring = reinterpret_cast<uint4*>(A.ring);
+  const size_t place = A.place;
+  const int places = (int)min((long long)A.ring_places, 4LL * A.n_steps + 1);  // that this launch uses  // of a place of the ring; its elements
   auto recorded = [&](long long i, int stage) { return reinterpret_cast<C*>(A.rec + ((size_t)i * 4 + stage - 1) * A.arr); };
   const int Pc = ng | 1;
   auto position = [&](const GridPiece& g) {
@@ -363,7 +378,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
     const int pi = 32 * q + lane, self = xidx(g);
     const bool ok = lane < g.len && p.k < ng && p.l < ng;
     const int si = lane < g.len ? self : xidx(g) - lane;  // (an address that exists)
-    for (int j = 0; j < 4 * np + 3 * ns; ++j) S.off[j * n + pi] = si;
+    for (int j = 0; j < 4 * np + 3 * ns; ++j) S.off[j * n + pi] = slot_of<C>(si);
     for (int j = 0; j < 4 * np + ns; ++j) S.w[j * n + pi] = (T)0;
     C yv = zero, cv = zero, dg = zero;
     if (ok) {
@@ -376,24 +391,25 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
       auto put = [&](int j, T w, int o, unsigned conj) {
         if (w == (T)0) return;
         S.w[j * n + pi] = w;
-        S.off[j * n + pi] = (int)((unsigned)o | conj);
+        S.off[j * n + pi] = (int)((unsigned)slot_of<C>(o) | conj);
       };
       for (int j = 0; j < np; ++j) {
         const int d = P.dlt[j];
+        const T f = !(fold >> j & 1u) ? (T)1 : (T)(g.kind == GRID_Y ? -P.a_im[j] : P.a_im[j]);
         unsigned c = 0u;
         if (g.kind <= GRID_H) {  // sources k - d, k + d, l - d, l + d
           int o = p.at(-d, 0, c);
-          put(4 * j, W.pair(j, 0)[p.k], g.off_r + o, c);
+          put(4 * j, f * W.pair(j, 0)[p.k], g.off_r + o, c);
           o = p.at(d, 0, c);
-          put(4 * j + 1, W.pair(j, 1)[p.k], g.off_r + o, c);
+          put(4 * j + 1, f * W.pair(j, 1)[p.k], g.off_r + o, c);
           o = p.at(0, -d, c);
-          put(4 * j + 2, W.pair(j, 2)[p.l], g.off_r + o, c);
+          put(4 * j + 2, f * W.pair(j, 2)[p.l], g.off_r + o, c);
           o = p.at(0, d, c);
-          put(4 * j + 3, W.pair(j, 3)[p.l], g.off_r + o, c);
+          put(4 * j + 3, f * W.pair(j, 3)[p.l], g.off_r + o, c);
         } else if (g.kind >= GRID_X) {
           const int x = g.kind == GRID_X ? 0 : 2;
-          put(4 * j, W.pair(j, x)[p.k], self - d, 0u);
-          put(4 * j + 1, W.pair(j, x + 1)[p.k], self + d, 0u);
+          put(4 * j, f * W.pair(j, x)[p.k], self - d, 0u);
+          put(4 * j + 1, f * W.pair(j, x + 1)[p.k], self + d, 0u);
         }
       }
       if (g.kind <= GRID_D)
@@ -405,9 +421,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
           unsigned c = 0u;
           const int o = g.kind == GRID_D ? p.k + d : p.at(d, d, c);
           put(4 * np + s, ww, g.off_r + o, c);
-          S.off[(4 * np + ns + s) * n + pi] = g.off_gx + p.k + d;
+          S.off[(4 * np + ns + s) * n + pi] = slot_of<C>(g.off_gx + p.k + d);
           S.off[(4 * np + 2 * ns + s) * n + pi] =
-              g.kind == GRID_H ? (int)((unsigned)(g.off_gx + p.l + d) | 0x80000000u) : g.off_gy + p.l + d;
+              g.kind == GRID_H ? (int)((unsigned)slot_of<C>(g.off_gx + p.l + d) | 0x80000000u) : slot_of<C>(g.off_gy + p.l + d);
         }
     }
     S.fl[pi] = (ok ? 1 : 0) | (g.kind == GRID_H && p.d == 0 ? 2 : 0);
@@ -422,9 +438,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
       if (lane == 0) S.pc[q].pad = (int)any;
     }
     if (lane < g.len) {
-      for (int r = 0; r < A.ring_places; ++r)
-        if (r != 1) slot_put(ring + r * place, slots, self, zero, 0u);
-      slot_put(ring + place, slots, self, yv, 1u);
+      for (int r = 0; r < places; ++r)
+        if (r != 1) slot_put(ring + r * place + slot_of<C>(self), zero, 0u);
+      slot_put(ring + place + slot_of<C>(self), yv, 1u);
       if (A.rec) recorded(0, 1)[self] = yv;
     }
   }
@@ -436,7 +452,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
   const double wd = A.dt / 6.0;
   const T w_hi = (T)wd, w_lo = (T)(wd - (double)w_hi);
   unsigned int no = 1;       // number and place of the stage's input
-  const C* in = ring + place;
+  const uint4* in = ring + place;
   int turn = 1;
   // the state after a step: y + (sum + k) dt / 6 with its rounding error carried along
   auto update = [&](C sum, C k, C yv, C& cv) {
@@ -457,24 +473,49 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
     }
     return nu;
   };
-  // SMALL: a warp's one piece, its offsets, state, sum and compensation in registers
-  int of[SMALL ? 14 : 1];
-  unsigned int on = 0u;
+  // a pair's contribution to k: values n0..n3 with weights w0..w3, coefficient a
+  auto pair_term = [&](bool folded, C a, T w0, T w1, T w2, T w3, C n0, C n1, C n2, C n3, C& k) {
+    if (folded) {  // k += i (w0 n0 + w1 n1 - w2 n2 - w3 n3)
+      k.x = fma(w3, n3.y, fma(w2, n2.y, fma(-w1, n1.y, fma(-w0, n0.y, k.x))));
+      k.y = fma(-w3, n3.x, fma(-w2, n2.x, fma(w1, n1.x, fma(w0, n0.x, k.y))));
+      return;
+    }
+    C p;
+    p.x = fma(w0, n0.x, -w3 * n3.x);
+    p.y = fma(w0, n0.y, -w3 * n3.y);
+    if (zero_bits(a.x)) {  // a = i b: the sum in one chain
+      p.x = fma(w1, n1.x, fma(-w2, n2.x, p.x));
+      p.y = fma(w1, n1.y, fma(-w2, n2.y, p.y));
+      k.x = fma(-a.y, p.y, k.x);
+      k.y = fma(a.y, p.x, k.y);
+    } else {
+      C b;
+      b.x = fma(w1, n1.x, -w2 * n2.x);
+      b.y = fma(w1, n1.y, -w2 * n2.y);
+      k = pair_sum(a, p, b, k);
+    }
+  };
+  // SMALL: a warp's one piece, its neighbours' slots, state, sum and compensation in registers
+  int of[NV];
+  unsigned int cj = 0u, sany = 0u;  // values to conjugate; sandwich terms present in the warp
   C y1 = zero, s1 = zero, c1 = zero, u1 = zero, dg1 = zero;
-  int kind1 = 0, xi1 = -1;
+  int kind1 = 0, xi1 = -1, xs1 = 0;
   bool real1 = false;
   if (SMALL && warp < cta.n) {
     const GridPiece& g = S.pc[warp];
-    const int pi = 32 * warp + lane;
+    const int pi = 32 * warp + lane, self = lane < g.len ? xidx(g) : xidx(g) - lane;
     kind1 = g.kind;
-    if (lane < g.len) xi1 = xidx(g);
-    const unsigned int any = (unsigned int)g.pad;
+    if (lane < g.len) xi1 = self;
+    xs1 = slot_of<C>(self);
+    sany = (unsigned int)g.pad;
 #pragma unroll
-    for (int i = 0; i < (SMALL ? 14 : 1); ++i) {
-      // values 0..7: pairs (points of G have two of each four); 8..13: sandwich terms
-      const bool want = i < 8 ? i < 4 * np && kind1 != GRID_D && (kind1 <= GRID_H || (i & 3) < 2) : any >> (i - 8) & 1u;
-      of[i] = want ? S.off[(i < 8 ? i : 4 * np + ((i - 8) % 3) * ns + (i - 8) / 3) * n + pi] : 0;
-      on |= (want ? 1u : 0u) << i;
+    for (int i = 0; i < NV; ++i) {
+      // values 0 .. 4 NPS - 1: pairs (points of G have two of each four), then sandwich terms
+      const int t = i - 4 * NPS, j = i < 4 * NPS ? i : 4 * np + t % 3 * ns + t / 3;
+      const bool want = i < 4 * NPS ? i < 4 * np && kind1 != GRID_D && (kind1 <= GRID_H || (i & 3) < 2) : sany >> t & 1u;
+      const int o = want ? S.off[j * n + pi] : slot_of<C>(self);
+      of[i] = o & 0x7fffffff;
+      cj |= ((unsigned)o >> 31) << i;
     }
     y1 = u1 = S.v0[pi];
     c1 = S.v2[pi];
@@ -492,40 +533,29 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
     for (int stage = 1; stage <= 4; ++stage) {
       const bool send = stage < 4 || step + 1 < A.n_steps;
       turn = turn + 1 == A.ring_places ? 0 : turn + 1;
-      C* out = ring + turn * place;
+      uint4* out = ring + turn * place;
       const C* Es = E + (((step >> 3) & 1) * 32 + (step & 7) * 4 + stage - 1) * BQ_GRID_MAXP;
       if constexpr (SMALL) {
-        if (on || warp < cta.n) {
+        if (warp < cta.n) {
           const T* w = S.w + 32 * warp + lane;
-          C v[14];
-          slots_wait<14>(in, slots, [&](int i) { return of[i]; }, on, no, v, A.error, &dead);
+          C v[NV];
+          slots_wait<NV>(in, [&](int i) { return of[i]; }, 0xffffffffu, no, v, A.error, &dead);
+          if (kind1 == GRID_H) {
+#pragma unroll
+            for (int i = 0; i < NV; ++i) v[i] = conj_bit(v[i], cj << (31 - i) & 0x80000000u);
+          }
           C k = cmul(dg1, u1);
           const unsigned int yc = kind1 == GRID_Y ? 0x80000000u : 0u;
 #pragma unroll
-          for (int j = 0; j < 2; ++j)
-            if (on >> (4 * j) & 1u) {  // (points of G: values and weights 2, 3 are zero)
-              const T w0 = w[(4 * j) * n], w1 = w[(4 * j + 1) * n], w2 = w[(4 * j + 2) * n], w3 = w[(4 * j + 3) * n];
-              const C a = conj_bit(Es[j], yc);
-              C p;
-              p.x = fma(w0, v[4 * j].x, -w3 * v[4 * j + 3].x);
-              p.y = fma(w0, v[4 * j].y, -w3 * v[4 * j + 3].y);
-              if (a.x == 0) {  // a = i b: the sum in one chain
-                p.x = fma(w1, v[4 * j + 1].x, fma(-w2, v[4 * j + 2].x, p.x));
-                p.y = fma(w1, v[4 * j + 1].y, fma(-w2, v[4 * j + 2].y, p.y));
-                k.x = fma(-a.y, p.y, k.x);
-                k.y = fma(a.y, p.x, k.y);
-              } else {
-                C b;
-                b.x = fma(w1, v[4 * j + 1].x, -w2 * v[4 * j + 2].x);
-                b.y = fma(w1, v[4 * j + 1].y, -w2 * v[4 * j + 2].y);
-                k = pair_sum(a, p, b, k);
-              }
-            }
+          for (int j = 0; j < NPS; ++j)
+            if (j < np && kind1 != GRID_D)
+              pair_term(fold >> j & 1u, conj_bit(Es[j], yc), w[(4 * j) * n], w[(4 * j + 1) * n], w[(4 * j + 2) * n],
+                        w[(4 * j + 3) * n], v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3], k);
 #pragma unroll
-          for (int s = 0; s < 2; ++s)
-            if (on >> (8 + 3 * s) & 1u) {
-              const C z = on >> (9 + 3 * s) & 1u ? cfma(v[9 + 3 * s], v[10 + 3 * s], v[8 + 3 * s]) : v[8 + 3 * s];
-              k = caxpy(w[(4 * np + s) * n], z, k);
+          for (int s = 0; s < NSS; ++s)
+            if (sany >> (3 * s) & 1u) {
+              const int i = 4 * NPS + 3 * s;
+              k = caxpy(w[(4 * np + s) * n], sany >> (3 * s + 1) & 1u ? cfma(v[i + 1], v[i + 2], v[i]) : v[i], k);
             }
           if (real1) k.y = (T)0;  // the diagonal of a Hermitian system is real
           if (stage < 4) {
@@ -535,7 +565,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
             y1 = u1 = update(s1, k, y1, c1);
           }
           if (send && xi1 >= 0) {
-            slot_put(out, slots, xi1, u1, no + 1);
+            slot_put(out + xs1, u1, no + 1);
             if (A.rec) (stage < 4 ? recorded(step, stage + 1) : recorded(step + 1, 1))[xi1] = u1;
           }
         }
@@ -551,22 +581,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
         C k = cmul(S.dg[pi], u);
         // pair j of R with its four neighbours, and a sandwich term with its three
         auto pair = [&](int j, C n0, C n1, C n2, C n3) {
-          const T w0 = w[(4 * j) * n], w1 = w[(4 * j + 1) * n], w2 = w[(4 * j + 2) * n], w3 = w[(4 * j + 3) * n];
-          const C a = Es[j];
-          C p;
-          p.x = fma(w0, n0.x, -w3 * n3.x);
-          p.y = fma(w0, n0.y, -w3 * n3.y);
-          if (a.x == 0) {  // a = i b: the sum in one chain
-            p.x = fma(w1, n1.x, fma(-w2, n2.x, p.x));
-            p.y = fma(w1, n1.y, fma(-w2, n2.y, p.y));
-            k.x = fma(-a.y, p.y, k.x);
-            k.y = fma(a.y, p.x, k.y);
-          } else {
-            C b;
-            b.x = fma(w1, n1.x, -w2 * n2.x);
-            b.y = fma(w1, n1.y, -w2 * n2.y);
-            k = pair_sum(a, p, b, k);
-          }
+          pair_term(fold >> j & 1u, Es[j], w[(4 * j) * n], w[(4 * j + 1) * n], w[(4 * j + 2) * n], w[(4 * j + 3) * n], n0, n1,
+                    n2, n3, k);
         };
         auto sand = [&](int s, C v, C x, C y) {
           k = caxpy(w[(4 * np + s) * n], P.has_sep ? cfma(x, y, v) : v, k);
@@ -577,14 +593,20 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
           for (int j0 = 0; j0 < np; j0 += 4) {
             const int m = min(4, np - j0);
             C v[8];
-            slots_wait<8>(in, slots, [&](int i) { return off[(4 * (j0 + i / 2) + (i & 1)) * n]; }, (1u << (2 * m)) - 1u, no, v,
+            slots_wait_conj<8>(in, [&](int i) { return off[(4 * (j0 + i / 2) + (i & 1)) * n]; }, (1u << (2 * m)) - 1u, no, v,
                           A.error, &dead);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               if (i >= m) break;
               const int j = j0 + i;
-              k = pair_sum(conj_bit(Es[j], kind == GRID_X ? 0u : 0x80000000u), cscale(v[2 * i], w[(4 * j) * n]),
-                           cscale(v[2 * i + 1], w[(4 * j + 1) * n]), k);
+              const T w0 = w[(4 * j) * n], w1 = w[(4 * j + 1) * n];
+              if (fold >> j & 1u) {
+                k.x = fma(-w1, v[2 * i + 1].y, fma(-w0, v[2 * i].y, k.x));
+                k.y = fma(w1, v[2 * i + 1].x, fma(w0, v[2 * i].x, k.y));
+              } else {
+                k = pair_sum(conj_bit(Es[j], kind == GRID_X ? 0u : 0x80000000u), cscale(v[2 * i], w0),
+                             cscale(v[2 * i + 1], w1), k);
+              }
             }
           }
         } else {
@@ -594,7 +616,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
             for (int j0 = 0; j0 < np; j0 += PB) {
               const int m = min(PB, np - j0);
               C v[4 * PB];
-              slots_wait<4 * PB>(in, slots, [&](int i) { return off[(4 * j0 + i) * n]; }, (1u << (4 * m)) - 1u, no, v, A.error, &dead);
+              slots_wait_conj<4 * PB>(in, [&](int i) { return off[(4 * j0 + i) * n]; }, (1u << (4 * m)) - 1u, no, v, A.error, &dead);
 #pragma unroll
               for (int i = 0; i < PB; ++i)
                 if (i < m) pair(j0 + i, v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
@@ -605,7 +627,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
             const unsigned int on = any >> (3 * s0) & 63u;
             if (!on) continue;
             C v[6];
-            slots_wait<6>(in, slots, [&](int i) { return soff(3 * s0 + i); }, on, no, v, A.error, &dead);
+            slots_wait_conj<6>(in, [&](int i) { return soff(3 * s0 + i); }, on, no, v, A.error, &dead);
 #pragma unroll
             for (int s = 0; s < 2; ++s)
               if (on >> (3 * s) & 1u) sand(s0 + s, v[3 * s], v[3 * s + 1], v[3 * s + 2]);
@@ -625,7 +647,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
         S.v3[pi] = nu;
         if (send && lane < len) {
           const int i = xidx(S.pc[q]);
-          slot_put(out, slots, i, nu, no + 1);
+          slot_put(out + slot_of<C>(i), nu, no + 1);
           if (A.rec) (stage < 4 ? recorded(step, stage + 1) : recorded(step + 1, 1))[i] = nu;
         }
       }
@@ -702,11 +724,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
   const GridTab<T> W(P, reinterpret_cast<const T*>(A.tab) + P.tab);
   for (int i = tid; i < 2 * ns * ng; i += THREADS) swt[i] = W.sand(0, 0)[i];
   __syncthreads();
-  C* const ring = reinterpret_cast<C*>(A.ring);
-  const size_t slots = A.arr / sizeof(C), place = 2 * slots;
+  uint4* const ring = reinterpret_cast<uint4*>(A.ring);
+  const size_t place = A.place;
+  const int places = (int)min((long long)A.ring_places, 4LL * A.n_steps + 1);  // that this launch uses
   auto xidx = [&](const GridPiece& g) {
     return (g.kind <= GRID_D ? g.off_r : g.kind == GRID_X ? g.off_gx : g.off_gy) + g.start + lane;
   };
+  int hre_any = 0;
   const T hh = (T)A.dt, w6 = hh * (T)(1.0 / 6.0), w3 = hh * (T)(1.0 / 3.0), h2 = hh * (T)0.5;
   for (int q = warp; q < cta.n; q += nw) {
     const GridPiece g = S.pc[q];
@@ -715,23 +739,23 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
     const int self = xidx(g), si = ok ? self : self - lane, i = g.start + lane;
     const int k = g.kind == GRID_R ? i / ng : i, l = g.kind == GRID_R ? i - k * ng : i;
     for (int j = 0; j < 4 * np + ns; ++j) {
-      S.off[j * n + pi] = si;
+      S.off[j * n + pi] = slot_of<C>(si);
       S.w[j * n + pi] = (T)0;
     }
     for (int t = 0; t < 2 * nt; ++t) S.w[(4 * np + ns + t) * n + pi] = (T)0;
     C v = zero, dg = zero;
     if (ok) {
       v = reinterpret_cast<const C*>(A.lam)[self];
-      for (int r = 0; r < A.ring_places; ++r)
-        if (r != 1) slot_put(ring + r * place, slots, self, zero, 0u);
-      slot_put(ring + place, slots, self, cscale(v, w6), 1u);
+      for (int r = 0; r < places; ++r)
+        if (r != 1) slot_put(ring + r * place + slot_of<C>(self), zero, 0u);
+      slot_put(ring + place + slot_of<C>(self), cscale(v, w6), 1u);
       if (g.kind <= GRID_D) dg = cadd(W.dx[k], W.dy[l]);
       else if (g.kind == GRID_X) dg = cadd(W.dx[k], cmk<C>(g.c_re, g.c_im));
       else dg = cadd(W.dy[k], cmk<C>(-g.c_re, -g.c_im));
       auto put = [&](int j, T w, int o) {
         if (w == (T)0) return;
         S.w[j * n + pi] = w;
-        S.off[j * n + pi] = o;
+        S.off[j * n + pi] = slot_of<C>(o);
       };
       // transposed sources: xmT at k + d, xpT at k - d, ymT at l + d, ypT at l - d
       for (int j = 0; j < np; ++j) {
@@ -759,6 +783,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
       for (int t = 0; t < nt; ++t) {
         const C h = g.kind <= GRID_D ? cadd(W.diagp(t, 0)[k], W.diagp(t, 1)[l])
                                      : (g.kind == GRID_X ? W.diagp(t, 0)[k] : W.diagp(t, 1)[k]);
+        if (h.x != (T)0) hre_any = 1;
         S.w[(4 * np + ns + 2 * t) * n + pi] = h.x;
         S.w[(4 * np + ns + 2 * t + 1) * n + pi] = h.y;
       }
@@ -783,24 +808,27 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
   const long long last = A.n_steps - 1;
   if (warp == nw - 1) grid_envelope<T>(A, P, E, last & ~7LL, segs);
   unsigned int block = 0;
+  const bool hre = __syncthreads_or(hre_any);
   if (!grid_sync(A.bar, A.error)) return;
 
   auto seg_of = [&](long long i, int j) { return segs[(((i >> 3) & 1) * 8 + (i & 7)) * BQ_GRID_MAXP + j]; };
 
   unsigned int no = 1;
-  const C* in = ring + place;
+  const uint4* in = ring + place;
   int turn = 1;
   // value of pair j at this point: a from sources x.lo, y.lo, b from x.hi, y.hi (see pair_sum)
   int of[ONE ? 14 : 1], go[ONE ? BQ_GRID_ROWS : 1];
   unsigned int on = 0u;
   C l1 = zero, a1 = zero, b1 = zero, dg1 = zero;
-  int kind1 = 0, xi1 = -1, rows = 0;
+  int kind1 = 0, xi1 = -1, xs1 = 0, rows = 0;
   if (ONE && warp < cta.n) {
     const GridPiece& g = S.pc[warp];
     const int pi = 32 * warp + lane;
     const bool isx = g.kind == GRID_X;
+    const int self = lane < g.len ? xidx(g) : xidx(g) - lane;  // (for values that a point lacks)
     kind1 = g.kind;
-    if (lane < g.len) xi1 = xidx(g);
+    if (lane < g.len) xi1 = self;
+    xs1 = slot_of<C>(self);
     l1 = a1 = S.v0[pi];
     b1 = S.v3[pi];
     dg1 = S.dg[pi];
@@ -808,7 +836,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
 #pragma unroll
       for (int i = 0; i < (ONE ? 14 : 1); ++i) {
         const bool want = i < 8 ? i < 4 * np && kind1 == GRID_R : (unsigned int)g.pad >> (i - 8) & 1u;
-        of[i] = want ? S.off[(i < 8 ? i : 4 * np + i - 8) * n + pi] : 0;
+        of[i] = want ? S.off[(i < 8 ? i : 4 * np + i - 8) * n + pi] : xs1;
         on |= (want ? 1u : 0u) << i;
       }
     } else {  // values 0..3: lo and hi of the pairs, 4..13: elements of the rows or columns of b_R
@@ -816,7 +844,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
       rows = P.has_r ? ns * nj : 0;
 #pragma unroll
       for (int i = 0; i < (ONE ? 14 : 1); ++i) {
-        of[i] = 0;
+        of[i] = xs1;
         if (i < 4) {
           if (i < 2 * np && xi1 >= 0) {
             of[i] = S.off[(4 * (i >> 1) + (i & 1)) * n + pi];
@@ -834,7 +862,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
             if (!P.r_diag && P.sst[s] && (j / P.sst[s]) % P.sM[s] != (kk / P.sst[s]) % P.sM[s]) wt = (T)0;
           }
           if (wt != (T)0) {
-            of[i] = g.off_r + (P.r_diag ? kk : isx ? kk * ng + j : j * ng + kk);
+            of[i] = slot_of<C>(g.off_r + (P.r_diag ? kk : isx ? kk * ng + j : j * ng + kk));
             go[t] = (isx ? g.off_gy : g.off_gx) + P.ss[s] + j;
             on |= 1u << i;
           }
@@ -843,16 +871,50 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
       }
     }
   }
-  auto grad_pair = [&](int j, C u, C a, C b) {
-    if (P.gpar[j] < 0 && P.gpwc[j] < 0) return;
-    C s = cadd(a, b), d;
-    d.x = a.x - b.x;
-    d.y = a.y - b.y;
+  // which sums pair j needs (bits 2 j, 2 j + 1: gy, gx): a static imaginary derivative only Im
+  unsigned int gneed = 0u;
+  for (int j = 0; j < np; ++j)
+    if (P.gpar[j] >= 0 || P.gpwc[j] >= 0)
+      gneed |= (P.gpwc[j] >= 0 || P.ch[j] >= 0 || P.cb_re[j] != 0.0 ? 3u : 1u) << (2 * j);
+  // q += av a - conj(av) b; s = a + b, d = a - b (where needed)
+  auto pair_q = [&](int j, C av, C a, C b, C& s, C& d, C& qv) {
+    s = cadd(a, b);
+    const bool im = zero_bits(av.x);
+    d = zero;
+    if (!im || (gneed >> (2 * j) & 2u)) {
+      d.x = a.x - b.x;
+      d.y = a.y - b.y;
+    }
+    qv.x = fma(-av.y, s.y, qv.x);
+    qv.y = fma(av.y, s.x, qv.y);
+    if (!im) {
+      qv.x = fma(av.x, d.x, qv.x);
+      qv.y = fma(av.x, d.y, qv.y);
+    }
+  };
+  auto pair_sums = [&](int j, C u, C s, C d) {
 #pragma unroll
     for (int i = 0; i < NP; ++i)
       if (i == j) {
-        grad_add(gx[i], u.x, d.x, -u.y, d.y);
-        grad_add(gy[i], u.x, s.y, u.y, s.x);
+        if (gneed >> (2 * i) & 1u) grad_add(gy[i], u.x, s.y, u.y, s.x);
+        if (gneed >> (2 * i) & 2u) grad_add(gx[i], u.x, d.x, -u.y, d.y);
+      }
+  };
+  auto pair_grad = [&](int j, C av, C a, C b, C u, C& qv) {
+    C s, d;
+    pair_q(j, av, a, b, s, d, qv);
+    pair_sums(j, u, s, d);
+  };
+  // u b dD/dtheta of the parameters on diagonal terms; their weights are imaginary unless hre
+  auto diag_grad = [&](const T* w, C u, C b) {
+    const T zy = fma(u.x, b.y, u.y * b.x);
+    const T zx = hre ? fma(u.x, b.x, -u.y * b.y) : (T)0;
+#pragma unroll
+    for (int t = 0; t < BQ_GRID_MAXT; ++t)
+      if (t < nt) {
+        const T hy = w[(4 * np + ns + 2 * t + 1) * n];
+        if (hre) grad_add(gt[t], zx, w[(4 * np + ns + 2 * t) * n], -zy, hy);
+        else grad_add(gt[t], -zy, hy);
       }
   };
 
@@ -866,7 +928,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
 #pragma unroll 1
     for (int stage = 4; stage >= 1; --stage) {
       turn = turn + 1 == A.ring_places ? 0 : turn + 1;
-      C* out = ring + turn * place;
+      uint4* out = ring + turn * place;
       const C* U = reinterpret_cast<const C*>(A.rec + ((size_t)it * 4 + stage - 1) * A.arr);
       const C* Es = E + (((it >> 3) & 1) * 32 + (it & 7) * 4 + stage - 1) * BQ_GRID_MAXP;
       if constexpr (ONE) {
@@ -880,8 +942,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
               if (t < rows) h[t] = on >> (4 + t) & 1u ? cscale(U[go[t]], w[(wrow + t) * n]) : zero;
           }
           C v[14];
-          slots_wait<14>(in, slots, [&](int i) { return of[i]; }, on, no, v, A.error, &dead);
-          C qv = cmul(dg1, b1);
+          slots_wait<14>(in, [&](int i) { return of[i]; }, 0xffffffffu, no, v, A.error, &dead);
+          // (the gradient sums follow the store: no other warp waits for them)
+          C qv = cmul(dg1, b1), ps[2] = {zero, zero}, pd[2] = {zero, zero};
           if (kind1 <= GRID_D) {
 #pragma unroll
             for (int j = 0; j < 2; ++j)
@@ -892,8 +955,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
                 a.y = fma(w0, v[4 * j].y, -w3_ * v[4 * j + 3].y);
                 c.x = fma(w1, v[4 * j + 1].x, -w2 * v[4 * j + 2].x);
                 c.y = fma(w1, v[4 * j + 1].y, -w2 * v[4 * j + 2].y);
-                qv = pair_sum(Es[j], a, c, qv);
-                grad_pair(j, u, a, c);
+                pair_q(j, Es[j], a, c, ps[j], pd[j], qv);
               }
 #pragma unroll
             for (int s = 0; s < 2; ++s)
@@ -924,21 +986,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
             for (int j = 0; j < 2; ++j)
               if (j < np) {
                 const C lo = cscale(v[2 * j], w[(4 * j) * n]), hi = cscale(v[2 * j + 1], w[(4 * j + 1) * n]);
-                qv = pair_sum(conj_bit(Es[j], isx ? 0u : 0x80000000u), lo, hi, qv);
                 // X: a lo - conj(a) hi;  Y: conj(a) lo - a hi = a (-hi) - conj(a) (-lo)
-                grad_pair(j, u, isx ? lo : cneg(hi), isx ? hi : cneg(lo));
+                pair_q(j, Es[j], isx ? lo : cneg(hi), isx ? hi : cneg(lo), ps[j], pd[j], qv);
               }
-            const C z = cmul(u, b1);
-            const double sg = isx ? 1.0 : -1.0;
-            dcs.x += sg * (double)z.x;
-            dcs.y += sg * (double)z.y;
           }
-          if (nt) {  // Re sum u b dD/dtheta of the parameters on diagonal terms
-            const C z = cmul(u, b1);
-#pragma unroll
-            for (int t = 0; t < BQ_GRID_MAXT; ++t)
-              if (t < nt) grad_add(gt[t], z.x, w[(4 * np + ns + 2 * t) * n], -z.y, w[(4 * np + ns + 2 * t + 1) * n]);
-          }
+          const C b0 = b1;
           a1 = cadd(a1, qv);  // (the step's sum starts as lam)
           if (stage > 1) {
             b1 = caxpy(stage == 4 ? hh : h2, qv, cscale(l1, stage == 2 ? w6 : w3));
@@ -946,7 +998,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
             l1 = a1;
             b1 = cscale(a1, w6);
           }
-          if (xi1 >= 0 && (it > 0 || stage > 1)) slot_put(out, slots, xi1, b1, no + 1);
+          if (xi1 >= 0 && (it > 0 || stage > 1)) slot_put(out + xs1, b1, no + 1);
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            if (j < np) pair_sums(j, u, ps[j], pd[j]);
+          if (nt) diag_grad(w, u, b0);
+          if (kind1 >= GRID_X) {
+            const C z = cmul(u, b0);
+            if (kind1 == GRID_X) dcs = make_double2(dcs.x + (double)z.x, dcs.y + (double)z.y);
+            else dcs = make_double2(dcs.x - (double)z.x, dcs.y - (double)z.y);
+          }
         }
       } else {
 #pragma unroll 1
@@ -970,25 +1031,24 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
             a.y = fma(w0, n0.y, -w3_ * n3.y);
             c.x = fma(w1, n1.x, -w2 * n2.x);
             c.y = fma(w1, n1.y, -w2 * n2.y);
-            qv = pair_sum(Es[j], a, c, qv);
-            grad_pair(j, u, a, c);
+            pair_grad(j, Es[j], a, c, u, qv);
           };
 #pragma unroll 1
             for (int j0 = 0; j0 < np; j0 += 2) {
               const int m = min(2, np - j0);
               C v[8];
-              slots_wait<8>(in, slots, [&](int i) { return off[(4 * j0 + i) * n]; }, (1u << (4 * m)) - 1u, no, v, A.error, &dead);
+              slots_wait<8>(in, [&](int i) { return off[(4 * j0 + i) * n]; }, (1u << (4 * m)) - 1u, no, v, A.error, &dead);
 #pragma unroll
               for (int i = 0; i < 2; ++i)
                 if (i < m) pair(j0 + i, v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
             }
-            slots_wait<4>(in, slots, [&](int i) { return off[(4 * np + i) * n]; }, any, no, sv, A.error, &dead);
+            slots_wait<4>(in, [&](int i) { return off[(4 * np + i) * n]; }, any, no, sv, A.error, &dead);
 #pragma unroll
           for (int s = 0; s < 4; ++s)
             if (any >> s & 1u) qv = caxpy(w[(4 * np + s) * n], sv[s], qv);
         } else if (kind == GRID_D) {
           C sv[4];
-          slots_wait<4>(in, slots, [&](int i) { return off[(4 * np + i) * n]; }, any, no, sv, A.error, &dead);
+          slots_wait<4>(in, [&](int i) { return off[(4 * np + i) * n]; }, any, no, sv, A.error, &dead);
 #pragma unroll
           for (int s = 0; s < 4; ++s)
             if (any >> s & 1u) qv = caxpy(w[(4 * np + s) * n], sv[s], qv);
@@ -1011,7 +1071,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
               if (P.r_diag) {
                 const T wj = lane == 0 ? wo[kk] : (T)0;  // (the whole warp calls slots_wait)
                 C x[1];
-                slots_wait<1>(in, slots, [&](int) { return g.off_r + kk; }, wj != (T)0 ? 1u : 0u, no, x, A.error, &dead);
+                slots_wait<1>(in, [&](int) { return slot_of<C>(g.off_r + kk); }, wj != (T)0 ? 1u : 0u, no, x, A.error, &dead);
                 if (wj != (T)0) v = cmul(x[0], cscale(go[kk], wj));
               } else {
                 const int mk = P.sst[s] ? (kk / P.sst[s]) % P.sM[s] : 0;
@@ -1026,7 +1086,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
                     const int j = j0 + 32 * i;
                     if (j < ng && wo[j] != (T)0 && !(P.sst[s] && (j / P.sst[s]) % P.sM[s] != mk)) on |= 1u << i;
                   }
-                  slots_wait<6>(in, slots, [&](int i) { return br + (j0 + 32 * i) * st; }, on, no, x, A.error, &dead);
+                  slots_wait<6>(in, [&](int i) { return slot_of<C>(br + (j0 + 32 * i) * st); }, on, no, x, A.error, &dead);
 #pragma unroll
                   for (int i = 0; i < 6; ++i)
                     if (on >> i & 1u) v = cfma(x[i], cscale(go[j0 + 32 * i], wo[j0 + 32 * i]), v);
@@ -1047,7 +1107,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
           for (int j0 = 0; j0 < np; j0 += 2) {
             const int m = min(2, np - j0);
             C v[4];
-            slots_wait<4>(in, slots, [&](int i) { return off[(4 * (j0 + i / 2) + (i & 1)) * n]; },
+            slots_wait<4>(in, [&](int i) { return off[(4 * (j0 + i / 2) + (i & 1)) * n]; },
                           ok ? (1u << (2 * m)) - 1u : 0u, no, v, A.error, &dead);
             if (ok) {
 #pragma unroll
@@ -1055,26 +1115,19 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
                 if (i >= m) break;
                 const int j = j0 + i;
                 const C lo = cscale(v[2 * i], w[(4 * j) * n]), hi = cscale(v[2 * i + 1], w[(4 * j + 1) * n]);
-                qv = pair_sum(conj_bit(Es[j], isx ? 0u : 0x80000000u), lo, hi, qv);
                 // X: a lo - conj(a) hi;  Y: conj(a) lo - a hi = a (-hi) - conj(a) (-lo)
-                grad_pair(j, u, isx ? lo : cneg(hi), isx ? hi : cneg(lo));
+                pair_grad(j, Es[j], isx ? lo : cneg(hi), isx ? hi : cneg(lo), u, qv);
               }
             }
           }
           if (ok) {
             const C z = cmul(u, b);
-            const double sg = isx ? 1.0 : -1.0;
-            dcs.x += sg * (double)z.x;
-            dcs.y += sg * (double)z.y;
+            if (isx) dcs = make_double2(dcs.x + (double)z.x, dcs.y + (double)z.y);
+            else dcs = make_double2(dcs.x - (double)z.x, dcs.y - (double)z.y);
           }
           __syncwarp();
         }
-        if (nt) {  // Re sum u b dD/dtheta of the parameters on diagonal terms
-          const C z = cmul(u, b);
-#pragma unroll
-          for (int t = 0; t < BQ_GRID_MAXT; ++t)
-            if (t < nt) grad_add(gt[t], z.x, w[(4 * np + ns + 2 * t) * n], -z.y, w[(4 * np + ns + 2 * t + 1) * n]);
-        }
+        if (nt) diag_grad(w, u, b);
         if (ok) {
           const C lv = S.v0[pi];
           const C av = cadd(S.v1[pi], qv);  // (the step's sum starts as lam)
@@ -1087,7 +1140,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
             bn = cscale(av, w6);
           }
           S.v3[pi] = bn;
-          if (it > 0 || stage > 1) slot_put(out, slots, xidx(g), bn, no + 1);
+          if (it > 0 || stage > 1) slot_put(out + slot_of<C>(xidx(g)), bn, no + 1);
         }
       }
       }
@@ -1120,6 +1173,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
         }
 #pragma unroll
         for (int t = 0; t < BQ_GRID_MAXT; ++t) {
+          if (t >= nt) break;
           const double x = sum(gt[t]);
           if (lane == 0) red[warp][2 * NP + t] = x;
           gt[t] = 0.0;
@@ -1194,8 +1248,9 @@ static const void* grid_func_t(int np, int ns, bool adj, int form) {
     if (np <= 4) return form == GRID_FEW ? (const void*)k_grid_adj<T, 4, 256, false> : (const void*)k_grid_adj<T, 4, 512, false>;
     return nullptr;
   }
-  if (form == GRID_ONE) return (const void*)k_grid_fwd<T, true, 256>;
-  return form == GRID_FEW ? (const void*)k_grid_fwd<T, false, 256> : (const void*)k_grid_fwd<T, false, 512>;
+  if (form == GRID_ONE)
+    return np > 1 ? (const void*)k_grid_fwd<T, 2, 2, 256> : ns > 1 ? (const void*)k_grid_fwd<T, 1, 2, 256> : (const void*)k_grid_fwd<T, 1, 1, 256>;
+  return form == GRID_FEW ? (const void*)k_grid_fwd<T, 0, 0, 256> : (const void*)k_grid_fwd<T, 0, 0, 512>;
 }
 
 static cudaError_t launch_grid_any(const void* f, const GridArgs& a, int ctas, int form, int smem_bytes, cudaStream_t s) {

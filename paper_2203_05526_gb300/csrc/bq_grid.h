@@ -61,7 +61,8 @@ struct GridArgs {
   const double* chpar;
   void* y;
   void* comp;
-  void* ring;     // exchange of stage inputs (adjoint: of b): ring_places x 2 arr bytes
+  void* ring;     // exchange of stage inputs (adjoint: of b): ring_places x place 16-byte words
+  size_t place;   // grid_place()
   int ring_places, block;  // places; steps (a power of two) between the CTAs' block counts
   char* rec;      // recorded stage inputs (4 per step) or null
   size_t arr;     // bytes of one state array
@@ -83,6 +84,8 @@ cudaError_t launch_grid_f64(const GridArgs& a, int np, int ns, bool adj, int cta
 const void* grid_func_f32(int np, int ns, bool adj, int form);
 const void* grid_func_f64(int np, int ns, bool adj, int form);
 
+// 16-byte words of a place of the ring: a state's slots, in whole groups of 32 (FP64: two words each).
+inline size_t grid_place(size_t elems, size_t cs) { return (elems + 31) / 32 * (cs == 16 ? 64 : 32); }
 // Forms of the kernels, by the largest number n of pieces in a CTA: a piece per warp in registers (small
 // problems), eight warps, sixteen warps.
 enum GridForm : int { GRID_ONE = 0, GRID_FEW = 1, GRID_MANY = 2 };

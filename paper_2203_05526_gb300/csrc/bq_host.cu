@@ -1274,9 +1274,9 @@ static const int64_t kGridMaxPoints = 152 * 2500;
 // (growing with the number from there; the resident kernel's 35 hold up to two systems per SM).
 static const int kGridFewSystems = 128;
 static const int kGridFewM = 20;  // of a single system: below, both are at their latencies
-// Steps between the block counts of the grid-resident kernels: two while the ring stays small
-// beside L2, one for larger states.
-static int grid_block(size_t arr) { return arr <= ((size_t)1 << 20) ? 2 : 1; }
+// Steps between the block counts of the grid-resident kernels (a power of two, at most four): fewer
+// while the ring would not stay small beside L2.
+static int grid_block(size_t arr) { return arr <= ((size_t)1 << 19) ? 4 : arr <= ((size_t)1 << 20) ? 2 : 1; }
 
 // X or Y term t's weights over the flat index of its side; S terms: of side y's dimensions.
 static std::vector<double> flat_weights(const Compiled& C, const TermDesc& td, int wbase, bool y) {
@@ -2037,7 +2037,7 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
   L.off_gpieces = seg(P.grid_cap * sizeof(bq::GridPiece));
   L.off_gctas = seg(P.grid_ok ? 3 * kGridMaxCtas * sizeof(bq::GridCta) : 0);
   L.off_gbar = seg(P.grid_ok ? BQ_GRID_BAR_WORDS * sizeof(unsigned int) : 0);
-  L.off_gring = seg(P.grid_ok ? 2 * (size_t)P.total_elems * cs * (8 * grid_block((size_t)P.total_elems * cs) + 1) : 0);
+  L.off_gring = seg(P.grid_ok ? 16 * bq::grid_place((size_t)P.total_elems, cs) * (8 * grid_block((size_t)P.total_elems * cs) + 1) : 0);
   L.off_dc = seg(P.dc.size() * sizeof(double2));
   L.off_groups = seg(P.groups.size() * sizeof(EvalGroup));
   L.off_entries = seg(P.entries.size() * sizeof(EvalEntry));
@@ -2412,6 +2412,7 @@ static bq::GridArgs grid_args(bq_state* s, int q, double dt) {
   a.comp = b + L.off_comp;
   a.arr = (size_t)s->total_elems * (s->dtype == BQ_F64 ? 16 : 8);
   a.ring = b + L.off_gring;
+  a.place = bq::grid_place((size_t)s->total_elems, s->dtype == BQ_F64 ? 16 : 8);
   a.block = grid_block(a.arr);
   a.ring_places = 8 * a.block + 1;
   a.bar = (unsigned int*)(b + L.off_gbar);

@@ -2041,7 +2041,7 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
   L.off_dc = seg(P.dc.size() * sizeof(double2));
   L.off_groups = seg(P.groups.size() * sizeof(EvalGroup));
   L.off_entries = seg(P.entries.size() * sizeof(EvalEntry));
-  L.off_out = seg(P.groups.size() * 2 * sizeof(double));
+  L.off_out = seg((P.groups.size() + 1) * 2 * sizeof(double)) + 2 * sizeof(double);  // (the error word's slot first)
   L.off_wtab = seg(P.wtab.size() * rs);
   L.off_diag = seg(P.diag.size() * cs);
   L.off_ctrl = seg(64);
@@ -3461,6 +3461,21 @@ extern "C" int bq_time(const bq_state* s, double* tau) {
 // ---------------------------------------------------------------------------------------
 // Evaluation.
 // ---------------------------------------------------------------------------------------
+// The first n results and the error word, which the kernel on st has placed before them; waits for st.
+// A few results come with the word in one copy; many go straight to the caller's array.
+static int read_results(bq_state* s, int n, double* out_host, cudaStream_t st) {
+  const char* out = s->pool + s->L.off_out;
+  const int kSmall = 256;
+  double buf[2 * (kSmall + 1)];
+  CUDA_TRY(cudaMemcpyAsync(buf, out - 16, n <= kSmall ? 16 * (size_t)(n + 1) : 16, cudaMemcpyDeviceToHost, st));
+  if (n > kSmall) CUDA_TRY(cudaMemcpyAsync(out_host, out, (size_t)n * 16, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaStreamSynchronize(st));
+  if (n <= kSmall) std::memcpy(out_host, buf + 2, (size_t)n * 16);
+  if (buf[0] != 0.0)
+    return fail(BQ_ETIMEOUT, "a bounded device wait gave up during stepping (error word %u)", (unsigned int)buf[0]);
+  return BQ_OK;
+}
+
 static int run_eval(bq_state* s, int g0, int n, int small, double* out_host, cudaStream_t st) {
   char* b = s->pool;
   const Layout& L = s->L;
@@ -3468,13 +3483,18 @@ static int run_eval(bq_state* s, int g0, int n, int small, double* out_host, cud
   CUDA_TRY(bq::launch_eval((const SysDesc*)(b + L.off_sys), (const EvalGroup*)(b + L.off_groups) + g0,
                            (const EvalEntry*)(b + L.off_entries), b + L.off_y, b + L.off_comp,
                            (double2*)(b + L.off_out) + g0, n,
-                           s->dtype, small, st));
+                           s->dtype, small, g0 == 0 ? (const unsigned int*)(b + L.off_ctrl + 32) : nullptr, st));
   g_launches++;
-  CUDA_TRY(cudaMemcpyAsync(out_host, b + L.off_out + (size_t)g0 * 16, (size_t)n * 16, cudaMemcpyDeviceToHost, st));
-  unsigned int err_word = 0;
-  CUDA_TRY(cudaMemcpyAsync(&err_word, b + L.off_ctrl + 32, sizeof(err_word), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaStreamSynchronize(st));
-  if (err_word) return fail(BQ_ETIMEOUT, "a bounded device wait gave up during stepping (error word %u)", err_word);
+  if (g0 == 0) {
+    const int r = read_results(s, n, out_host, st);
+    if (r != BQ_OK) return r;
+  } else {
+    CUDA_TRY(cudaMemcpyAsync(out_host, b + L.off_out + (size_t)g0 * 16, (size_t)n * 16, cudaMemcpyDeviceToHost, st));
+    unsigned int err_word = 0;
+    CUDA_TRY(cudaMemcpyAsync(&err_word, b + L.off_ctrl + 32, sizeof(err_word), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    if (err_word) return fail(BQ_ETIMEOUT, "a bounded device wait gave up during stepping (error word %u)", err_word);
+  }
   for (int i = 0; i < 2 * n; ++i)
     if (!std::isfinite(out_host[i])) return fail(BQ_ENONFINITE, "non-finite observable");
   return BQ_OK;
@@ -3488,14 +3508,15 @@ static int enqueue_trace(bq_state* s, cudaStream_t st) {
   const Layout& L = s->L;
   if (s->obs_valid) {
     CUDA_TRY(bq::launch_obs_sum((const double2*)(b + L.off_obs), (const EvalGroup*)(b + L.off_groups),
-                                s->n_trace_groups, (double2*)(b + L.off_out), st));
+                                s->n_trace_groups, (double2*)(b + L.off_out), (const unsigned int*)(b + L.off_ctrl + 32), st));
     g_launches++;
     return BQ_OK;
   }
   CUDA_TRY(ensure_comp(s, st));
   CUDA_TRY(bq::launch_eval((const SysDesc*)(b + L.off_sys), (const EvalGroup*)(b + L.off_groups),
                            (const EvalEntry*)(b + L.off_entries), b + L.off_y, b + L.off_comp,
-                           (double2*)(b + L.off_out), s->n_trace_groups, s->dtype, s->trace_small, st));
+                           (double2*)(b + L.off_out), s->n_trace_groups, s->dtype, s->trace_small,
+                           (const unsigned int*)(b + L.off_ctrl + 32), st));
   g_launches++;
   return BQ_OK;
 }
@@ -3506,11 +3527,8 @@ extern "C" int bq_evaluate(bq_state* s, double* out_host, void* stream) {
   const int n = s->n_trace_groups;
   int r = enqueue_trace(s, st);
   if (r != BQ_OK) return r;
-  CUDA_TRY(cudaMemcpyAsync(out_host, s->pool + s->L.off_out, (size_t)n * 16, cudaMemcpyDeviceToHost, st));
-  unsigned int err_word = 0;
-  CUDA_TRY(cudaMemcpyAsync(&err_word, s->pool + s->L.off_ctrl + 32, sizeof(err_word), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaStreamSynchronize(st));
-  if (err_word) return fail(BQ_ETIMEOUT, "a bounded device wait gave up during stepping (error word %u)", err_word);
+  r = read_results(s, n, out_host, st);
+  if (r != BQ_OK) return r;
   for (int i = 0; i < 2 * n; ++i)
     if (!std::isfinite(out_host[i])) return fail(BQ_ENONFINITE, "non-finite observable of problem %d", i / 2);
   return BQ_OK;

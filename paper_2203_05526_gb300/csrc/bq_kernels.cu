@@ -2574,11 +2574,18 @@ struct StateView {
   }
 };
 
+// The error word next to the results (in the slot before the first), so that the host reads both with
+// one copy: two pageable copies were 16 of the 69 us of a one-step call and its observable.
+__device__ __forceinline__ void out_error(const unsigned int* error, double2* out) {
+  if (error) out[-1] = make_double2((double)*error, 0.0);
+}
+
 template <typename T>
 __global__ void k_eval(const SysDesc* __restrict__ sys, const EvalGroup* __restrict__ groups,
                        const EvalEntry* __restrict__ entries, const void* ystate, const void* cstate, double2* out,
-                       int n_groups) {
+                       int n_groups, const unsigned int* error) {
   using C = typename C2T<T>::type;
+  if (blockIdx.x == 0 && threadIdx.x == 0) out_error(error, out);
   const StateView<C> y{reinterpret_cast<const C*>(ystate), reinterpret_cast<const C*>(cstate)};
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -2622,8 +2629,9 @@ __global__ void k_eval(const SysDesc* __restrict__ sys, const EvalGroup* __restr
 template <typename T>
 __global__ void k_eval_small(const SysDesc* __restrict__ sys, const EvalGroup* __restrict__ groups,
                              const EvalEntry* __restrict__ entries, const void* ystate, const void* cstate, double2* out,
-                             int n_groups) {
+                             int n_groups, const unsigned int* error) {
   using C = typename C2T<T>::type;
+  if (blockIdx.x == 0 && threadIdx.x == 0) out_error(error, out);
   const StateView<C> y{reinterpret_cast<const C*>(ystate), reinterpret_cast<const C*>(cstate)};
   const int gi = blockIdx.x * blockDim.x + threadIdx.x;
   if (gi >= n_groups) return;
@@ -3051,22 +3059,23 @@ cudaError_t launch_stage(const StageArgs& a, int dtype, int nm, int n_work, int 
 }
 
 cudaError_t launch_eval(const SysDesc* sys, const EvalGroup* groups, const EvalEntry* entries, const void* y,
-                        const void* comp, double2* out, int n_groups, int dtype, int small, cudaStream_t s) {
+                        const void* comp, double2* out, int n_groups, int dtype, int small, const unsigned int* error,
+                        cudaStream_t s) {
   if (n_groups <= 0) return cudaSuccess;
   const int threads = 256;
   if (small) {
     const int blocks = (n_groups + threads - 1) / threads;
     if (dtype == 0)
-      k_eval_small<double><<<blocks, threads, 0, s>>>(sys, groups, entries, y, comp, out, n_groups);
+      k_eval_small<double><<<blocks, threads, 0, s>>>(sys, groups, entries, y, comp, out, n_groups, error);
     else
-      k_eval_small<float><<<blocks, threads, 0, s>>>(sys, groups, entries, y, comp, out, n_groups);
+      k_eval_small<float><<<blocks, threads, 0, s>>>(sys, groups, entries, y, comp, out, n_groups, error);
     return cudaGetLastError();
   }
   const int blocks = (n_groups * 32 + threads - 1) / threads;
   if (dtype == 0)
-    k_eval<double><<<blocks, threads, 0, s>>>(sys, groups, entries, y, comp, out, n_groups);
+    k_eval<double><<<blocks, threads, 0, s>>>(sys, groups, entries, y, comp, out, n_groups, error);
   else
-    k_eval<float><<<blocks, threads, 0, s>>>(sys, groups, entries, y, comp, out, n_groups);
+    k_eval<float><<<blocks, threads, 0, s>>>(sys, groups, entries, y, comp, out, n_groups, error);
   return cudaGetLastError();
 }
 
@@ -3074,7 +3083,8 @@ cudaError_t launch_eval(const SysDesc* sys, const EvalGroup* groups, const EvalE
 // left (Eq. 11: the sum over the problem's initial conditions), one thread per problem,
 // summed in system order.
 __global__ void k_obs_sum(const double2* __restrict__ obs, const EvalGroup* __restrict__ groups, int n_groups,
-                          double2* __restrict__ out) {
+                          double2* __restrict__ out, const unsigned int* error) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) out_error(error, out);
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= n_groups) return;
   const EvalGroup gr = groups[g];
@@ -3087,10 +3097,11 @@ __global__ void k_obs_sum(const double2* __restrict__ obs, const EvalGroup* __re
   out[g] = make_double2(re, im);
 }
 
-cudaError_t launch_obs_sum(const double2* obs, const EvalGroup* groups, int n_groups, double2* out, cudaStream_t s) {
+cudaError_t launch_obs_sum(const double2* obs, const EvalGroup* groups, int n_groups, double2* out, const unsigned int* error,
+                           cudaStream_t s) {
   if (n_groups <= 0) return cudaSuccess;
   const int threads = 256;
-  k_obs_sum<<<(n_groups + threads - 1) / threads, threads, 0, s>>>(obs, groups, n_groups, out);
+  k_obs_sum<<<(n_groups + threads - 1) / threads, threads, 0, s>>>(obs, groups, n_groups, out, error);
   return cudaGetLastError();
 }
 

@@ -47,6 +47,8 @@ __device__ __forceinline__ void group_sync(int id, int n) {
   asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Conjugate where m is the sign bit, unchanged where m is zero (integer pipe: FP64 is scarce).
 __device__ __forceinline__ float2 conj_if(float2 v, unsigned m) {
   v.y = __uint_as_float(__float_as_uint(v.y) ^ m);
@@ -573,6 +575,16 @@ __global__ void __launch_bounds__(32 * BQ_RES_WARPS(2 * sizeof(T), HERM), sizeof
   const ResGroup g = A.groups[gi];
   if (A.flags && (A.flags[g.sys] != 0) != (A.want != 0)) return;
   const int gt = (int)threadIdx.x - 32 * g.warp0, gn = 32 * g.nwarps;
+  {  // The residual and the parameters are read after the state, each behind a barrier: ask for them now.
+     // (One step of 65 536 systems, whose arrays come from HBM: 1394 -> 1313 us, the streamed step
+     // kernel 1331; 16 384: 358 -> 337; 4096, all in L2: 79 -> 80.)
+    const int eb = 2 * sizeof(T), nc = A.comp_zero ? 0 : g.blk_elems * eb;
+    const char* c = reinterpret_cast<const char*>(A.comp) + (size_t)g.blk_off * eb;
+    for (int o = gt * 128; o < nc; o += gn * 128) prefetch_l2(c + o);
+    const char* b = reinterpret_cast<const char*>(A.params) + g.param_off;
+    const int nb = (int)sizeof(ResHdr) + g.M * (2 * eb + 8 * (int)sizeof(T));
+    for (int o = gt * 128; o < nb; o += gn * 128) prefetch_l2(b + o);
+  }
   const int bar = 1 + g.warp0 / 2;  // groups have at least two warps
   unsigned char* sm = smem_raw + g.smem_off;
   if (gt >= gn - 32) {

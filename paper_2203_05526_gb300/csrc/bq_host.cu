@@ -1122,10 +1122,12 @@ static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, co
   herm = w[0] == w[2] && w[1] == w[3];
   for (int k = 0; k < M && herm; ++k) herm = d[M + k] == std::conj(d[k]);
   herm = herm && same_table(w[4], w[5]) && same_table(w[6], w[7]);
-  blk.resize(sizeof(h));
+  blk.resize(sizeof(h) + (size_t)12 * M * (cs / 2));
+  unsigned char* to = blk.data() + sizeof(h);
   auto put = [&](double v) {
-    if (cs == 16) blk.insert(blk.end(), (unsigned char*)&v, (unsigned char*)&v + 8);
-    else { float f = (float)v; blk.insert(blk.end(), (unsigned char*)&f, (unsigned char*)&f + 4); }
+    const float f = (float)v;
+    std::memcpy(to, cs == 16 ? (const void*)&v : (const void*)&f, cs / 2);
+    to += cs / 2;
   };
   for (const cplx& v : d) { put(v.real()); put(v.imag()); }
   for (auto& v : w)

@@ -2580,6 +2580,14 @@ static cudaError_t enqueue_steps(bq_state* s, double dt, int64_t n, cudaStream_t
 
 static const int kGraphSteps = 64;
 
+// What a replay of bq_step's graph leaves on the host: the flags that enqueue_steps left at its capture
+// (the graph is dropped with the schedule it was captured under).
+static void steps_replayed(bq_state* s) {
+  s->obs_valid = s->use_pipe && s->pipe_obs;
+  s->res_known = 0;
+  s->res_dirty = 1;
+}
+
 extern "C" int bq_step(bq_state* s, double dt, int64_t n_steps, void* stream) {
   if (!s) return fail(BQ_EINVAL, "state is NULL");
   if (n_steps < 0) return fail(BQ_EINVAL, "n_steps < 0");
@@ -2618,6 +2626,7 @@ extern "C" int bq_step(bq_state* s, double dt, int64_t n_steps, void* stream) {
     }
     while (left >= kGraphSteps) {
       CUDA_TRY(cudaGraphLaunch(s->graph, st));
+      steps_replayed(s);
       g_launches += kGraphSteps * kernels_per_step(s);
       left -= kGraphSteps;
     }

@@ -178,3 +178,26 @@ def test_other_forms_keep_the_other_kernels():
     assert gpu_state(_problem(3, measured={((1,), (1,)): 1.0})).get_tune()["resident"] == 0
     assert gpu_state(_problem(9), r_layout="off").get_tune()["resident"] == 0
     assert gpu_state([_problem(9), _problem(43)]).get_tune()["resident"] == 0  # one problem decides for the batch
+
+
+def test_replayed_graphs_leave_no_stale_observables():
+    """bq_step on the one-CTA-per-system kernel (the second call of 64 steps replays its graph) with a
+    resident solve in between: the observables, and the next solve, are those of the current state.
+    (dt: FP32 phases of the highest level stay at O(1) rad, as the tolerance assumes.)"""
+    ps, dt = [_problem(N, steps=200) for N in (6, 13, 16)], 2e-4
+    a, b = gpu_state(ps, dtype="f32"), gpu_state(ps, dtype="f32")
+    a.set_tune(stage_path="system")
+    assert a.get_tune()["resident"] == 1
+    b.set_tune(resident=0)
+    a.step(dt, 64)
+    b.step(dt, 64)
+    a.solve(dt, 5)
+    b.step(dt, 5)
+    before = a.evaluate()
+    a.step(dt, 64)
+    b.step(dt, 64)
+    assert not np.array_equal(a.evaluate(), before)
+    _agree(a, b, "f32")
+    a.solve(dt, 5)
+    b.step(dt, 5)
+    _agree(a, b, "f32")

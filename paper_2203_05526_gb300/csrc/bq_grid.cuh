@@ -806,7 +806,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
 #pragma unroll
   for (int t = 0; t < BQ_GRID_MAXT; ++t) gt[t] = 0.0;
   const long long last = A.n_steps - 1;
-  if (warp == nw - 1) grid_envelope<T>(A, P, E, last & ~7LL, segs);
+  // Both halves of the table: the first step may be the lowest of its eight, whose last stage already
+  // asks for the segment of the step below, and no block boundary lies between.
+  if (warp == nw - 1) {
+    grid_envelope<T>(A, P, E, last & ~7LL, segs);
+    if (last > 7) grid_envelope<T>(A, P, E, (last & ~7LL) - 8, segs);
+  }
   unsigned int block = 0;
   const bool hre = __syncthreads_or(hre_any);
   if (!grid_sync(A.bar, A.error)) return;
@@ -923,8 +928,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
     if (it != last && ((it + 1) & (A.block - 1)) == 0) {
       if (!block_sync(A.bar, ++block, A.error, &dead)) return;
     }
-    // the eight steps below this batch, in its first step (a block boundary, with one before their use)
-    if (((it & 7) == 7 || it == last) && it > 7 && warp == nw - 1) grid_envelope<T>(A, P, E, (it & ~7LL) - 8, segs);
+    // The eight steps below this batch replace those above it, in its first step: the block boundary just
+    // passed ended the reads of the upper batch, and the boundary after the batch's first four steps (blocks
+    // are of four steps at most) comes before the first read, of a segment in its last step.
+    if ((it & 7) == 7 && it != last && it > 7 && warp == nw - 1) grid_envelope<T>(A, P, E, (it & ~7LL) - 8, segs);
 #pragma unroll 1
     for (int stage = 4; stage >= 1; --stage) {
       turn = turn + 1 == A.ring_places ? 0 : turn + 1;

@@ -221,3 +221,25 @@ def test_few_single_mode_systems(instances, N):
     a.solve(ps[0].dt, 5)
     b.step(ps[0].dt, 5)
     _agree(a, b, "f64")
+
+
+@pytest.mark.parametrize("N", [4, 14])
+@pytest.mark.parametrize("every", [9, 10, 11, 12, 16, 17, 25])
+def test_gradient_segments_of_every_remainder(N, every):
+    """Segments of n steps with every n mod 8 that starts the backward sweep in a batch's lowest four
+    steps (and 8 and 16 beside them), the pulse changing its value at every step: the parameter sums are
+    reduced at each change.  Blocks of four steps (N = 4) and of two (N = 14)."""
+    p = configs.two_mode_control(n_seg=25, T=25 * 0.005, steps_per_seg=1, N=N)
+    p.rho0 = {((0, 0), (0, 0)): 0.7, ((1, 0), (0, 1)): 0.1j, ((0, 1), (1, 0)): -0.1j, ((1, 0), (1, 0)): 0.3}
+    a, b = gpu_state(p), gpu_state(p)
+    assert a.get_tune()["resident"] == 1
+    b.set_tune(resident=0)
+    la, ga = a.grad(p.dt, p.n_steps, every)
+    lb, gb = b.grad(p.dt, p.n_steps, every)
+    assert p.n_steps == 25
+    assert abs(la[0] - lb[0]) <= 1e-13 * max(1.0, abs(lb[0]))
+    assert np.max(np.abs(ga - gb)) <= 1e-12 * np.max(np.abs(gb))
+    if N == 4:
+        loss, gt, gp = ograd.loss_and_grad(p, checkpoint_every=every)
+        ref = np.concatenate([gt, gp[0].reshape(-1)])
+        assert np.max(np.abs(ga - ref)) <= 1e-10 * np.max(np.abs(ref))

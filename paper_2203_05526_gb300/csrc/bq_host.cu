@@ -440,7 +440,7 @@ static int compile_problem(const bq_problem* p, const bq_map_opts& o, Compiled& 
   C.diag.assign(doff[ND], cplx(0, 0));
   std::map<std::tuple<int, int, int, int, std::vector<int>>, std::pair<cplx, cplx>> merged;  // (c, cb)
   for (auto& t : raw) {
-    if (t.c == cplx(0, 0)) continue;
+    if (t.c == cplx(0, 0) && t.cb == cplx(0, 0)) continue;  // (at a parameter of 0 only c is 0)
     bool diag = true;
     int nact = 0, dact = -1;
     for (int d = 0; d < ND; ++d) {
@@ -1372,25 +1372,29 @@ static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wba
   for (int t = 0; t < nt; ++t) {
     if (used[t] || term(t).side != bq::SIDE_X) continue;
     const TermDesc& tm = term(t);
-    const cplx a(tm.c_re, tm.c_im);
+    const cplx a(tm.c_re, tm.c_im), cb(tm.cb_re, tm.cb_im);
     const int dl = -tm.deltaGx;
-    auto find = [&](int side, int delta, cplx c, int conj) {
+    // The partner with coefficient f(a), and f(cb) with its parameter set to 1: the kernels take all four
+    // coefficients and their derivatives from this term, and at a parameter of zero every a is 0.  Shifts are
+    // compared in the flat index only: each piece keeps its own weights, and a weight is zero where its source
+    // leaves the grid of a mode.
+    auto find = [&](int side, int delta, cplx (*f)(cplx), int conj) {
       for (int q = 0; q < nt; ++q) {
         const TermDesc& o = term(q);
         if (used[q] || q == t || o.side != side || (side == bq::SIDE_X ? o.deltaGx : o.deltaGy) != delta) continue;
-        if (o.ch != tm.ch || o.param != tm.param || cplx(o.c_re, o.c_im) != c || (o.ch >= 0 && o.conj != conj)) continue;
-        // the same shifts per mode, up to the sign
+        if (o.ch != tm.ch || o.param != tm.param || (o.ch >= 0 && o.conj != conj)) continue;
+        if (cplx(o.c_re, o.c_im) != f(a) || cplx(o.cb_re, o.cb_im) != f(cb)) continue;
         return q;
       }
       return -1;
     };
-    const int xp = find(bq::SIDE_X, dl, -std::conj(a), 1 - tm.conj);
+    const int xp = find(bq::SIDE_X, dl, [](cplx v) { return -std::conj(v); }, 1 - tm.conj);
     if (xp < 0) return false;
     used[t] = used[xp] = 1;
-    const int yp = find(bq::SIDE_Y, dl, -a, tm.conj);
+    const int yp = find(bq::SIDE_Y, dl, [](cplx v) { return -v; }, tm.conj);
     if (yp < 0) return false;
     used[yp] = 1;
-    const int ym = find(bq::SIDE_Y, -dl, std::conj(a), 1 - tm.conj);
+    const int ym = find(bq::SIDE_Y, -dl, [](cplx v) { return std::conj(v); }, 1 - tm.conj);
     if (ym < 0 || G.np == BQ_GRID_MAXP) return false;
     used[ym] = 1;
     const int j = G.np++;

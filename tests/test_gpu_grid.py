@@ -243,3 +243,32 @@ def test_gradient_segments_of_every_remainder(N, every):
         loss, gt, gp = ograd.loss_and_grad(p, checkpoint_every=every)
         ref = np.concatenate([gt, gp[0].reshape(-1)])
         assert np.max(np.abs(ga - ref)) <= 1e-10 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("modes", [1, 2])
+def test_gradients_at_a_parameter_of_zero(modes):
+    """theta = 0: the coefficients of theta's terms are 0, their derivatives are not (they differ between
+    terms, which a comparison of coefficients alone does not see).  Two modes at N = 3, where
+    (a_2^dag)^2 and a_1^dag a_2 shift the flat index alike; one mode with a drive and a detuning."""
+    if modes == 2:
+        p = _driven(3, drive="pwc")
+        p.rho0 = {((0, 0), (0, 0)): 0.6, ((1, 0), (1, 0)): 0.3, ((0, 1), (1, 0)): 0.1j, ((1, 0), (0, 1)): -0.1j}
+        extra = [((0, 2), (0, 0), 1.0), ((1, 0), (0, 1), 0.5j)]
+    else:
+        p = configs.kerr_driven(N=6, dt=0.002, T=18 * 0.002)
+        extra = [((1,), (0,), 0.4 + 0.3j)]
+        p.rho0 = {((0,), (0,)): 0.6, ((1,), (1,)): 0.4, ((0,), (1,)): 0.1j, ((1,), (0,)): -0.1j}
+    q = len(p.params)
+    p.h_terms = list(p.h_terms) + [HTerm(0.3, (1,) + (0,) * (modes - 1), (1,) + (0,) * (modes - 1), param=q)]
+    for u, v, c in extra:
+        p.h_terms += [HTerm(c, u, v, param=q), HTerm(complex(c).conjugate(), v, u, param=q)]
+    p.params = list(p.params) + [0.0]
+    loss, gt, gp = ograd.loss_and_grad(p, checkpoint_every=8)
+    ref = np.concatenate([gt] + [gp[c].reshape(-1) for c in sorted(gp)])
+    assert abs(gt[q]) > 1e-6
+    for kw in (dict(resident=1), dict(resident=0), dict(resident=0, grad_coop=0)):
+        st = gpu_state(p)
+        st.set_tune(**kw)
+        l, g = st.grad(p.dt, p.n_steps, 8)
+        assert abs(l[0] - loss) <= 1e-12 * max(1.0, abs(loss))
+        assert np.max(np.abs(g - ref)) <= 1e-10 * np.max(np.abs(ref)), kw

@@ -1516,7 +1516,7 @@ __global__ void __launch_bounds__(BLK, 2) k_solve_m1(const SolveArgs A) {
 // and <b, T_t u> = <T_t^T b, u>, so the parameter sums need u only at the point itself.
 // The transposed separable source uses the reductions of k_adj_src.
 // ---------------------------------------------------------------------------------------
-#define BQ_MAX_GT 16
+#define BQ_MAX_GT 16  // gradient terms whose sums a thread keeps in registers
 
 __device__ __forceinline__ int pwc_segment(const ChanDesc& cd, const double* par, double t) {
   const double* p = par + cd.par_off;
@@ -1524,6 +1524,12 @@ __device__ __forceinline__ int pwc_segment(const ChanDesc& cd, const double* par
   const double x = floor((t - p[0]) / p[1]);
   if (!(x >= 0.0) || x >= (double)n_seg) return -1;
   return (int)x;
+}
+
+// (a call: inlined, it costs the callers registers on the path of the usual 16 terms or fewer)
+__device__ __noinline__ void add_shared(double* to, double x, double y) {
+  atomicAdd(to, x);
+  atomicAdd(to + 1, y);
 }
 
 // One work item of an adjoint stage (k_adj_stage: one per CTA; the cooperative backward
@@ -1548,10 +1554,15 @@ __device__ __forceinline__ void adj_stage_body(const AdjArgs& A, int item, bool 
   __shared__ int s_ngt, s_nS;
   __shared__ int sidx[BQ_MAX_TERMS];       // ordinal of an S term
   __shared__ double red[BQ_BLOCK / 32][2 * BQ_MAX_GT + 2];  // per-warp sums of the gradient terms
+  // sums of the gradient terms beyond BQ_MAX_GT (rare: 17 and more); zero except between a call that
+  // keeps its sums and the CTA's next
+  __shared__ double more[2 * (BQ_MAX_TERMS - BQ_MAX_GT)];
 
   const int tid = threadIdx.x;
   const int stage = A.stage;
   __syncthreads();  // the CTA's previous item is done with the shared copies
+  if (fresh)
+    for (int i = tid; i < 2 * (BQ_MAX_TERMS - BQ_MAX_GT); i += blockDim.x) more[i] = 0.0;
   if (tid == 0 && fresh) {
     wi = A.work[item];
     sd = A.sys[wi.sys];
@@ -1567,7 +1578,7 @@ __device__ __forceinline__ void adj_stage_body(const AdjArgs& A, int item, bool 
     int g = 0, s = 0;
     for (int t = 0; t < nt; ++t) {
       const TermDesc& td = A.terms[sd.term_off + t];
-      gidx[t] = (td.gslot_param >= 0 || td.gslot_pwc >= 0) && g < BQ_MAX_GT ? g++ : -1;
+      gidx[t] = td.gslot_param >= 0 || td.gslot_pwc >= 0 ? g++ : -1;
       sidx[t] = td.side == SIDE_S ? s++ : -1;
     }
     s_ngt = g;
@@ -1631,6 +1642,10 @@ __device__ __forceinline__ void adj_stage_body(const AdjArgs& A, int item, bool 
     if (g < 0) return;
     const C v = cmul(ub, cscale(bv, w));
     const double vx = (double)v.x, vy = (double)v.y;
+    if (g >= BQ_MAX_GT) {
+      add_shared(more + 2 * (g - BQ_MAX_GT), vx, vy);
+      return;
+    }
     switch (g) {
 #define BQ_GACC_CASE(q) case q: gacc[q].x += vx; gacc[q].y += vy; break;
       BQ_GACC_CASE(0) BQ_GACC_CASE(1) BQ_GACC_CASE(2) BQ_GACC_CASE(3) BQ_GACC_CASE(4) BQ_GACC_CASE(5)
@@ -1815,7 +1830,13 @@ __device__ __forceinline__ void adj_stage_body(const AdjArgs& A, int item, bool 
       const int g = gidx[t];
       if (g >= 0) {
         double2 a = make_double2(0.0, 0.0);
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { a.x += red[w][2 * g]; a.y += red[w][2 * g + 1]; }
+        if (g < BQ_MAX_GT) {
+          for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { a.x += red[w][2 * g]; a.y += red[w][2 * g + 1]; }
+        } else {
+          double* m = more + 2 * (g - BQ_MAX_GT);
+          a = make_double2(m[0], m[1]);
+          m[0] = m[1] = 0.0;
+        }
         const TermDesc& td = st[t];
         double2 e = make_double2(1.0, 0.0);
         double t_phys = 0.0;

@@ -259,3 +259,29 @@ def test_control_problem_full_size():
         b.channels = [Channel("pwc", tuple(pb))]
         fd = (loss_at(a) - loss_at(b)) / (2 * h)
         assert abs(g[3 + j] - fd) <= 1e-5 * max(abs(fd), 1e-3 * np.max(np.abs(g)))
+
+
+@pytest.mark.parametrize("modes", [1, 2])
+@pytest.mark.parametrize("n_terms", [16, 18, 40])
+def test_grad_with_many_gradient_terms(modes, n_terms):
+    """16, 18 and 40 stencil terms that carry a gradient (the adjoint kernels keep the sums of 16 in
+    registers), against the oracle's adjoint, on the cooperative segments and per stage."""
+    from workloads.spec import HTerm, Problem
+    p = _small_control(n_modes=modes, N=4)
+    h, params = [t for t in p.h_terms if t.param < 0], []
+    have = 2 * sum(1 for t in h if t.channel >= 0)  # a left and a right stencil term each
+    while have < n_terms:
+        q = len(params)
+        u = tuple(int(j == q % modes) for j in range(modes))
+        h.append(HTerm(0.3 + 0.05 * q, u, u, param=q))
+        params.append(0.02 + 0.01 * q)
+        have += 2
+    p = Problem(**{**p.__dict__, "h_terms": h, "params": params})
+    loss_o, gt, gp = ograd.loss_and_grad(p, checkpoint_every=5)
+    ref = _flat_oracle(gt, gp)
+    for coop in (1, 0):
+        st = gpu_state(p)
+        st.set_tune(grad_coop=coop, resident=0)
+        loss, g = st.grad(p.dt, p.n_steps, 5)
+        assert abs(loss[0] - loss_o) <= 1e-12 * max(1.0, abs(loss_o))
+        assert np.max(np.abs(g - ref)) <= 1e-10 * np.max(np.abs(ref)), (coop, g, ref)

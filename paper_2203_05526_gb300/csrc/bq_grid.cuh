@@ -466,10 +466,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
     } else {  // (w_lo is zero)
       d.x = fma(w_hi, s.x, -cv.x);
       d.y = fma(w_hi, s.y, -cv.y);
-      nu.x = yv.x + d.x;
-      nu.y = yv.y + d.y;
-      cv.x = (nu.x - yv.x) - d.x;
-      cv.y = (nu.y - yv.y) - d.y;
+      if (A.single_mode) {
+        sum_ordered(yv, d, nu, e);
+        cv = cneg(e);
+      } else {  // Fast2Sum, as the tiled kernel's: exact unless the increment is larger than the element
+        nu.x = yv.x + d.x;
+        nu.y = yv.y + d.y;
+        cv.x = (nu.x - yv.x) - d.x;
+        cv.y = (nu.y - yv.y) - d.y;
+      }
     }
     return nu;
   };

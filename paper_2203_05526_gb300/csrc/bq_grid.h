@@ -72,6 +72,7 @@ struct GridArgs {
   double* grad;
   const double2* dc;
   int comp_zero, reverse, n_steps;
+  int single_mode;  // FP64: the state update is error-free whatever the increment (as in the single-mode kernels)
   int herm;       // the pieces hold the Hermitian problems in the Hermitian layout
   long long step0;      // the first step is at tau0 + step0 dt
   double dt, tau0, horizon;

@@ -2425,6 +2425,7 @@ static bq::GridArgs grid_args(bq_state* s, int q, double dt) {
   a.error = (unsigned int*)(b + L.off_ctrl + 32);
   a.dc = (const double2*)(b + L.off_dc);
   a.reverse = s->reverse;
+  a.single_mode = s->use_m1;
   a.herm = q == 0;
   a.dt = dt;
   a.horizon = s->horizon;

@@ -16,7 +16,7 @@
 // What it replaces and measured (one GB300): the streamed step kernel was bound by HBM traffic
 // and issue, the earlier persistent solve by issue (160 instructions per point and stage, most of
 // them loads and rebuilding of per-stage coefficients).  4096 ragged FP32 oscillators (N 10..40):
-// 84 -> 18.6 us per step; 16 384: 351 -> 79; 1024 in FP64: 413 -> 118; one in FP32 (N = 40):
+// 84 -> 18.6 us per step; 16 384: 351 -> 79; 1024 in FP64: 413 -> 120; one in FP32 (N = 40):
 // 14.2 -> 2.0; one in FP64: 145 -> 36.  What bounds it now: in FP32 shared-memory wavefronts and
 // issue about equally (a half each, 20 warps per SM to hide the latencies); in FP64 the FP64 pipe
 // (88%).
@@ -59,21 +59,13 @@ __device__ __forceinline__ double2 conj_if(double2 v, unsigned m) {
   return v;
 }
 
-// y + d exactly as (y, -comp): TwoSum in FP32 (the increment may exceed a small element); in FP64
-// Fast2Sum, whose error where |d| > |y| is of the order of the rounding of d itself.
-__device__ __forceinline__ void res_update(float2 d, float2& y, float2& c) {
-  float2 t, e;
-  two_sum(y, d, t, e);
+// y + d exactly as (y, -comp), whichever of the two is larger.
+template <typename C>
+__device__ __forceinline__ void res_update(C d, C& y, C& c) {
+  C t, e;
+  sum_ordered(y, d, t, e);
   y = t;
   c = cneg(e);
-}
-__device__ __forceinline__ void res_update(double2 d, double2& y, double2& c) {
-  double2 t;
-  t.x = y.x + d.x;
-  t.y = y.y + d.y;
-  c.x = (t.x - y.x) - d.x;
-  c.y = (t.y - y.y) - d.y;
-  y = t;
 }
 
 // Products of the off-diagonal coefficient: a p - conj(a) q added to k.

@@ -201,3 +201,50 @@ def test_replayed_graphs_leave_no_stale_observables():
     a.solve(dt, 5)
     b.step(dt, 5)
     _agree(a, b, "f32")
+
+
+@pytest.mark.parametrize("measured", [None, GENERAL])
+@pytest.mark.parametrize("instances", [1, 200])
+def test_fp64_update_keeps_the_bits_of_elements_below_their_increment(instances, measured):
+    """A step's update is error-free in FP64 as on the streaming kernels, also where the increment is the
+    larger operand: elements of 2^-100 with increments above 2^-40 are left as the sum's residual.  One
+    system (the grid kernel) and 200 (the resident kernel)."""
+    import torch
+    ps = [_problem(24, measured=measured) for _ in range(instances)]
+    a, b = gpu_state(ps, dtype="f64"), gpu_state(ps, dtype="f64")
+    assert a.get_tune()["resident"] == 1
+    b.set_tune(resident=0)
+    eps, n = 2.0 ** -100, 24
+    info = [a.system_info(i) for i in range(a.n_systems())]
+    host = torch.zeros(a.state_bytes() // 16, dtype=torch.complex128)
+    rng, off, small = np.random.default_rng(3), 0, []
+    for s in info:
+        z = rng.normal(size=(n, n)) + 1j * rng.normal(size=(n, n))
+        z = z + z.conj().T
+        for i in range(0, n - 2, 3):
+            z[i, i + 2] = z[i + 2, i] = eps
+        g = rng.normal(size=n) + 1j * rng.normal(size=n)
+        for v, m in ((g, s["n_gx"]), (g.conj(), s["n_gy"]), (z.reshape(-1), s["n_r"])):
+            host[off:off + m] = torch.from_numpy(v)
+            if m > n:
+                small += [off + i * n + i + 2 for i in range(0, n - 2, 3)]
+            off += (m + 3) & ~3
+    host = host.pin_memory()
+
+    def residual(st):
+        """The rounding residual of the state, which follows the state in the pool."""
+        st.load_state(host.data_ptr())
+        st.step(ps[0].dt, 1)
+        y = torch.empty(st.state_bytes(), dtype=torch.uint8, pin_memory=True)
+        st.store_state(y.data_ptr())
+        torch.cuda.synchronize()
+        y, pool = y.numpy().tobytes(), st.pool.cpu().numpy().tobytes()
+        at = pool.find(y)
+        assert at >= 0
+        at = (at + len(y) + 255) // 256 * 256
+        return np.frombuffer(y, complex)[small], np.frombuffer(pool[at:at + len(y)], complex)[small]
+
+    for st in (b, a):
+        y, c = residual(st)
+        assert np.min(np.abs(y.real)) > 2.0 ** -40
+        assert np.all(c.real == -eps)

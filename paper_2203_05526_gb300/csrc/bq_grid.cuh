@@ -54,14 +54,25 @@ __device__ __forceinline__ bool grid_sync(unsigned int* bar, unsigned int* error
 template <typename T>
 struct GridTab {
   using C = typename C2T<T>::type;
-  const C *dx, *dy;
+  const C* d;  // hi parts of dx, dy, then their lo parts
   const T* w;
   int ng, np, ns;
   // b: the problem's tables
   __device__ __forceinline__ GridTab(const GridProb& p, const T* b) : ng(p.ng), np(p.np), ns(p.ns) {
-    dx = reinterpret_cast<const C*>(b);
-    dy = dx + ng;
-    w = b + 4 * ng;
+    d = reinterpret_cast<const C*>(b);
+    w = b + 8 * ng;
+  }
+  // a + b + c, rounded (almost) once: a and b may cancel to far below their size
+  static __device__ __forceinline__ C sum3(C a, C b, C c) {
+    C s, e;
+    two_sum(a, b, s, e);
+    return cadd(s, cadd(e, c));
+  }
+  // diagonal coefficient of (k, l) of R, and of point k of G_x (side 0) or G_y (side 1) with c = C or -C
+  __device__ __forceinline__ C diag(int k, int l) const { return sum3(d[k], d[ng + l], cadd(d[2 * ng + k], d[3 * ng + l])); }
+  __device__ __forceinline__ C diag(int side, int k, double c_re, double c_im) const {
+    const C hi = cmk<C>(c_re, c_im);
+    return sum3(d[side * ng + k], hi, cadd(d[(2 + side) * ng + k], cmk<C>(c_re - (double)hi.x, c_im - (double)hi.y)));
   }
   __device__ __forceinline__ const T* pair(int j, int q) const { return w + (4 * j + q) * ng; }  // xm xp ym yp
   __device__ __forceinline__ const T* sand(int j, int q) const { return w + (4 * np + 2 * j + q) * ng; }
@@ -385,9 +396,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
       const int i = g.kind == GRID_H ? g.off_r + p.k * ng + p.l : self;
       yv = reinterpret_cast<const C*>(A.y)[i];
       if (!A.comp_zero) cv = reinterpret_cast<const C*>(A.comp)[i];
-      if (g.kind <= GRID_D) dg = cadd(W.dx[p.k], W.dy[p.l]);
-      else if (g.kind == GRID_X) dg = cadd(W.dx[p.k], cmk<C>(g.c_re, g.c_im));
-      else dg = cadd(W.dy[p.k], cmk<C>(-g.c_re, -g.c_im));
+      if (g.kind <= GRID_D) dg = W.diag(p.k, p.l);
+      else if (g.kind == GRID_X) dg = W.diag(0, p.k, g.c_re, g.c_im);
+      else dg = W.diag(1, p.k, -g.c_re, -g.c_im);
       auto put = [&](int j, T w, int o, unsigned conj) {
         if (w == (T)0) return;
         S.w[j * n + pi] = w;
@@ -754,9 +765,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
       for (int r = 0; r < places; ++r)
         if (r != 1) slot_put(ring + r * place + slot_of<C>(self), zero, 0u);
       slot_put(ring + place + slot_of<C>(self), cscale(v, w6), 1u);
-      if (g.kind <= GRID_D) dg = cadd(W.dx[k], W.dy[l]);
-      else if (g.kind == GRID_X) dg = cadd(W.dx[k], cmk<C>(g.c_re, g.c_im));
-      else dg = cadd(W.dy[k], cmk<C>(-g.c_re, -g.c_im));
+      if (g.kind <= GRID_D) dg = W.diag(k, l);
+      else if (g.kind == GRID_X) dg = W.diag(0, k, g.c_re, g.c_im);
+      else dg = W.diag(1, k, -g.c_re, -g.c_im);
       auto put = [&](int j, T w, int o) {
         if (w == (T)0) return;
         S.w[j * n + pi] = w;

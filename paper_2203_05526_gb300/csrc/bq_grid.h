@@ -18,7 +18,7 @@
 namespace bq {
 
 // Per-problem tables, element type of the state, n_g entries each, from element offset tab (in
-// reals): dx, dy (complex), then per pair xm xp ym yp (real), per sandwich term sx sy (real);
+// reals): dx, dy, then what they lack of the exact sums (complex), then per pair xm xp ym yp (real), per sandwich term sx sy (real);
 // for the adjoint the same weights at the transposed sources: per pair xmT xpT ymT ypT, per
 // sandwich term sxT syT; per diagonal parameter hx hy (complex).
 struct GridProb {

@@ -244,12 +244,38 @@ struct RawTerm {
   int a[BQ_MAXD], b[BQ_MAXD];
 };
 
+// A sum of doubles and products with its rounding errors carried along.
+struct PairSum {
+  double hi = 0.0, lo = 0.0;
+  void add(double v) {
+    const double s = hi + v, b = s - hi;
+    lo += (hi - (s - b)) + (v - b);
+    hi = s;
+  }
+  void add(double a, double b) {
+    const volatile double p = a * b;  // (rounded here: not contracted into a sum)
+    add(p);
+    lo += std::fma(a, b, -p);
+  }
+  void add(const PairSum& o) {
+    add(o.hi);
+    lo += o.lo;
+  }
+  // as hi and lo in the state's precision
+  void put(bool f32, double& h, double& l) const {
+    const double s = hi + lo, e = lo - (s - hi);
+    h = f32 ? (double)(float)s : s;
+    l = (s - h) + e;
+  }
+};
+
 struct Compiled {
   int nm, M[BQ_MAX_MODES], method, basis, has_sep, has_r, r_diag = 0;
   int n_g, n_r;
   std::vector<TermDesc> terms;         // wtab offsets relative to this problem's weight block
   std::vector<double> wtab;            // weight tables
   std::vector<cplx> diag;              // 2*nm tables
+  std::vector<PairSum> diag_sum[2];    // their real and imaginary parts to twice the precision (empty: not wanted)
   struct Sys {
     int p_flat, q_flat;
     cplx w, C;
@@ -360,7 +386,8 @@ static void jacobi_svd(int n, std::vector<cplx>& W, std::vector<cplx>& V) {
   }
 }
 
-static int compile_problem(const bq_problem* p, const bq_map_opts& o, Compiled& C) {
+// want_sums: the diagonal tables to twice the precision too (the grid-resident kernels)
+static int compile_problem(const bq_problem* p, const bq_map_opts& o, bool want_sums, Compiled& C) {
   const int nm = p->nm;
   C.nm = nm;
   C.method = o.method;
@@ -438,6 +465,7 @@ static int compile_problem(const bq_problem* p, const bq_map_opts& o, Compiled& 
   std::vector<int> doff(ND + 1, 0);
   for (int d = 0; d < ND; ++d) doff[d + 1] = doff[d] + Md[d];
   C.diag.assign(doff[ND], cplx(0, 0));
+  for (auto& v : C.diag_sum) v.assign(want_sums ? doff[ND] : 0, PairSum());
   std::map<std::tuple<int, int, int, int, std::vector<int>>, std::pair<cplx, cplx>> merged;  // (c, cb)
   for (auto& t : raw) {
     if (t.c == cplx(0, 0) && t.cb == cplx(0, 0)) continue;  // (at a parameter of 0 only c is 0)
@@ -454,6 +482,10 @@ static int compile_problem(const bq_problem* p, const bq_map_opts& o, Compiled& 
         for (int i = 0; i < t.a[d]; ++i) w *= (double)(k - i);  // k!/(k-a)!
         if (k < t.a[d]) w = 0.0;
         C.diag[doff[d] + k] += t.c * w;
+        if (want_sums) {
+          C.diag_sum[0][doff[d] + k].add(t.c.real(), w);
+          C.diag_sum[1][doff[d] + k].add(t.c.imag(), w);
+        }
       }
       continue;
     }
@@ -523,6 +555,8 @@ static int compile_problem(const bq_problem* p, const bq_map_opts& o, Compiled& 
       const double a = m * (1.0 + sh.nb(m - 1)) + (m + 1) * sh.nb(m);
       C.diag[doff[j] + m] += -0.5 * sh.kappa * a;
       C.diag[doff[nm + j] + m] += -0.5 * sh.kappa * a;
+      if (want_sums)
+        for (int d : {j, nm + j}) C.diag_sum[0][doff[d] + m].add(-0.5 * sh.kappa, a);
     }
     if (!C.has_r) continue;
     bool any_up = false;
@@ -1298,7 +1332,7 @@ static std::vector<double> flat_weights(const Compiled& C, const TermDesc& td, i
   return w;
 }
 
-static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wbase, int grad_off, bq::GridProb& G,
+static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wbase, int grad_off, bool f32, bq::GridProb& G,
                          std::vector<double>& tab, bool& herm) {
   const int ng = C.n_g, nm = C.nm;
   std::memset(&G, 0, sizeof(G));
@@ -1306,15 +1340,26 @@ static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wba
   G.has_sep = C.has_sep; G.has_r = C.has_r; G.r_diag = C.r_diag;
   G.n_params = C.n_params;
   G.grad_off = grad_off;
-  std::vector<cplx> d[2];
+  // The diagonal coefficient of a point is the difference of two large sums over the modes (in the lab
+  // frame; equal for a permuted index): each is kept to twice the precision (hi, lo).  With sums rounded
+  // per side the error of a three-mode direct run against 80-bit arithmetic was 2.5 times the tiled
+  // kernel's, which adds mode by mode; so it is 0.3 to 1.1 times.  (One mode has no sum.)
+  const bool sums = !C.diag_sum[0].empty();
+  std::vector<PairSum> d[2][2];  // side, real / imaginary part
   for (int y = 0; y < 2; ++y) {
-    d[y].assign(ng, cplx(0, 0));
+    for (auto& v : d[y]) v.resize(ng);
     for (int k = 0; k < ng; ++k) {
       int r = k;
       for (int j = nm - 1; j >= 0; --j) {
         int off = 0;
         for (int q = 0; q < y * nm + j; ++q) off += C.M[q % nm];
-        d[y][k] += C.diag[off + r % C.M[j]];
+        const int i = off + r % C.M[j];
+        if (sums) {
+          for (int q = 0; q < 2; ++q) d[y][q][k].add(C.diag_sum[q][i]);
+        } else {
+          d[y][0][k].add(C.diag[i].real());
+          d[y][1][k].add(C.diag[i].imag());
+        }
         r /= C.M[j];
       }
     }
@@ -1351,7 +1396,10 @@ static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wba
     if (shift0) {
       if (td.ch >= 0) return false;
       const std::vector<double> w = flat_weights(C, td, wbase, y);
-      for (int k = 0; k < ng; ++k) d[y][k] += c * w[k];
+      for (int k = 0; k < ng; ++k) {
+        d[y][0][k].add(c.real(), w[k]);
+        d[y][1][k].add(c.imag(), w[k]);
+      }
       if (td.gslot_param >= 0) {
         int q = 0;
         while (q < G.nt && G.tpar[q] != td.gslot_param) ++q;
@@ -1420,10 +1468,18 @@ static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wba
   }
   for (int t = 0; t < nt; ++t)
     if (!used[t]) return false;
+  std::vector<cplx> dh[2], dl[2];
+  for (int y = 0; y < 2; ++y)
+    for (int k = 0; k < ng; ++k) {
+      double h[2], l[2];
+      for (int q = 0; q < 2; ++q) d[y][q][k].put(f32, h[q], l[q]);
+      dh[y].push_back(cplx(h[0], h[1]));
+      dl[y].push_back(cplx(l[0], l[1]));
+    }
   // Hermitian structure: mirrored weights
   herm = C.has_r && !C.r_diag && ng >= 4;
   for (int k = 0; k < ng && herm; ++k) {
-    herm = d[1][k] == std::conj(d[0][k]);
+    herm = dh[1][k] == std::conj(dh[0][k]) && dl[1][k] == std::conj(dl[0][k]);
     for (int j = 0; j < G.np && herm; ++j) herm = pw[4 * j][k] == pw[4 * j + 2][k] && pw[4 * j + 1][k] == pw[4 * j + 3][k];
   }
   for (int s = 0; s < G.ns && herm; ++s) herm = same_table(sw[2 * s], sw[2 * s + 1]);
@@ -1439,8 +1495,8 @@ static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wba
   };
   while (tab.size() % 2) tab.push_back(0.0);
   G.tab = (long long)tab.size();
-  putc(d[0]);
-  putc(d[1]);
+  for (int y = 0; y < 2; ++y) putc(dh[y]);
+  for (int y = 0; y < 2; ++y) putc(dl[y]);
   for (auto& w : pw) putr(w);
   for (auto& w : sw) putr(w);
   for (int j = 0; j < G.np; ++j) {  // sources k - dlt, k + dlt, l - dlt, l + dlt
@@ -1492,7 +1548,7 @@ static void make_grid_plan(Plan& P, const bq_problem* const* probs, const bq_map
   for (int b = 0; b < B; ++b) {
     bq::GridProb G;
     bool hm = false;
-    if (!grid_problem(P, P.comp[b], term_off[b], P.wbase[b], P.grad_offs[b], G, P.gtab, hm)) {
+    if (!grid_problem(P, P.comp[b], term_off[b], P.wbase[b], P.grad_offs[b], o.dtype == BQ_F32, G, P.gtab, hm)) {
       P.gprobs.clear();
       P.gtab.clear();
       return;
@@ -1596,7 +1652,7 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
   for (int b = 0; b < B; ++b) {
     if (!probs[b]) return fail(BQ_EINVAL, "problem %d is NULL", b);
     if (probs[b]->nm != nm) return fail(BQ_EINVAL, "all problems of a batch need the same number of modes");
-    int r = compile_problem(probs[b], *o, P.comp[b]);
+    int r = compile_problem(probs[b], *o, nm > 1 && B <= BQ_GRID_MAX_CTAS, P.comp[b]);
     if (r != BQ_OK) return r;
     Compiled& C = P.comp[b];
     if (C.sys.empty()) return fail(BQ_EINVAL, "problem %d: measured operator is zero on the grid", b);

@@ -3,6 +3,7 @@
 states, both precisions, gradients, and the forms they must leave to the tiled kernels."""
 
 import dataclasses
+import itertools
 
 import numpy as np
 import pytest
@@ -272,3 +273,26 @@ def test_gradients_at_a_parameter_of_zero(modes):
         l, g = st.grad(p.dt, p.n_steps, 8)
         assert abs(l[0] - loss) <= 1e-12 * max(1.0, abs(loss))
         assert np.max(np.abs(g - ref)) <= 1e-10 * np.max(np.abs(ref)), kw
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_frequencies_that_cancel_cancel_exactly(dtype):
+    """Three equal uncoupled oscillators in the lab frame: between permutations of the same occupation numbers
+    the frequencies cancel, and such elements of A do not change (rounded sums over the modes differ with
+    the order: the test takes the permutations where they do)."""
+    N, w, eta = 5, 20.1, 1.3
+    unit = lambda j, x: tuple(x if i == j else 0 for i in range(3))  # noqa: E731
+    d = [(np.float64 if dtype == "f64" else np.float32)(w * k + eta * k * (k - 1)) for k in range(N)]
+    meas = {}
+    for k in itertools.permutations(range(N), 3):
+        if d[k[0]] + d[k[1]] + d[k[2]] != d[k[1]] + d[k[2]] + d[k[0]]:
+            meas[(k, k[1:] + k[:1])] = 1.0 + 0.5j
+    assert meas
+    h = [HTerm(w, unit(j, 1), unit(j, 1)) for j in range(3)] + [HTerm(eta, unit(j, 2), unit(j, 2)) for j in range(3)]
+    q = configs.table_one_network(3, N, steps=4000)
+    p = dataclasses.replace(q, h_terms=h, channels=[], secular=[], jumps=[], measured=meas, T=40 * q.dt)
+    st = gpu_state(p, dtype=dtype, method="direct")
+    assert st.get_tune()["resident"] == 1
+    before = _raw(st, dtype)
+    st.step(p.dt, 40)
+    assert np.array_equal(_raw(st, dtype), before)

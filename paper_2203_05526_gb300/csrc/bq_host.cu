@@ -1537,7 +1537,7 @@ static size_t grid_count(const std::vector<SysDesc>& sys, const std::vector<bq::
 static void make_grid_plan(Plan& P, const bq_problem* const* probs, const bq_map_opts& o) {
   const int B = (int)P.comp.size();
   int64_t pts = 0;
-  for (const SysDesc& sd : P.sys) pts += sd.n_r + 2 * (sd.has_sep ? sd.n_g : 0);
+  for (const SysDesc& sd : P.sys) pts += (sd.has_r ? sd.n_r : 0) + 2 * (sd.has_sep ? sd.n_g : 0);
   if (P.total_elems >= ((int64_t)1 << 31) || pts > kGridMaxPoints || B > kGridMaxCtas) return;
   std::vector<int> term_off(B, 0);
   std::vector<char> herm(B, 1);

@@ -6,7 +6,7 @@
 
 #include "bq_internal.h"
 
-#define BQ_GRID_MAX_CTAS 256
+#define BQ_GRID_MAX_CTAS 152  // one per SM of a GB300
 #define BQ_GRID_MAXP 8   // off-diagonal pairs of a problem
 #define BQ_GRID_MAXS 4   // sandwich terms
 #define BQ_GRID_MAXT 4   // parameters that multiply diagonal terms

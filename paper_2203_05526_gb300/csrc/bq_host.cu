@@ -817,7 +817,7 @@ struct bq_state {
   ResList rlist[3];
   // grid-resident kernels: lists (forward Hermitian, forward general, adjoint) and variant sizes
   GridList glist[3];
-  int grid_np = 0, grid_ns = 0, grid_herm = 0;
+  int grid_np = 0, grid_ns = 0, grid_herm = 0, grid_fit[3] = {0, 0, 0};  // fit: the pool has room for the list
   int grid_few = 0;  // single-mode: bq_step and bq_solve take the grid-resident kernel
   int grid_pieces = 0, grid_adj = 0;  // pieces in the pool so far; the adjoint's list has been built
   std::vector<bq::GridProb> gprobs;
@@ -909,7 +909,7 @@ struct Plan {
   std::vector<bq::ResBin> rbins;
   ResList rlist[3];
   // grid-resident kernels (k_grid_fwd, k_grid_adj): problems, tables, capacity of the lists' pieces
-  int grid_ok = 0, grid_np = 0, grid_ns = 0, grid_herm = 0, grid_few = 0;
+  int grid_ok = 0, grid_np = 0, grid_ns = 0, grid_herm = 0, grid_few = 0, grid_fit[3] = {0, 0, 0};
   size_t grid_cap = 0;
   std::vector<bq::GridProb> gprobs;
   std::vector<double> gtab;
@@ -1302,7 +1302,7 @@ static void make_res_plan(Plan& P, const bq_problem* const* probs, const std::ve
 // shared memory holds.
 // ---------------------------------------------------------------------------------------
 static const int kGridMaxCtas = BQ_GRID_MAX_CTAS;
-static const int64_t kGridMaxPoints = 152 * 2500;
+static const int64_t kGridMaxPoints = kGridMaxCtas * 2500;  // (more stored points never fit: not worth a plan)
 // Few single-mode systems in FP64 take the grid-resident kernel: the resident kernel keeps a system on
 // one SM, whose FP64 pipe then takes longer for a stage than the exchange between SMs does.  Measured
 // (us per step, resident / grid): one system N = 16 10.0 / 8.8, N = 20 10.8 / 9.0, N = 40 34.9 / 9.7;
@@ -1528,10 +1528,41 @@ static void grid_kinds(const SysDesc& sd, const bq::GridProb& G, int list, F f) 
     if (!hm) f(bq::GRID_Y, sd.n_g, len);
   }
 }
-static size_t grid_count(const std::vector<SysDesc>& sys, const std::vector<bq::GridProb>& probs, int list) {
-  size_t n = 0;
-  for (const SysDesc& sd : sys) grid_kinds(sd, probs[sd.prob], list, [&](int, int pts, int len) { n += (pts + len - 1) / len; });
-  return n;
+// The largest share of pieces of a CTA when a list is spread over at most nsm CTAs, every CTA within one
+// problem (the adjoint: one system), with the kernel's form and shared memory; share 0: it does not fit
+// in smem_max bytes a CTA.
+struct GridShape {
+  int share = 0, form = 0;
+  size_t smem = 0, pieces = 0;
+};
+static GridShape grid_shape(const std::vector<SysDesc>& sys, const std::vector<bq::GridProb>& probs, int list, int dtype,
+                            int nsm, size_t smem_max) {
+  GridShape g;
+  std::vector<size_t> unit;
+  int last = -1;
+  for (int i = 0; i < (int)sys.size(); ++i) {
+    const int u = list == 2 ? i : sys[i].prob;
+    if (u != last) {  // (a problem's systems are contiguous)
+      if ((int)unit.size() == nsm) return g;
+      unit.push_back(0);
+      last = u;
+    }
+    grid_kinds(sys[i], probs[sys[i].prob], list, [&](int, int pts, int len) { unit.back() += (pts + len - 1) / len; });
+  }
+  for (size_t n : unit) g.pieces += n;
+  int share = std::max(1, (int)((g.pieces + nsm - 1) / nsm));
+  for (;; ++share) {
+    size_t n = 0;
+    for (size_t v : unit) n += (v + share - 1) / share;
+    if (n <= (size_t)nsm) break;
+  }
+  g.form = share <= 8 ? bq::GRID_ONE : bq::GRID_MANY;
+  for (const bq::GridProb& p : probs)
+    if (g.form == bq::GRID_ONE && !bq::grid_small(p, list == 2)) g.form = bq::GRID_FEW;
+  for (const bq::GridProb& p : probs)
+    g.smem = std::max(g.smem, bq::grid_smem(share, p, list == 2, g.form, dtype == BQ_F64 ? 16 : 8));
+  if (g.smem <= smem_max) g.share = share;
+  return g;
 }
 
 static void make_grid_plan(Plan& P, const bq_problem* const* probs, const bq_map_opts& o) {
@@ -1565,32 +1596,45 @@ static void make_grid_plan(Plan& P, const bq_problem* const* probs, const bq_map
     P.grid_ns = std::max(P.grid_ns, G.ns);
     P.gprobs.push_back(G);
   }
-  for (int list = P.grid_herm ? 0 : 1; list < 3; ++list) P.grid_cap += grid_count(P.sys, P.gprobs, list);
+  // Lists that the largest grid may hold, at an SM's whole shared memory: nothing is reserved for others.
+  // (bq_map decides for the device and the kernels' own limit.)
+  for (int list = P.grid_herm ? 0 : 1; list < 3; ++list) {
+    const GridShape g = grid_shape(P.sys, P.gprobs, list, o.dtype, kGridMaxCtas, 227 * 1024);
+    P.grid_fit[list] = g.share > 0;
+    if (P.grid_fit[list]) P.grid_cap += g.pieces;
+  }
+  if (!P.grid_fit[1]) {
+    P.gprobs.clear();
+    P.gtab.clear();
+    P.grid_cap = 0;
+    return;
+  }
   P.grid_ok = 1;
   int m = 0;
   for (const bq::GridProb& g : P.gprobs) m = std::max(m, g.ng);
-  P.grid_few = P.res_ok && o.dtype == BQ_F64 && B <= kGridFewSystems && (B > 1 || m >= kGridFewM);
+  P.grid_few = P.res_ok && o.dtype == BQ_F64 && (!P.grid_herm || P.grid_fit[0]) && B <= kGridFewSystems && (B > 1 || m >= kGridFewM);
 }
 
 // The pieces of a list (0: forward, Hermitian layout where possible; 1: forward, general layout; 2:
-// adjoint), spread over at most nsm CTAs with the smallest largest share, every CTA within one
-// problem (the adjoint: one system).  A unit's pieces are dealt out to its CTAs in turn, since the
-// kinds differ in cost.  gl.n_ctas is 0 where the list does not fit.
+// adjoint).  A unit's pieces are dealt out to its CTAs in turn, since the kinds differ in cost.
+// gl.n_ctas is 0 where the list does not fit.
 static int build_grid_list(const std::vector<SysDesc>& sys, const std::vector<bq::GridProb>& probs, int list, int dtype,
                            int np, int ns, std::vector<bq::GridPiece>& pieces, std::vector<bq::GridCta>& ctas, GridList& gl) {
   int dev = 0, nsm = 0;
   CUDA_TRY(cudaGetDevice(&dev));
   CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  nsm = std::min(nsm, kGridMaxCtas);
   gl.n_ctas = gl.smem = 0;
+  const GridShape shape = grid_shape(sys, probs, list, dtype, std::min(nsm, kGridMaxCtas), BQ_GRID_SMEM_MAX);
+  int most = 0;
+  if (shape.share) CUDA_TRY(bq::grid_max_ctas(dtype, np, ns, list == 2, shape.form, (int)shape.smem, &most));
+  if (!most) return BQ_OK;
+  const int share = shape.share;
   std::vector<std::vector<bq::GridPiece>> unit;
-  size_t total = 0;
   int last = -1;
   for (int i = 0; i < (int)sys.size(); ++i) {
     const SysDesc& sd = sys[i];
     const int u = list == 2 ? i : sd.prob;
-    if (u != last) {  // (a problem's systems are contiguous)
-      if ((int)unit.size() == nsm) return BQ_OK;
+    if (u != last) {
       unit.emplace_back();
       last = u;
     }
@@ -1604,14 +1648,7 @@ static int build_grid_list(const std::vector<SysDesc>& sys, const std::vector<bq
         g.dc_off = sd.dc_off;
         unit.back().push_back(g);
       }
-      total += (pts + len - 1) / len;
     });
-  }
-  int share = std::max(1, (int)((total + nsm - 1) / nsm));
-  for (;; ++share) {
-    size_t n = 0;
-    for (auto& v : unit) n += (v.size() + share - 1) / share;
-    if (n <= (size_t)nsm) break;
   }
   pieces.clear();
   ctas.clear();
@@ -1624,17 +1661,10 @@ static int build_grid_list(const std::vector<SysDesc>& sys, const std::vector<bq
       ctas.push_back(cta);
     }
   }
-  int form = share <= 8 ? bq::GRID_ONE : bq::GRID_MANY;
-  for (const bq::GridProb& g : probs)
-    if (form == bq::GRID_ONE && !bq::grid_small(g, list == 2)) form = bq::GRID_FEW;
-  size_t sm = 0;
-  for (const bq::GridProb& g : probs) sm = std::max(sm, bq::grid_smem(share, g, list == 2, form, dtype == BQ_F64 ? 16 : 8));
-  int most = 0;
-  if (sm <= BQ_GRID_SMEM_MAX) CUDA_TRY(bq::grid_max_ctas(dtype, np, ns, list == 2, form, (int)sm, &most));
   if (most < (int)ctas.size()) return BQ_OK;
   gl.n_ctas = (int)ctas.size();
-  gl.smem = (int)sm;
-  gl.form = form;
+  gl.smem = (int)shape.smem;
+  gl.form = shape.form;
   return BQ_OK;
 }
 
@@ -2232,8 +2262,10 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
   int grid_pieces = 0;
   if (P.grid_ok) {
     for (int q = P.use_m1 && !P.grid_few ? 2 : P.grid_herm ? 0 : 1; q < 2; ++q) {
+      if (!P.grid_fit[q]) continue;
       r = build_grid_list(P.sys, P.gprobs, q, o->dtype, P.grid_np, P.grid_ns, gpieces[q], gctas[q], glist[q]);
       if (r != BQ_OK) return r;
+      if (!glist[q].n_ctas) continue;
       for (bq::GridCta& c : gctas[q]) c.p0 += grid_pieces;
       CUDA_TRY(up(L.off_gpieces + grid_pieces * sizeof(bq::GridPiece), gpieces[q].data(), gpieces[q].size() * sizeof(bq::GridPiece)));
       glist[q].c0 = q * kGridMaxCtas;
@@ -2301,7 +2333,7 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
   st->res_variant = P.res_variant;
   st->res_obs = P.res_obs;
   for (int q = 0; q < 3; ++q) st->rlist[q] = P.rlist[q];
-  for (int q = 0; q < 3; ++q) st->glist[q] = glist[q];
+  for (int q = 0; q < 3; ++q) st->glist[q] = glist[q], st->grid_fit[q] = P.grid_fit[q];
   st->grid_np = P.grid_np;
   st->grid_ns = P.grid_ns;
   st->grid_herm = P.grid_herm;
@@ -2497,7 +2529,7 @@ static cudaError_t launch_grid(bq_state* s, const bq::GridArgs& a, int q, cudaSt
 static int ensure_grid_adjoint(bq_state* s) {
   if (s->grid_adj || s->gprobs.empty()) return BQ_OK;
   for (int q = s->use_m1 && s->glist[1].n_ctas == 0 ? 1 : 2; q < 3; ++q) {
-    if (q == 2 && s->glist[1].n_ctas == 0) break;
+    if (!s->grid_fit[q] || (q == 2 && s->glist[1].n_ctas == 0)) break;
     std::vector<bq::GridPiece> pieces;
     std::vector<bq::GridCta> ctas;
     GridList gl;

@@ -145,3 +145,23 @@ def test_svd_initial_conditions_plan_fewer_systems():
     svd = _plan(p, ic_mode="svd")
     assert svd["n_systems"] <= 16 < mono["n_systems"]
     assert svd["total_elems"] < mono["total_elems"]
+
+
+def test_pool_reserves_the_exchange_only_where_it_is_used():
+    """The grid-resident kernels' exchange ring is many times the state: it is not reserved for states
+    whose points do not fit the SMs' shared memory."""
+    def arrays_and_total(spec, **kw):
+        h = bq.problem_from_spec(spec)
+        arr = (C.c_void_p * 1)(h.ptr.value)
+        info = binding.bq_plan_info()
+        opts = bq.map_opts(dt=spec.dt, horizon=spec.T, **kw)
+        assert bq.lib().bq_plan(arr, 1, C.byref(opts), C.byref(info)) == 0
+        st, total = required(spec, dt=spec.dt, horizon=spec.T, **kw)
+        assert st == 0
+        return 5 * info.total_elems * (16 if kw.get("dtype", "f64") == "f64" else 8), total
+
+    # two modes, direct: 234 256 points in FP64 do not fit, 20 736 do
+    big, total = arrays_and_total(configs.two_mode(N=22, T=0.01, dt=0.001), method="direct")
+    assert total < 1.3 * big
+    small, total = arrays_and_total(configs.two_mode(N=12, T=0.01, dt=0.001), method="direct")
+    assert total > 2.0 * small

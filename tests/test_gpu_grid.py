@@ -298,10 +298,10 @@ def test_frequencies_that_cancel_cancel_exactly(dtype):
     assert np.array_equal(_raw(st, dtype), before)
 
 
-@pytest.mark.parametrize("N", [5, 6])
-def test_states_without_R_count_the_points_they_hold(N):
-    """Three modes with R = 0: 64 and 125 systems of G_x and G_y alone (54 000 points at N = 6, 5.8 million
-    if R were stored) take the grid kernel."""
-    p = configs.table_one_network(3, N, steps=4000)
+@pytest.mark.parametrize("modes,N", [(3, 5), (3, 6), (4, 4)])
+def test_states_without_R_count_the_points_they_hold(modes, N):
+    """R = 0: 64 to 125 systems of G_x and G_y alone (three modes at N = 6: 54 000 points, 5.8 million if R
+    were stored) take the grid kernel."""
+    p = configs.table_one_network(modes, N, steps=4000)
     a, b = _both(dataclasses.replace(p, T=12 * p.dt), "f64", 12, r_layout="off")
     _agree(a, b, "f64")

@@ -819,6 +819,7 @@ struct bq_state {
   GridList glist[3];
   int grid_np = 0, grid_ns = 0, grid_herm = 0, grid_fit[3] = {0, 0, 0};  // fit: the pool has room for the list
   int grid_few = 0;  // single-mode: bq_step and bq_solve take the grid-resident kernel
+  int ring_in_pool = 0;  // the pool holds the exchange ring (else bq_grad's workspace does)
   int grid_pieces = 0, grid_adj = 0;  // pieces in the pool so far; the adjoint's list has been built
   std::vector<bq::GridProb> gprobs;
   // steps of equal length taken by the resident kernels since tau was run_tau0: their times are
@@ -1313,6 +1314,11 @@ static const int kGridFewM = 20;  // of a single system: below, both are at thei
 // Steps between the block counts of the grid-resident kernels (a power of two, at most four): fewer
 // while the ring would not stay small beside L2.
 static int grid_block(size_t arr) { return arr <= ((size_t)1 << 19) ? 4 : arr <= ((size_t)1 << 20) ? 2 : 1; }
+
+// Bytes of the exchange ring of a state.
+static size_t grid_ring_bytes(size_t elems, size_t cs) {
+  return 16 * bq::grid_place(elems, cs) * (8 * grid_block(elems * cs) + 1);
+}
 
 // X or Y term t's weights over the flat index of its side; S terms: of side y's dimensions.
 static std::vector<double> flat_weights(const Compiled& C, const TermDesc& td, int wbase, bool y) {
@@ -2129,7 +2135,8 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
   L.off_gpieces = seg(P.grid_cap * sizeof(bq::GridPiece));
   L.off_gctas = seg(P.grid_ok ? 3 * kGridMaxCtas * sizeof(bq::GridCta) : 0);
   L.off_gbar = seg(P.grid_ok ? BQ_GRID_BAR_WORDS * sizeof(unsigned int) : 0);
-  L.off_gring = seg(P.grid_ok ? 16 * bq::grid_place((size_t)P.total_elems, cs) * (8 * grid_block((size_t)P.total_elems * cs) + 1) : 0);
+  // (single-mode states that step with other kernels exchange in bq_grad only: in its workspace)
+  L.off_gring = seg(P.grid_ok && (!P.use_m1 || P.grid_few) ? grid_ring_bytes((size_t)P.total_elems, cs) : 0);
   L.off_dc = seg(P.dc.size() * sizeof(double2));
   L.off_groups = seg(P.groups.size() * sizeof(EvalGroup));
   L.off_entries = seg(P.entries.size() * sizeof(EvalEntry));
@@ -2338,6 +2345,7 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
   st->grid_ns = P.grid_ns;
   st->grid_herm = P.grid_herm;
   st->grid_few = P.grid_few && glist[1].n_ctas > 0 && (!P.grid_herm || glist[0].n_ctas > 0);
+  st->ring_in_pool = P.grid_ok && (!P.use_m1 || P.grid_few);
   st->grid_pieces = grid_pieces;
   st->gprobs = P.gprobs;
   if (!P.use_m1 && glist[1].n_ctas > 0) st->res_on = 1;
@@ -3161,7 +3169,7 @@ static int run_eval(bq_state* s, int g0, int n, int small, double* out_host, cud
 // Gradients (discrete adjoint with checkpointing).
 // ---------------------------------------------------------------------------------------
 struct GradLayout {
-  size_t ckpt, rec, lam, lacc, ba, bb, srcred, grad, total;
+  size_t ckpt, rec, lam, lacc, ba, bb, srcred, grad, ring, total;
   size_t rec_seg;  // bytes of one segment's recorded stage inputs (4 k states)
   int64_t n_ckpt;
 };
@@ -3181,6 +3189,7 @@ static GradLayout grad_layout(const bq_state* s, int64_t n_steps, int k) {
   g.bb = seg(arr);
   g.srcred = seg((size_t)s->n_sys * std::max(1, s->srcred_stride) * cs);
   g.grad = seg((size_t)std::max(1, s->grad_size) * sizeof(double));
+  g.ring = seg(s->use_m1 && !s->ring_in_pool && s->grid_fit[2] ? grid_ring_bytes((size_t)s->total_elems, cs) : 0);
   // two segments' stage inputs (recompute overlaps the backward sweep), last: a larger
   // workspace holds further recordings (bq_grad records that many segments in its forward
   // pass and does not recompute them)
@@ -3291,6 +3300,7 @@ extern "C" int bq_grad(bq_state* s, double dt, int64_t n_steps, int checkpoint_e
   auto coop_fwd = [&](double tau_seg, int64_t n, char* rec, cudaStream_t cs) -> cudaError_t {
     if (grid) {
       bq::GridArgs a = grid_args(s, 1, dt);
+      if (!s->ring_in_pool) a.ring = w + G.ring;
       a.rec = rec;
       a.tau0 = tau_seg;
       a.n_steps = (int)n;
@@ -3366,6 +3376,7 @@ extern "C" int bq_grad(bq_state* s, double dt, int64_t n_steps, int checkpoint_e
       }
       if (grid) {
         bq::GridArgs a = grid_args(s, 2, dt);
+        if (!s->ring_in_pool) a.ring = w + G.ring;
         a.rec = rec;
         a.lam = lam;
         a.grad = (double*)(w + G.grad);

@@ -160,6 +160,9 @@ def test_pool_reserves_the_exchange_only_where_it_is_used():
         assert st == 0
         return 5 * info.total_elems * (16 if kw.get("dtype", "f64") == "f64" else 8), total
 
+    # a single-mode state that steps with the resident kernel exchanges in bq_grad's workspace only
+    big, total = arrays_and_total(configs.kerr_driven(N=40, dt=0.001, T=0.01), dtype="f32")
+    assert total < 1.5 * big + 65536  # (tables and lists; every segment is rounded up)
     # two modes, direct: 234 256 points in FP64 do not fit, 20 736 do
     big, total = arrays_and_total(configs.two_mode(N=22, T=0.01, dt=0.001), method="direct")
     assert total < 1.3 * big

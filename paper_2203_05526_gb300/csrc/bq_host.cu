@@ -206,10 +206,17 @@ static double binom(int n, int k) {
   for (int i = 1; i <= k; ++i) r = r * (n - k + i) / i;
   return r;
 }
+// n! (a table: the weights of a 4096-oscillator batch ask for half a million)
 static double fact(int n) {
-  double r = 1.0;
-  for (int i = 2; i <= n; ++i) r *= i;
-  return r;
+  struct Table {
+    double v[171];
+    Table() {
+      v[0] = 1.0;
+      for (int i = 1; i < 171; ++i) v[i] = v[i - 1] * i;
+    }
+  };
+  static const Table t;
+  return n < 1 ? 1.0 : n < 171 ? t.v[n] : HUGE_VAL;  // (171! is beyond the range of a double)
 }
 
 static Poly product(const Key& m1, const Key& m2, cplx c) {
@@ -1055,9 +1062,9 @@ static int res_shape(int M, int cs, bool herm, bool few, int& rb, int& nb) {
 
 // Row and column tables of a sandwich term are alike: they differ by a factor only (its rate, to
 // rounding).
-static bool same_table(const std::vector<double>& x, const std::vector<double>& y) {
+static bool same_table(const double* x, const double* y, int n) {
   double r = 0.0;
-  for (size_t k = 0; k < x.size(); ++k) {
+  for (int k = 0; k < n; ++k) {
     if ((x[k] == 0.0) != (y[k] == 0.0)) return false;
     if (x[k] == 0.0) continue;
     if (r == 0.0) r = x[k] / y[k];
@@ -1066,13 +1073,23 @@ static bool same_table(const std::vector<double>& x, const std::vector<double>& 
   return true;
 }
 
-static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, const EvalGroup& eg, int term_off,
-                        int wbase, size_t cs, std::vector<unsigned char>& blk, int& variant, bool& herm) {
+template <typename T>
+static unsigned char* put_real(unsigned char* to, const double* v, int n) {
+  T* p = reinterpret_cast<T*>(to);
+  for (int i = 0; i < n; ++i) p[i] = (T)v[i];
+  return to + n * sizeof(T);
+}
+
+// The block of problem C appended to P.rparams (tables on the stack, written in place: this runs for
+// every problem of a batch, twice per map).
+static bool res_problem(Plan& P, const Compiled& C, const EvalGroup& eg, int term_off, int wbase, size_t cs, int& variant,
+                        bool& herm) {
   const int M = C.M[0];
   if (M < 4 || M > 42 || !C.has_r || C.r_diag || eg.n_e > 32) return false;
-  std::vector<cplx> d(C.diag.begin(), C.diag.begin() + 2 * M);
-  std::vector<double> w[8];  // xm xp ym yp smx smy spx spy
-  for (auto& v : w) v.assign(M, 0.0);
+  cplx d[2 * 42];
+  std::copy(C.diag.begin(), C.diag.begin() + 2 * M, d);
+  double w[8][42];  // xm xp ym yp smx smy spx spy
+  for (auto& v : w) std::fill(v, v + M, 0.0);
   const TermDesc* off[4] = {nullptr, nullptr, nullptr, nullptr};  // xm xp ym yp
   int sdiag = -1;
   bool splus = false;
@@ -1088,9 +1105,9 @@ static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, co
       const int s = td.deltaGx, dg = td.diagp1 ? 1 : 0;
       if (td.ch >= 0 || c.imag() != 0.0 || s != td.deltaGy || (s != -1 && s != 1) || (sdiag >= 0 && sdiag != dg)) return false;
       sdiag = dg;
-      std::vector<double>&wx = w[s < 0 ? 4 : 6], &wy = w[s < 0 ? 5 : 7];
-      for (double v : wy)
-        if (v != 0.0) return false;  // a second term of this direction
+      double *wx = w[s < 0 ? 4 : 6], *wy = w[s < 0 ? 5 : 7];
+      for (int k = 0; k < M; ++k)
+        if (wy[k] != 0.0) return false;  // a second term of this direction
       const double *tx = table(0), *ty = table(1);
       for (int k = 0; k < M; ++k) {
         wx[k] = c.real() * (tx ? tx[k] : 1.0);
@@ -1154,30 +1171,27 @@ static bool res_problem(const Plan& P, const Compiled& C, const bq::M1Sys& m, co
     }
   }
   variant = (imag ? 0 : 1) | (splus ? 2 : 0) | (sdiag > 0 ? 4 : 0);
-  herm = w[0] == w[2] && w[1] == w[3];
+  herm = std::equal(w[0], w[0] + M, w[2]) && std::equal(w[1], w[1] + M, w[3]);
   for (int k = 0; k < M && herm; ++k) herm = d[M + k] == std::conj(d[k]);
-  herm = herm && same_table(w[4], w[5]) && same_table(w[6], w[7]);
-  blk.resize(sizeof(h) + (size_t)12 * M * (cs / 2));
-  unsigned char* to = blk.data() + sizeof(h);
-  auto put = [&](double v) {
-    const float f = (float)v;
-    std::memcpy(to, cs == 16 ? (const void*)&v : (const void*)&f, cs / 2);
-    to += cs / 2;
-  };
-  for (const cplx& v : d) { put(v.real()); put(v.imag()); }
-  for (auto& v : w)
-    for (double x : v) put(x);
-  while (blk.size() % 16) blk.push_back(0);
-  h.obs_off = (int)blk.size();
+  herm = herm && same_table(w[4], w[5], M) && same_table(w[6], w[7], M);
+  h.obs_off = (int)((sizeof(h) + (size_t)12 * M * (cs / 2) + 15) & ~(size_t)15);
   h.n_obs = eg.n_e;
+  const size_t at = P.rparams.size();
+  P.rparams.resize(at + h.obs_off + eg.n_e * sizeof(bq::PipeObs<double2>));
+  unsigned char* to = P.rparams.data() + at;
+  std::memcpy(to, &h, sizeof(h));
+  to += sizeof(h);
+  const auto put = cs == 16 ? put_real<double> : put_real<float>;
+  to = put(to, reinterpret_cast<const double*>(d), 4 * M);
+  for (auto& v : w) to = put(to, v, M);
+  to = P.rparams.data() + at + h.obs_off;
   for (int e = 0; e < eg.n_e; ++e) {
     const EvalEntry& en = P.entries[eg.e_off + e];
     bq::PipeObs<double2> o;
     std::memset(&o, 0, sizeof(o));
     o.kx = en.kx; o.ly = en.ly; o.f = make_double2(en.f_re, en.f_im);
-    blk.insert(blk.end(), (const unsigned char*)&o, (const unsigned char*)&o + sizeof(o));
+    std::memcpy(to + e * sizeof(o), &o, sizeof(o));
   }
-  std::memcpy(blk.data(), &h, sizeof(h));
   return true;
 }
 
@@ -1246,20 +1260,22 @@ static bool res_pack(Plan& P, const std::vector<int>& which, const std::vector<i
   return true;
 }
 
-// progs: the term program of every problem (single-mode states).
-static void make_res_plan(Plan& P, const bq_problem* const* probs, const std::vector<bq::M1Sys>& progs, size_t cs) {
+static void make_res_plan(Plan& P, const bq_problem* const* probs, size_t cs) {
   if (P.total_elems >= ((int64_t)1 << 31)) return;
   const int B = (int)P.comp.size();
   std::vector<int> term_off(B, 0), poff(B, 0);
   for (const SysDesc& sd : P.sys) term_off[sd.prob] = sd.term_off;
   std::vector<char> herm(B, 0);
-  std::vector<unsigned char> blk;
   int sd = -1;
+  size_t bytes = 0;
+  for (int b = 0; b < B; ++b)
+    bytes += sizeof(bq::ResHdr) + 12 * P.comp[b].M[0] * (cs / 2) + 16 + P.groups[b].n_e * sizeof(bq::PipeObs<double2>);
+  P.rparams.reserve(bytes);
   for (int b = 0; b < B; ++b) {
     bool hm = false;
     int variant = 0;
-    blk.clear();
-    if (!res_problem(P, P.comp[b], progs[b], P.groups[b], term_off[b], P.wbase[b], cs, blk, variant, hm)) return;
+    poff[b] = (int)P.rparams.size();
+    if (!res_problem(P, P.comp[b], P.groups[b], term_off[b], P.wbase[b], cs, variant, hm)) return;
     // one kernel per launch: the restriction to k = l holds for all sandwich terms of the batch or
     // for none (problems without sandwich terms go with either)
     bool has_s = false;
@@ -1276,8 +1292,6 @@ static void make_res_plan(Plan& P, const bq_problem* const* probs, const std::ve
       }
     }
     herm[b] = hm;
-    poff[b] = (int)P.rparams.size();
-    P.rparams.insert(P.rparams.end(), blk.begin(), blk.end());
   }
   std::vector<int> hs, gs;
   for (int i = 0; i < (int)P.sys.size(); ++i) {
@@ -1488,7 +1502,7 @@ static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wba
     herm = dh[1][k] == std::conj(dh[0][k]) && dl[1][k] == std::conj(dl[0][k]);
     for (int j = 0; j < G.np && herm; ++j) herm = pw[4 * j][k] == pw[4 * j + 2][k] && pw[4 * j + 1][k] == pw[4 * j + 3][k];
   }
-  for (int s = 0; s < G.ns && herm; ++s) herm = same_table(sw[2 * s], sw[2 * s + 1]);
+  for (int s = 0; s < G.ns && herm; ++s) herm = same_table(sw[2 * s].data(), sw[2 * s + 1].data(), ng);
   // tables
   auto putc = [&](const std::vector<cplx>& v) { for (const cplx& x : v) { tab.push_back(x.real()); tab.push_back(x.imag()); } };
   auto putr = [&](const std::vector<double>& v) { tab.insert(tab.end(), v.begin(), v.end()); };
@@ -2042,7 +2056,7 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
         P.use_pipe = pipe_ok && 2 * (size_t)P.pipe_slot <= 200 * 1024 ? 1 : 0;
 
       }
-      if (P.use_pipe) make_res_plan(P, probs, progs, cs);
+      if (P.use_pipe) make_res_plan(P, probs, cs);
       if (!P.res_ok) {
         P.rparams.clear();
         P.rgroups.clear();

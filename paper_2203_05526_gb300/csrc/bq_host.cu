@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <complex>
 #include <cstdarg>
@@ -1270,6 +1271,7 @@ static void make_res_plan(Plan& P, const bq_problem* const* probs, size_t cs) {
   size_t bytes = 0;
   for (int b = 0; b < B; ++b)
     bytes += sizeof(bq::ResHdr) + 12 * P.comp[b].M[0] * (cs / 2) + 16 + P.groups[b].n_e * sizeof(bq::PipeObs<double2>);
+  if (bytes > INT_MAX) return;  // (32-bit offsets of the blocks)
   P.rparams.reserve(bytes);
   for (int b = 0; b < B; ++b) {
     bool hm = false;
@@ -1988,6 +1990,7 @@ static int make_plan(const bq_problem* const* probs, int B, const bq_map_opts* o
           P.pparams.insert(P.pparams.end(), blk.begin(), blk.end());
           par_max = std::max(par_max, blk.size());
         }
+        pipe_ok = pipe_ok && P.pparams.size() <= INT_MAX;  // (32-bit offsets of the blocks)
         static_assert(sizeof(bq::PipeCoef<float2>) == 16 && sizeof(bq::PipeCoef<double2>) == 32,
                       "coefficient records as written above");
         static_assert(sizeof(bq::PipeObs<float2>) == 16 && sizeof(bq::PipeObs<double2>) == 32,

@@ -178,7 +178,7 @@ int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* opts, void*
 /* Advances every system of the state by n_steps RK4 steps of size dt (the mapped value
  * of dt must not exceed the bound checked at bq_map).  Single-mode states of the resident form
  * (bq_tune resident): all n_steps in one launch, every system on chip.  Tiled states of that
- * form that fit the SMs' shared memory, and FP64 states of up to 128 single-mode systems: all
+ * form that fit the SMs' shared memory, and FP64 states of up to 128 single-mode problems: all
  * n_steps in one cooperative launch that exchanges stage inputs through L2 (the waits are bounded:
  * one longer than a few seconds sets the error word, BQ_ETIMEOUT from the next synchronising call).  Else fused stage kernels: on the pipelined single-mode path the four stages of a step run in one launch
  * (bq_tune pipe_fused), otherwise one launch per stage; replayed from a CUDA graph.

@@ -1320,13 +1320,17 @@ static void make_res_plan(Plan& P, const bq_problem* const* probs, size_t cs) {
 // ---------------------------------------------------------------------------------------
 static const int kGridMaxCtas = BQ_GRID_MAX_CTAS;
 static const int64_t kGridMaxPoints = kGridMaxCtas * 2500;  // (more stored points never fit: not worth a plan)
-// Few single-mode systems in FP64 take the grid-resident kernel: the resident kernel keeps a system on
-// one SM, whose FP64 pipe then takes longer for a stage than the exchange between SMs does.  Measured
-// (us per step, resident / grid): one system N = 16 10.0 / 8.8, N = 20 10.8 / 9.0, N = 40 34.9 / 9.7;
-// 4 systems N = 12 20.9 / 8.9, N = 40 33.3 / 9.0; 64 systems N = 12 26.1 / 9.1, N = 40 34.9 / 12.7
-// (growing with the number from there; the resident kernel's 35 hold up to two systems per SM).
-static const int kGridFewSystems = 128;
-static const int kGridFewM = 20;  // of a single system: below, both are at their latencies
+// Single-mode FP64 states of few problems take the grid-resident kernel where its list fits: the resident
+// kernel keeps a system on one SM, whose FP64 pipe then takes longer for a stage than the exchange between
+// SMs does.  Measured (us per call of 64 steps, resident / grid): one system N = 12 652 / 481, N = 20 703 /
+// 507, N = 40 2266 / 516; problems of one system at N = 12: 4 1354 / 513, 16 1699 / 480, 128 1705 / 507;
+// one problem of 64 initial conditions 3629 / 511, 25 problems of four 3630 / 532, 100 of four 3636 / 2244.
+// A single small system is the exception: one step and its observable, which the resident kernel leaves
+// ready, take 44.7 / 46.2 us at N = 16, 45.6 / 46.0 at 20, 54.4 / 46.3 at 24 (from four steps a call on the
+// grid kernel is ahead at any N).  128 problems: each takes a CTA at least, of 152; at 150 the grid kernel
+// is still ahead (N = 12, 16 steps 466 / 164).
+static const int kGridFewProblems = 128;
+static const int kGridFewM = 20;  // of a single system
 // Steps between the block counts of the grid-resident kernels (a power of two, at most four): fewer
 // while the ring would not stay small beside L2.
 static int grid_block(size_t arr) { return arr <= ((size_t)1 << 19) ? 4 : arr <= ((size_t)1 << 20) ? 2 : 1; }
@@ -1634,7 +1638,8 @@ static void make_grid_plan(Plan& P, const bq_problem* const* probs, const bq_map
   P.grid_ok = 1;
   int m = 0;
   for (const bq::GridProb& g : P.gprobs) m = std::max(m, g.ng);
-  P.grid_few = P.res_ok && o.dtype == BQ_F64 && (!P.grid_herm || P.grid_fit[0]) && B <= kGridFewSystems && (B > 1 || m >= kGridFewM);
+  P.grid_few = P.res_ok && o.dtype == BQ_F64 && (!P.grid_herm || P.grid_fit[0]) && B <= kGridFewProblems &&
+               (P.sys.size() > 1 || m >= kGridFewM);
 }
 
 // The pieces of a list (0: forward, Hermitian layout where possible; 1: forward, general layout; 2:

@@ -305,3 +305,17 @@ def test_states_without_R_count_the_points_they_hold(modes, N):
     p = configs.table_one_network(modes, N, steps=4000)
     a, b = _both(dataclasses.replace(p, T=12 * p.dt), "f64", 12, r_layout="off")
     _agree(a, b, "f64")
+
+
+@pytest.mark.parametrize("instances,N,entries", [(1, 8, 4), (1, 8, 64), (25, 9, 4), (100, 8, 4), (40, 40, 4)])
+def test_few_problems_of_several_initial_conditions(instances, N, entries):
+    """One-mode FP64 problems whose measured operator has several entries (a system each), on both sides of
+    what the grid kernels hold (40 problems of four at N = 40 stay with the resident kernel)."""
+    meas = {((i % 8,), (i // 8,)): 1.0 / (1 + i) + 0.1j for i in range(entries)}
+    ps = [dataclasses.replace(configs.kerr_driven(N=N, dt=0.002, T=0.05, n_th=0.1), measured=meas) for _ in range(instances)]
+    a, b = gpu_state(ps, dtype="f64"), gpu_state(ps, dtype="f64")
+    b.set_tune(resident=0)
+    for n in (1, 13):
+        a.step(ps[0].dt, n)
+        b.step(ps[0].dt, n)
+    _agree(a, b, "f64")

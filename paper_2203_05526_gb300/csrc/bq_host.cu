@@ -3278,6 +3278,10 @@ extern "C" int bq_grad(bq_state* s, double dt, int64_t n_steps, int checkpoint_e
   const size_t arr = (size_t)s->total_elems * cs;
   const double tau0 = s->tau;
   const int res_known0 = s->res_known, res_dirty0 = s->res_dirty;
+  // (until the state is back as it was: a call that fails on the way leaves it elsewhere)
+  s->obs_valid = 0;
+  s->res_known = 0;
+  s->res_dirty = 1;
   const int k = checkpoint_every;
   CUDA_TRY(cudaMemsetAsync(w + G.grad, 0, (size_t)std::max(1, s->grad_size) * sizeof(double), st));
   // Cooperative segment kernels (tiled path): one launch per segment and direction, grids of

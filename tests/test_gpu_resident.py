@@ -248,3 +248,27 @@ def test_fp64_update_keeps_the_bits_of_elements_below_their_increment(instances,
         y, c = residual(st)
         assert np.min(np.abs(y.real)) > 2.0 ** -40
         assert np.all(c.real == -eps)
+
+
+def test_a_gradient_that_fails_leaves_no_stale_observables():
+    """Elements near the largest FP32 value overflow in a step and spread by at most four rows in each: the
+    gradient is refused, and the observables afterwards are not those of the step before it."""
+    import paper_2203_05526_gb300 as bq
+    import torch
+    p = _problem(14, steps=40)
+    p.rho0 = {((0,), (0,)): 1.0}
+    st = gpu_state(p, dtype="f32")
+    assert st.get_tune()["resident"] == 1
+    host = torch.zeros(st.state_bytes() // 8, dtype=torch.complex64)
+    info = st.system_info(0)
+    off = ((info["n_gx"] + 3) & ~3) + ((info["n_gy"] + 3) & ~3)
+    host[off] = 1.0
+    host[off + 12 * 14:off + 14 * 14] = 2.9e38 + 2.9e38j
+    host = host.pin_memory()
+    st.load_state(host.data_ptr())
+    st.step(1e-9, 1)
+    assert np.all(np.isfinite(st.evaluate()))
+    with pytest.raises(bq.BQError):
+        st.grad(p.dt, 16, 8)
+    with pytest.raises(bq.BQError):
+        st.evaluate()

@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
   __syncthreads();
   uint4* const ring = reinterpret_cast<uint4*>(A.ring);
   const size_t place = A.place;
-  const int places = (int)min((long long)A.ring_places, 4LL * A.n_steps + 1);  // that this launch uses  // of a place of the ring; its elements
+  const int places = (int)min((long long)A.ring_places, 4LL * A.n_steps + 1);  // that this launch uses
   auto recorded = [&](long long i, int stage) { return reinterpret_cast<C*>(A.rec + ((size_t)i * 4 + stage - 1) * A.arr); };
   const int Pc = ng | 1;
   auto position = [&](const GridPiece& g) {
@@ -706,11 +706,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_fwd(const GridArgs A) {
 
 // The adjoint of n_steps recorded steps, last first (see k_adj_stage in bq_kernels.cu for the
 // recursion): q = J^T b with the transposed weights at the same neighbours, b of the previous
-// stage exchanged through L2, one barrier per stage.  The transposed separable source needs, at a
-// point of G, sums over a row or column of b_R, which is complete once the stage's barrier has
-// passed: a warp per G point sums it directly, in the same phase as the points of R (no
-// reduction phase of its own).  Parameter sums stay in registers: per pair u P^T b and u Q^T b,
-// reduced into the gradient slots when an envelope changes its value and at the end.
+// stage exchanged through the numbered slots.  The transposed separable source needs, at a
+// point of G, sums over a row or column of b_R: a warp per G point waits for those elements and sums
+// them directly, beside the points of R (no reduction phase of its own).  Parameter sums stay in
+// registers: per pair u P^T b and u Q^T b, reduced into the gradient slots when an envelope changes
+// its value and at the end.
 // ONE (at most two pairs, two sandwich terms, eight pieces a CTA and ten row values a lane): a warp's one piece with its
 // offsets and state in registers and every value it needs in one batch of loads.
 template <typename T, int NP, int THREADS, bool ONE>
@@ -1076,15 +1076,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
           for (int s = 0; s < 4; ++s)
             if (any >> s & 1u) qv = caxpy(w[(4 * np + s) * n], sv[s], qv);
         } else {
-          // points of G, BQ_GRID_GLEN per piece, the whole warp on each: the transposed source's
-          // sum over a row (G_x) or column (G_y) of b_R, then the point's own lane the rest
+          // a point of G, the whole warp on it: the transposed source's sum over a row (G_x) or column
+          // (G_y) of b_R, then the point's own lane the rest
           const bool isx = kind == GRID_X;
-          C mine = zero;
-          for (int gi = 0; gi < len && P.has_r && ns; ++gi) {
-            const int k = g.start + gi;
-            C src = zero;
+          C src = zero;
+          if (P.has_r) {
             for (int s = 0; s < ns; ++s) {
-              const int kk = k - P.ss[s];  // row / column of b_R
+              const int kk = g.start - P.ss[s];  // row / column of b_R
               if (kk < 0 || kk >= ng) continue;
               const T wt = swt[(2 * s + (isx ? 0 : 1)) * ng + kk];
               if (wt == (T)0) continue;
@@ -1123,9 +1121,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_grid_adj(const GridArgs A) {
               src.x += __shfl_xor_sync(0xffffffffu, src.x, o);
               src.y += __shfl_xor_sync(0xffffffffu, src.y, o);
             }
-            if (lane == gi) mine = src;
           }
-          qv = cadd(qv, mine);
+          if (ok) qv = cadd(qv, src);
 #pragma unroll 1
           for (int j0 = 0; j0 < np; j0 += 2) {
             const int m = min(2, np - j0);

@@ -13,7 +13,6 @@
 #define BQ_GRID_SMEM_MAX (200 * 1024)
 #define BQ_GRID_ROWS 10   // row values a lane of an adjoint piece of G may need (GRID_ONE)
 #define BQ_GRID_BAR_WORDS 5
-#define BQ_GRID_GLEN 1   // G points of an adjoint piece
 
 namespace bq {
 
@@ -41,8 +40,8 @@ struct GridProb {
 
 enum GridKind : int { GRID_R = 0, GRID_H = 1, GRID_D = 2, GRID_X = 3, GRID_Y = 4 };
 
-// Up to 32 points of one kind of one system, one per lane (the adjoint: G points in pieces of
-// BQ_GRID_GLEN, a warp per point).  start: first point in the kind's own numbering.
+// Up to 32 points of one kind of one system, one per lane (the adjoint: a point of G is a piece, a warp
+// sums its row or column).  start: first point in the kind's own numbering.
 struct GridPiece {
   int sys, kind, start, len;
   int off_gx, off_gy, off_r, pad;

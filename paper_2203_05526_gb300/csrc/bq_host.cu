@@ -821,7 +821,7 @@ struct bq_state {
   // systems of list 0 are known to hold Hermitian states (false once a state was loaded or
   // another kernel stepped it: then res_dirty asks for a check of the data before the next
   // launch, and the systems that fail it take list 2)
-  int res_ok = 0, res_on = 0, res_variant = 0, res_obs = 0, res_known = 1, res_dirty = 0;
+  int res_ok = 0, res_on = 0, res_variant = 0, res_known = 1, res_dirty = 0;
   ResList rlist[3];
   // grid-resident kernels: lists (forward Hermitian, forward general, adjoint) and variant sizes
   GridList glist[3];
@@ -912,7 +912,7 @@ struct Plan {
   double rho = 0.0, dt_max = 0.0;
   // resident kernel (k_resident): parameter blocks per problem, groups (the Hermitian layout's,
   // then the general layout's) and the CTAs' bins
-  int res_ok = 0, res_variant = 0, res_obs = 1;
+  int res_ok = 0, res_variant = 0;
   std::vector<unsigned char> rparams;
   std::vector<bq::ResGroup> rgroups;
   std::vector<bq::ResBin> rbins;
@@ -1137,9 +1137,6 @@ static bool res_problem(Plan& P, const Compiled& C, const EvalGroup& eg, int ter
   w[1][M - 1] = w[3][M - 1] = w[6][M - 1] = w[7][M - 1] = 0.0;
   bq::ResHdr h;
   std::memset(&h, 0, sizeof(h));
-  h.M = M;
-  h.has_sep = C.has_sep;
-  h.sdiag = sdiag > 0;
   int n_off = 0;
   for (auto* o : off) n_off += o != nullptr;
   bool imag = true;
@@ -1212,7 +1209,7 @@ static bool res_pack(Plan& P, const std::vector<int>& which, const std::vector<i
       bq::ResGroup g;
       std::memset(&g, 0, sizeof(g));
       const int cols = herm ? M | 1 : M;
-      const int w = res_shape(M, (int)cs, herm, which.size() <= 152, g.rb, g.nb);
+      const int w = res_shape(M, (int)cs, herm, which.size() <= BQ_GRID_MAX_CTAS, g.rb, g.nb);
       if (!w) return false;
       g.sys = which[i];
       g.M = M;
@@ -1544,7 +1541,7 @@ static bool grid_problem(const Plan& P, const Compiled& C, int term_off, int wba
 template <typename F>
 static void grid_kinds(const SysDesc& sd, const bq::GridProb& G, int list, F f) {
   const bool hm = list == 0 && G.herm;
-  const int cols = sd.n_g | 1, len = list == 2 ? BQ_GRID_GLEN : 32;
+  const int cols = sd.n_g | 1, len = list == 2 ? 1 : 32;
   if (sd.has_r) {
     if (hm) f(bq::GRID_H, (cols / 2 + 1) * cols, 32);
     else f(sd.r_diag ? bq::GRID_D : bq::GRID_R, sd.n_r, 32);
@@ -2360,7 +2357,6 @@ extern "C" int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* 
   st->pipe_ok = st->use_pipe;
   st->res_ok = st->res_on = P.res_ok && st->pipe_ok;
   st->res_variant = P.res_variant;
-  st->res_obs = P.res_obs;
   for (int q = 0; q < 3; ++q) st->rlist[q] = P.rlist[q];
   for (int q = 0; q < 3; ++q) st->glist[q] = glist[q], st->grid_fit[q] = P.grid_fit[q];
   st->grid_np = P.grid_np;
@@ -2633,7 +2629,7 @@ static cudaError_t enqueue_resident(bq_state* s, double dt, int64_t n, cudaStrea
   a.chpar = (const double*)(b + L.off_chpar);
   a.y = b + L.off_y;
   a.comp = b + L.off_comp;
-  a.obs = s->res_obs ? (double2*)(b + L.off_obs) : nullptr;
+  a.obs = (double2*)(b + L.off_obs);
   a.reverse = s->reverse;
   a.dt = dt;
   a.horizon = s->horizon;
@@ -2666,7 +2662,7 @@ static cudaError_t enqueue_resident(bq_state* s, double dt, int64_t n, cudaStrea
     done += m;
   }
   run_end(s, dt, n);
-  s->obs_valid = s->res_obs;
+  s->obs_valid = 1;
   return cudaSuccess;
 }
 

@@ -532,29 +532,27 @@ __device__ __forceinline__ void res_gwarp(const ResArgs& A, const ResGroup& g, u
   V.stage_out(V.yg, g.blk_elems);
   place(gc);
   V.stage_out(V.cg, g.blk_elems);
-  if (A.obs) {
-    // Tr(rho0 A)'s contribution: w sum_e f_e (G_x[k] G_y[l] + R[k, l]) of y - comp
-    const PipeObs<double2>* ob = reinterpret_cast<const PipeObs<double2>*>(V.blk + h.obs_off);
-    double2 v = make_double2(0.0, 0.0);
-    auto val = [&](int i) {
-      const C p = V.yg[i], q = V.cg[i];
-      return make_double2((double)(p.x - q.x), (double)(p.y - q.y));
-    };
-    if (lane < h.n_obs) {
-      const PipeObs<double2> o = ob[lane];
-      v = val(g.r_off + o.kx * M + o.ly);
-      if (V.sep) v = cadd(v, cmul(val(o.kx), val(g.gy_off + o.ly)));
-      v = cmul(cmul(make_double2(g.w_re, g.w_im), o.f), v);
-    }
-    if (h.n_obs > 1) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-      }
-    }
-    if (lane == 0) A.obs[g.sys] = v;
+  // Tr(rho0 A)'s contribution: w sum_e f_e (G_x[k] G_y[l] + R[k, l]) of y - comp
+  const PipeObs<double2>* ob = reinterpret_cast<const PipeObs<double2>*>(V.blk + h.obs_off);
+  double2 v = make_double2(0.0, 0.0);
+  auto val = [&](int i) {
+    const C p = V.yg[i], q = V.cg[i];
+    return make_double2((double)(p.x - q.x), (double)(p.y - q.y));
+  };
+  if (lane < h.n_obs) {
+    const PipeObs<double2> o = ob[lane];
+    v = val(g.r_off + o.kx * M + o.ly);
+    if (V.sep) v = cadd(v, cmul(val(o.kx), val(g.gy_off + o.ly)));
+    v = cmul(cmul(make_double2(g.w_re, g.w_im), o.f), v);
   }
+  if (h.n_obs > 1) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+      v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+    }
+  }
+  if (lane == 0) A.obs[g.sys] = v;
 }
 
 template <typename T, int MODE, int NS, bool SD, bool HERM>

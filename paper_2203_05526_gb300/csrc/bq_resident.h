@@ -47,11 +47,9 @@ struct ResBin {
 //   right-hand (Y) terms; smx smy / spx spy: row and column weights of the sandwich terms with
 //   sources (k - 1, l - 1) / (k + 1, l + 1), their rate folded into the row weight.
 struct ResHdr {
-  int M, has_sep, sdiag, n_obs;
+  int n_obs, obs_off;  // the observable's entries: count and byte offset
   int ch;             // 1: the off-diagonal terms follow the envelope below
   int conj;           // of the X term with source k - 1
-  int obs_off;        // byte offset of the observable's entries
-  int pad;
   double a_re, a_im;  // coefficient of the X term with source k - 1 (static part)
   PipeChan chan;
 };
@@ -64,7 +62,7 @@ struct ResArgs {
   const unsigned char* flags;  // per system: state is Hermitian (null: not consulted)
   void* y;
   void* comp;
-  double2* obs;                // per system w sum_e f_e G(k_e, l_e) of the final state (or null)
+  double2* obs;                // per system w sum_e f_e G(k_e, l_e) of the final state
   int want;                    // with flags: 1 = systems whose flag is set, 0 = the others
   int comp_zero;               // comp is known to be zero and not read
   int reverse;

@@ -97,6 +97,10 @@ N_RANGE = (10, 40)  # Fock truncation range of the instances (--n-range)
 # FMA counts two): diagonal (2 + 6), four neighbour terms (4 x 8), one sandwich term with its
 # separable source (18), the RK4 combine (13 on average over the four stages).
 FLOP_PER_POINT_STAGE = 70
+# The resident kernel on this workload (Hermitian systems: half of R and G_x are held, the drive's
+# coefficient is imaginary), per held point of R and stage: diagonal 6, neighbours 18, sandwich and source
+# 12, combine 11.5 (FP32) or 9 (FP64) on average; per point of G_x diagonal 6, neighbours 10, combine.
+RESIDENT_FLOP = {"f32": (47.5, 27.5), "f64": (45.0, 25.0)}
 
 # DRAM traffic of the fused step kernel per launch (one RK4 step), from one ncu capture of
 # dram__bytes_read.sum + dram__bytes_write.sum on the default workload (65 536 instances,
@@ -162,6 +166,15 @@ def points_of(specs):
         n = p.N[0]
         tot += n * n + 2 * n
     return tot
+
+
+def flops_per_step(specs, resident: bool, dtype: str) -> float:
+    """Floating-point operations of one RK4 step that the stepping kernel executes on the specs."""
+    if not resident:
+        return 4.0 * FLOP_PER_POINT_STAGE * points_of(specs)
+    r, g = RESIDENT_FLOP[dtype]
+    odd = [p.N[0] | 1 for p in specs]
+    return 4.0 * sum(r * q * (q // 2 + 1) + g * p.N[0] for p, q in zip(specs, odd))
 
 
 def host_cores() -> int:
@@ -352,8 +365,9 @@ def alu_peaks():
 
 def fp64_leg(n_inst: int, peaks: dict, steps: int = 5, warmup: int = 3):
     """The headline workload in complex FP64: stage-kernel time per RK4 step, updates/s, and
-    the two roofs that could bind it (HBM on 64 B per grid-point stage; the measured FP64 FMA
-    rate on FLOP_PER_POINT_STAGE); GB300's FP64 pipe makes the latter bind."""
+    the two roofs that could bind it (HBM: on the resident kernel the state and its residual in and
+    out once per call, else 64 B per grid-point stage; the measured FP64 FMA rate on the kernel's
+    own operations); GB300's FP64 pipe makes the latter bind."""
     import torch
 
     import paper_2203_05526_gb300 as bq
@@ -372,8 +386,9 @@ def fp64_leg(n_inst: int, peaks: dict, steps: int = 5, warmup: int = 3):
     torch.cuda.synchronize()
     s_per_step = e0.elapsed_time(e1) / 1e3 / steps
     ups = 4 * pts / s_per_step
-    hbm = 64 * ups / 1e9
-    flops = FLOP_PER_POINT_STAGE * ups
+    resident = st.get_tune()["stage_path"] == "pipe" and st.get_tune()["resident"] == 1
+    hbm = (4 * 16 * pts / steps / s_per_step if resident else 64 * ups) / 1e9
+    flops = flops_per_step(specs, resident, "f64") / s_per_step
     f64_peak = 2 * peaks.get("fp64_fma_per_s", float("nan"))
     hbm_peak = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("hbm_gbs", 6800.0) \
         if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else 6800.0
@@ -382,7 +397,8 @@ def fp64_leg(n_inst: int, peaks: dict, steps: int = 5, warmup: int = 3):
                           "frac": flops / f64_peak}}
     bound = max(roofs, key=lambda k: roofs[k]["frac"])
     return {"workload": f"kerr_batch x{n_inst}, complex FP64, {steps} RK4 steps", "ms_per_step": 1e3 * s_per_step,
-            "updates_per_s": ups, "stage_path": st.get_tune()["stage_path"], "roofs": roofs, "bound": bound}
+            "updates_per_s": ups, "stage_path": st.get_tune()["stage_path"], "resident": int(resident), "roofs": roofs,
+            "bound": bound}
 
 
 def batched_leg(world: int):
@@ -419,12 +435,14 @@ def batched_leg(world: int):
     if out["schedule"]["solve_kernel"] == "step":  # bq_solve would step: time the persistent kernel
         st.set_tune(solve_kernel="merged" if st.solve_eligible() else "program")
     out["persistent_kernel"] = st.get_tune()["solve_kernel"]
+    resident = st.get_tune()["resident"] == 1 and out["persistent_kernel"] == "merged" and st.get_tune()["solve_ctas_per_sm"] == 0
     n0 = bq.launch_count()
     t_solve = timed(lambda: st.solve(DT, n_steps))
     launches = bq.launch_count() - n0
     ev = st.evaluate()
     out["persistent"] = {"seconds": t_solve, "solves_per_s": 4096 / t_solve,
-                         "updates_per_s": 4 * pts * n_steps / t_solve, "launches": launches,
+                         "updates_per_s": 4 * pts * n_steps / t_solve, "launches": launches, "resident": int(resident),
+                         "flops_per_s": flops_per_step(specs, resident, "f32") * n_steps / t_solve,
                          "finite": bool(np.all(np.isfinite(ev)))}
     st2 = bq.State(handles, opts)
     st2.step(DT, 128)
@@ -704,10 +722,11 @@ def fig2_leg(modes=(1, 2, 3), target: float = 1e-4, steps: int = 2000, n_max: in
 
 def secular_leg(B: int = 32768, steps: int = 20):
     """The paper's secular dissipator (Eq. 203 / Eq. S9, zero temperature) on kerr_batch's
-    instances (secular_batch: same draws, complex FP32): grid-point RK-stage updates/s of the
-    stage kernel (the projector term is restricted to diagonal index pairs) and its HBM
-    bandwidth on the algorithmic bytes of the headline roofline (16 array transfers per point
-    and step), with the kernel's own transfer count beside it."""
+    instances (secular_batch: same draws, complex FP32): grid-point RK-stage updates/s (the
+    projector term is restricted to diagonal index pairs) and the HBM bandwidth on the bytes
+    the kernel cannot do without: the state and its residual in and out once per call on the
+    resident kernel, 16 array transfers per point and step on the streaming ones, with the
+    kernel's own transfer count beside it."""
     import torch
 
     import paper_2203_05526_gb300 as bq
@@ -930,9 +949,8 @@ def main():
         batched = batched_leg(world)
         f32_peak = 2 * peaks_alu["fp32_fma_per_s"]
         p = batched["persistent"]
-        p["alu_roofline"] = {"bound": "alu", "achieved": FLOP_PER_POINT_STAGE * p["updates_per_s"] / 1e12,
-                             "peak": f32_peak / 1e12, "unit": "TFLOP/s",
-                             "frac": FLOP_PER_POINT_STAGE * p["updates_per_s"] / f32_peak,
+        p["alu_roofline"] = {"bound": "alu", "achieved": p["flops_per_s"] / 1e12,
+                             "peak": f32_peak / 1e12, "unit": "TFLOP/s", "frac": p["flops_per_s"] / f32_peak,
                              "peak_source": "measured (bq_fma_peak, FP32)"}
     grads = None
     if not args.no_grads and world == 1:

@@ -142,7 +142,10 @@ int bq_problem_set_rho0(bq_problem* p, int n, const int* k, const int* l, const 
 
 /* ---- mapping (Eqs. 6, 10-13, 304) ---------------------------------------------------- */
 
-/* Device bytes bq_map() needs for B problems mapped with the same options. */
+/* Device bytes bq_map() needs for B problems mapped with the same options.  Beside the tables and five
+ * arrays of the state's size, a state that bq_step spreads over the SMs (see bq_tune resident) holds the
+ * ring through which they exchange stage inputs: 33, 17 or 9 slots of 32 bytes (FP64) or 16 (FP32) per
+ * element for arrays of up to 512 KiB, up to 1 MiB, or more. */
 int bq_required_bytes(const bq_problem* const* probs, int B, const bq_map_opts* opts, size_t* out);
 
 /* Host-only view of the plan bq_map() would build (no device needed; no counterpart in the
@@ -180,8 +183,9 @@ int bq_map(const bq_problem* const* probs, int B, const bq_map_opts* opts, void*
  * (bq_tune resident): all n_steps in one launch, every system on chip.  Tiled states of that
  * form that fit the SMs' shared memory, and FP64 states of up to 128 single-mode problems: all
  * n_steps in one cooperative launch that exchanges stage inputs through L2 (the waits are bounded:
- * one longer than a few seconds sets the error word, BQ_ETIMEOUT from the next synchronising call).  Else fused stage kernels: on the pipelined single-mode path the four stages of a step run in one launch
- * (bq_tune pipe_fused), otherwise one launch per stage; replayed from a CUDA graph.
+ * one longer than a few seconds sets the error word, BQ_ETIMEOUT from the next synchronising call).
+ * Else fused stage kernels: on the pipelined single-mode path the four stages of a step run in one
+ * launch (bq_tune pipe_fused), otherwise one launch per stage; replayed from a CUDA graph.
  * Asynchronous on stream. */
 int bq_step(bq_state* s, double dt, int64_t n_steps, void* stream);
 
@@ -209,8 +213,10 @@ int bq_solve_eligible(const bq_state* s, int* eligible);
  * The paper leaves the parallel schedule open (independent initial conditions processed
  * "in an ideal fashion", main text after Eq. 13).  A state carries a schedule for bq_step
  * and one for bq_solve; bq_map picks defaults from occupancy, bq_autotune measures the
- * candidates on the state itself and keeps the fastest.  Changing a schedule never changes
- * the arithmetic: every candidate computes the same RK4 step in the same order per point. */
+ * candidates on the state itself and keeps the fastest.  The schedules of the streaming, tiled
+ * and persistent kernels compute the same RK4 step in the same order per point.  The resident
+ * kernels compute it to rounding: static couplings are part of their weights, and Hermitian
+ * systems are held as half of their points (after bq_load_state in the layout the data need). */
 #define BQ_PATH_TILED 0    /* generic kernel, tiles of R with halo windows (any mode count) */
 #define BQ_PATH_SYSTEM 1   /* single mode, one CTA per system */
 #define BQ_PATH_PIPE 2     /* single mode, persistent CTAs with bulk-copy prefetch */
@@ -250,7 +256,8 @@ typedef struct bq_tune {
                           * group of warps; few FP64 systems over all SMs; also BQ_SOLVE_MERGED
                           * with solve_ctas_per_sm = 0) and BQ_PATH_TILED (the state spread over the SMs, one cooperative launch;
                           * also bq_grad's segments with grad_coop).  0 = the kernels that the
-                          * other fields describe */
+                          * other fields describe (bq_get_tune reports those fields either way;
+                          * a zeroed struct has it at 0) */
 } bq_tune;
 
 /* Current schedules of the state (step_us / solve_us: last bq_autotune result, else 0). */
@@ -286,7 +293,8 @@ int bq_grad_size(const bq_state* s, int* n);
 
 /* Device bytes of the gradient workspace for n_steps steps checkpointed every
  * checkpoint_every steps: ceil(n/k) checkpoints of the state and 2 x 4 k recorded stage
- * inputs (two segments), plus four cotangent arrays. */
+ * inputs (two segments), plus four cotangent arrays and, for single-mode states that bq_step does not
+ * spread over the SMs, the exchange ring (see bq_required_bytes). */
 int bq_grad_required_bytes(const bq_state* s, int64_t n_steps, int checkpoint_every, size_t* out);
 
 /* Bytes of one segment's recorded stage inputs (4 checkpoint_every states) and the number of
@@ -337,9 +345,9 @@ int bq_autotune_grad(bq_state* s, double dt, int trial_steps, int checkpoint_eve
  * complex FP64 or 524 288 complex FP32 elements; larger states get BQ_EUNSUPPORTED and should
  * use bq_step).  Every GPU that loads the library holds that array until the process
  * exits.  The state's own scratch regions in its pool are not touched; its state arrays are
- * updated exactly as bq_step updates them (same kernels, same arithmetic).  Plain kernel
- * launches on stream (4 per step) after clearing the used part of the three buffers; no
- * allocation, no cudaFree, no allocating library routine.
+ * updated exactly as bq_step with bq_tune resident = 0 updates them (same kernels, same
+ * arithmetic).  Plain kernel launches on stream (4 per step) after clearing the used part of the
+ * three buffers; no allocation, no cudaFree, no allocating library routine.
  *   - The first call on a device looks up the array's device address (cudaGetSymbolAddress,
  *     once per device, with that device current); make that first call before any stream
  *     capture is begun on the calling thread.

@@ -15,7 +15,7 @@
 // bq_resident.cuh for the layout) hold half the points.
 // Measured (one GB300, FP64, per RK4 step; one launch per stage / a grid barrier per stage / slots):
 // two modes at N = 12 45 / 20 / 9.8 us, three modes at N = 6 direct 183 / 68 / 28, mapped with R(xy)
-// (125 systems) 279 / 66 / 37; the 131-parameter control gradient 201 / 76 / 46; one oscillator at N =
+// (125 systems) 279 / 66 / 37, with R = 0 88 / - / 20; the 131-parameter control gradient 201 / 76 / 46; one oscillator at N =
 // 40, which the resident kernel keeps on one SM in 36 us, 9.  What bounds a stage now: small states
 // the chain store, L2, poll, arithmetic of one warp (about 2 us); large ones the FP64 pipe (one warp
 // instruction per 16 cycles and SM: 65% busy).

@@ -255,7 +255,8 @@ typedef struct bq_tune {
                           * whatever the other schedule fields say: BQ_PATH_PIPE (one system per
                           * group of warps; few FP64 systems over all SMs; also BQ_SOLVE_MERGED
                           * with solve_ctas_per_sm = 0) and BQ_PATH_TILED (the state spread over the SMs, one cooperative launch;
-                          * also bq_grad's segments with grad_coop).  0 = the kernels that the
+                          * also bq_grad's segments with grad_coop; of single-mode states
+                          * outside the resident form with grad_coop alone).  0 = the kernels that the
                           * other fields describe (bq_get_tune reports those fields either way;
                           * a zeroed struct has it at 0) */
 } bq_tune;

@@ -1316,7 +1316,9 @@ static void make_res_plan(Plan& P, const bq_problem* const* probs, size_t cs) {
 // shared memory holds.
 // ---------------------------------------------------------------------------------------
 static const int kGridMaxCtas = BQ_GRID_MAX_CTAS;
-static const int64_t kGridMaxPoints = kGridMaxCtas * 2500;  // (more stored points never fit: not worth a plan)
+// (An FP64 point takes at least 84 bytes of a CTA's 200 KB: more stored points never fit, nor do FP32 ones
+// with a pair and two sandwich terms.  Not worth a plan.)
+static const int64_t kGridMaxPoints = kGridMaxCtas * 2500;
 // Single-mode FP64 states of few problems take the grid-resident kernel where its list fits: the resident
 // kernel keeps a system on one SM, whose FP64 pipe then takes longer for a stage than the exchange between
 // SMs does.  Measured (us per call of 64 steps, resident / grid): one system N = 12 652 / 481, N = 20 703 /
